@@ -272,17 +272,12 @@ template <typename T, int V> __device__ __forceinline__ void ldv(const C<T> *p, 
         const float4 u = __ldg(reinterpret_cast<const float4 *>(p));
         v[0] = make_float2(u.x, u.y);
         v[1] = make_float2(u.z, u.w);
-    } else if constexpr (is_df<T>) {
-        const float4 u = __ldg(reinterpret_cast<const float4 *>(p));
-        v[0] = cdf{df(u.x, u.y), df(u.z, u.w)};
     } else {
         v[0] = __ldg(p);
     }
 }
 template <typename T, int V> __device__ __forceinline__ void stv(C<T> *p, const C<T> (&v)[V]) {
-    if constexpr (is_df<T>) {
-        *p = cdf{df_norm(v[0].x), df_norm(v[0].y)};
-    } else if constexpr (V == 2) {
+    if constexpr (V == 2) {
         *reinterpret_cast<float4 *>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
     } else {
         *p = v[0];
@@ -316,17 +311,8 @@ __device__ __forceinline__ void gather_rows(const Rec<T> *__restrict__ rec, int6
                 for (int v = 0; v < V; ++v)
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
-                        if constexpr (is_df<T>) {
-                            df_acc(acc[a][j][v].x, b[3 * a], x0[v].x);
-                            df_acc(acc[a][j][v].x, b[3 * a + 1], x1[v].x);
-                            df_acc(acc[a][j][v].x, b[3 * a + 2], x2[v].x);
-                            df_acc(acc[a][j][v].y, b[3 * a], x0[v].y);
-                            df_acc(acc[a][j][v].y, b[3 * a + 1], x1[v].y);
-                            df_acc(acc[a][j][v].y, b[3 * a + 2], x2[v].y);
-                        } else {
-                            acc[a][j][v].x += b[3 * a] * x0[v].x + b[3 * a + 1] * x1[v].x + b[3 * a + 2] * x2[v].x;
-                            acc[a][j][v].y += b[3 * a] * x0[v].y + b[3 * a + 1] * x1[v].y + b[3 * a + 2] * x2[v].y;
-                        }
+                        acc[a][j][v].x += b[3 * a] * x0[v].x + b[3 * a + 1] * x1[v].x + b[3 * a + 2] * x2[v].x;
+                        acc[a][j][v].y += b[3 * a] * x0[v].y + b[3 * a + 1] * x1[v].y + b[3 * a + 2] * x2[v].y;
                     }
             }
         }
@@ -383,6 +369,166 @@ __global__ void __launch_bounds__(256) k_project(const int64_t *__restrict__ ptr
         const int32_t r = rbase + row % SLAB;
         const int64_t nn = n0 + nd;
         if (r < R && nn < Ng) grid[(int64_t(d) * R + r) * Ng + nn] = sm[nd * ROWS + row];
+    }
+}
+
+// ---- FP64 and double-float gathers by real columns.  A block is real, so the
+// complex dense operand [rows][3][R] is a real one of C = 2R columns and re and
+// im never mix: a lane owns a column (or J of them, 32 apart) instead of a
+// complex right-hand side.  Both forms are bound by their arithmetic pipe (FP64:
+// 16 cycles per warp instruction and SM; double-float: 12 FP32 operations per
+// term), so what counts is full lanes and few operations: terms are chained
+// FMAs (three per record, column and component; a product sum added to the
+// accumulator takes four).
+// A row's sum is the sum, in order, of the partial sums of SEG equal runs of its
+// records.  With few columns a warp takes several runs at once, one per group of
+// C lanes, and several rows; the order of the sum, and so the result, does not
+// depend on how many right-hand sides are in the call.
+template <typename T> __device__ __forceinline__ T ld_col(const T *p) {
+    if constexpr (is_df<T>) {
+        const float2 u = __ldg(reinterpret_cast<const float2 *>(p));
+        return df(u.x, u.y);
+    } else {
+        return __ldg(p);
+    }
+}
+__device__ __forceinline__ void col_acc(double &acc, double b, double x) { acc = ::fma(b, x, acc); }
+__device__ __forceinline__ void col_acc(df &acc, df b, df x) { df_acc(acc, b, x); }
+__device__ __forceinline__ double col_sum(double a, double b) { return a + b; }
+// unnormalised: exact two-sum of the high parts, its error and the low parts in the low part
+__device__ __forceinline__ df col_sum(df a, df b) { return df_qadd(a, b); }
+__device__ __forceinline__ double col_val(double a) { return a; }
+__device__ __forceinline__ df col_val(df a) { return df_norm(a); }
+
+// Lane of a row's team: G groups of C lanes, 32 / (G C) rows per warp (one
+// group and J column sets when C > 16).
+template <int J, int G> struct ColLane {
+    int row, rpw, g;   // row of the warp's rpw rows, group
+    int32_t c[J];      // columns (lanes beyond the last column repeat a valid one)
+    bool col[J], on;   // column exists; lane belongs to a row
+    __device__ __forceinline__ ColLane(int32_t C, int32_t slab0, int lane) {
+        if constexpr (G == 1) {
+            row = g = 0;
+            rpw = 1;
+            on = true;
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                col[j] = slab0 + lane + 32 * j < C;
+                c[j] = col[j] ? slab0 + lane + 32 * j : slab0 + (lane & 1);
+            }
+        } else {
+            static_assert(J == 1, "one column per lane in a group");
+            rpw = 32 / (G * C);
+            row = lane / (G * C);
+            g = (lane - row * G * C) / C;
+            c[0] = lane - (row * G + g) * C;
+            on = row < rpw;
+            col[0] = on;
+        }
+    }
+};
+
+// v[a][j] = sum over row [e0, e1) of sum_b rec.b[3a+b] X[col][b][c[j]], in the
+// order described above, in the lanes of group 0.  Every lane of the warp calls.
+template <typename T, int J, int G, int SEG>
+__device__ __forceinline__ void gather_cols(const Rec<T> *__restrict__ rec, int64_t e0, int64_t e1,
+                                            const T *__restrict__ X, int32_t C, const ColLane<J, G> &l, int lane,
+                                            T (&v)[3][J]) {
+    constexpr int PER = SEG / G;      // runs per group
+    static_assert(PER * G == SEG, "runs divide among the groups");
+    const int64_t ld = 3 * int64_t(C);
+    const int64_t len = e1 - e0;
+    T part[G == 1 ? 1 : PER][3][J];   // G > 1: kept apart until the groups are joined
+#pragma unroll(G == 1 ? 1 : PER)
+    for (int q = 0; q < PER; ++q) {
+        T acc[3][J];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int j = 0; j < J; ++j) acc[a][j] = T(0.0);
+        const int s = l.g * PER + q;
+        const int64_t b0 = e0 + len * s / SEG, b1 = e0 + len * (s + 1) / SEG;
+#pragma unroll 2
+        for (int64_t e = b0; e < b1; ++e) {
+            T b[9];
+            const int64_t col = load_rec<T>(rec + e, b);
+            const T *x = X + col * ld;
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const T x0 = ld_col(x + l.c[j]), x1 = ld_col(x + C + l.c[j]), x2 = ld_col(x + 2 * C + l.c[j]);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    col_acc(acc[a][j], b[3 * a], x0);
+                    col_acc(acc[a][j], b[3 * a + 1], x1);
+                    col_acc(acc[a][j], b[3 * a + 2], x2);
+                }
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                if constexpr (G == 1) v[a][j] = q == 0 ? acc[a][j] : col_sum(v[a][j], acc[a][j]);
+                else part[q][a][j] = acc[a][j];
+            }
+    }
+    if constexpr (G > 1) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            v[a][0] = part[0][a][0];
+#pragma unroll
+            for (int q = 1; q < PER; ++q) v[a][0] = col_sum(v[a][0], part[q][a][0]);
+        }
+#pragma unroll 1
+        for (int g = 1; g < G; ++g)
+#pragma unroll
+            for (int q = 0; q < PER; ++q)
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    v[a][0] = col_sum(v[a][0], shfl1(part[q][a][0], (lane + g * C) & 31));
+    }
+}
+
+// Grid currents as k_project, by real columns: a warp takes its rpw nodes, a
+// block kProjNodes of them (8 warps' worth), grid (node blocks, slabs of 32 J
+// columns).  FP64, bond wires: 48 right-hand sides 3.82 ms (6.29 with a complex
+// right-hand side per lane), 20k triangles and 8: 0.235 (1.19) ms.
+constexpr int kProjSeg = 4, kTriSeg = 8;   // runs per row (a node has about 20 records, a triangle 300)
+template <typename T, int J> __host__ __device__ constexpr int proj_cols_pitch() { return 3 * 32 * J + 2; }   // 2 x odd: distinct banks
+template <typename T, int J, int G>
+__global__ void __launch_bounds__(256) k_project_cols(const int64_t *__restrict__ ptr, const Rec<T> *__restrict__ rec,
+                                                      const T *__restrict__ cT, int64_t Ng, int32_t R,
+                                                      C<T> *__restrict__ grid) {
+    constexpr int SLAB = 32 * J, ROWS = proj_cols_pitch<T, J>();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *sm = reinterpret_cast<T *>(smem_raw);   // [8 rpw nodes][pitch]
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int32_t Cn = 2 * R, slab0 = int32_t(blockIdx.y) * SLAB;
+    const ColLane<J, G> l(Cn, slab0, lane);
+    const int nodes = kProjNodes * l.rpw;
+    // several nodes per warp: their columns fit one pitch of the single-node form
+    const int pitch = G == 1 ? ROWS : 3 * Cn + 2;
+    const int64_t n0 = int64_t(blockIdx.x) * nodes, n = n0 + w * l.rpw + l.row;
+    T v[3][J];
+    const bool act = l.on && n < Ng;
+    gather_cols<T, J, G, kProjSeg>(rec, act ? ptr[n] : 0, act ? ptr[n + 1] : 0, cT, Cn, l, lane, v);
+    const int dstep = G == 1 ? SLAB : Cn;
+    if (l.on && l.g == 0) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int j = 0; j < J; ++j)
+                if (l.col[j]) sm[(w * l.rpw + l.row) * pitch + a * dstep + (l.c[j] - slab0)] = col_val(v[a][j]);
+    }
+    __syncthreads();
+    const int nr = min(SLAB, Cn - slab0) / 2;   // right-hand sides of the slab
+    for (int i = threadIdx.x; i < 3 * nr * nodes; i += blockDim.x) {
+        const int row = i / nodes, nd = i - row * nodes;
+        const int d = row / nr, rl = row - d * nr;
+        const int64_t nn = n0 + nd;
+        if (nn < Ng)
+            grid[(int64_t(d) * R + slab0 / 2 + rl) * Ng + nn] =
+                *reinterpret_cast<const C<T> *>(sm + nd * pitch + d * dstep + 2 * rl);
     }
 }
 
@@ -494,36 +640,7 @@ __device__ __forceinline__ void tri_epilogue(const C<T> (&acc)[3][J][V], int64_t
                                              const float2 *__restrict__ coef_dd, int ncond, int64_t nt,
                                              TourE<T> *__restrict__ y_tri) {
     const int cd = cond[t];
-    if constexpr (is_df<T>) {
-        // double-float product: Gram term and Eq. Zb in double-float like the field
-        DD G[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) G[i] = dd_from(__ldg(gram + 9 * t + i));
-#pragma unroll
-        for (int j = 0; j < J; ++j)
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                const int32_t r = rl + 32 * V * j + v;
-                if (r >= R) continue;
-                const float2 *cf = coef_dd + int64_t(r) * (2 * ncond + 1);
-                const float2 zr = cf[2 * cd], zi = cf[2 * cd + 1], cl = cf[2 * ncond];
-                cdf c[3];
-#pragma unroll
-                for (int l = 0; l < 3; ++l) c[l] = cT[(t * 3 + l) * R + r];
-                float4 *out = y_tri + (int64_t(r) * nt + t) * 3;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    DD gr = dd_mul(G[3 * k], to_dd(c[0].x)), gi = dd_mul(G[3 * k], to_dd(c[0].y));
-#pragma unroll
-                    for (int l = 1; l < 3; ++l) {
-                        gr = dd_add(gr, dd_mul(G[3 * k + l], to_dd(c[l].x)));
-                        gi = dd_add(gi, dd_mul(G[3 * k + l], to_dd(c[l].y)));
-                    }
-                    out[k] = dd_zb_df(zr, zi, cl, gr, gi, to_dd(df_norm(acc[k][j][v].x)),
-                                         to_dd(df_norm(acc[k][j][v].y)));
-                }
-            }
-    } else if constexpr (is_f32<T>) {
+    if constexpr (is_f32<T>) {
         // mixed form: Gram term in FP32 like the field, Eq. Zb in double-float
         float G[9];
 #pragma unroll
@@ -608,6 +725,88 @@ __global__ void __launch_bounds__(256)
         gather_rows<T, V, J, false>(pt_rec, pt_ptr[t], pt_ptr[t + 1], phiT, R, rl, acc);
     }
     tri_epilogue<T, V, J>(acc, t, rl, R, cT, gram, cond, coef, coef_dd, ncond, nt, y_tri);
+}
+
+// k_tri_gather by real columns (FP64 and double-float): a warp takes its rpw
+// triangles and a slab of 32 J columns.  Column c = 2 r + p holds the real
+// (p = 0) or imaginary (p = 1) part of right-hand side r, so the two halves of a
+// complex product sit in neighbouring lanes: each lane forms its own half of
+// Eq. Zb from its Gram term and its neighbour's.
+// FP64 on the bond wires (40k triangles, 14.1M records), 48 right-hand sides:
+// 20.3 ms, 96 % of the FP64 pipe, against 38.6 ms with a complex right-hand side
+// per lane (48 of 64 lanes, four operations per term); 20k triangles, 8
+// right-hand sides: 1.71 against 9.06 ms; 1.5k triangles, one: 44 against 843 us.
+// Double-float on the 40k triangles, 16: 2.37 against 3.65 ms.
+template <typename T, int J, int G>
+__global__ void __launch_bounds__(256)
+    k_tri_cols(const int64_t *__restrict__ near_ptr, const Rec<T> *__restrict__ near_rec,
+               const int64_t *__restrict__ pt_ptr, const Rec<T> *__restrict__ pt_rec, const T *__restrict__ cT,
+               const T *__restrict__ phiT, const double *__restrict__ gram, const int32_t *__restrict__ cond,
+               const double *__restrict__ coef, const float2 *__restrict__ coef_dd, int ncond, int64_t nt, int32_t R,
+               int32_t nslab, TourE<T> *__restrict__ y_tri) {
+    const int64_t gw = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const int32_t Cn = 2 * R, slab0 = int32_t(gw % nslab) * 32 * J;
+    const ColLane<J, G> l(Cn, slab0, lane);
+    const int64_t t0 = gw / nslab * l.rpw;
+    if (t0 >= nt) return;
+    const bool act = l.on && t0 + l.row < nt;
+    const int64_t t = act ? t0 + l.row : t0;
+    T acc[3][J], far[3][J];
+    gather_cols<T, J, G, kTriSeg>(near_rec, near_ptr[t], near_ptr[t + 1], cT, Cn, l, lane, acc);
+    gather_cols<T, J, G, kTriSeg>(pt_rec, pt_ptr[t], pt_ptr[t + 1], phiT, Cn, l, lane, far);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int j = 0; j < J; ++j) acc[a][j] = col_sum(acc[a][j], far[a][j]);
+    const int cd = cond[t];
+    const int im = lane & 1;   // C is even and slabs start at multiples of 32: lane and column parity agree
+    T gm[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const double v = __ldg(gram + 9 * t + i);
+        if constexpr (is_df<T>) {
+            const DD d = dd_from(v);
+            gm[i] = df(d.hi, d.lo);
+        } else {
+            gm[i] = v;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const T *x = cT + t * 3 * Cn + l.c[j];
+        const T x0 = ld_col(x), x1 = ld_col(x + Cn), x2 = ld_col(x + 2 * Cn);
+        const int32_t r = l.c[j] >> 1;
+        const bool out_on = act && l.g == 0 && l.col[j];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const T f = col_val(acc[k][j]);
+            if constexpr (is_df<T>) {
+                DD g = dd_mul(to_dd(gm[3 * k]), to_dd(x0));
+                g = dd_add(g, dd_mul(to_dd(gm[3 * k + 1]), to_dd(x1)));
+                g = dd_add(g, dd_mul(to_dd(gm[3 * k + 2]), to_dd(x2)));
+                const df go = shfl1(df(g.hi, g.lo), lane ^ 1), fo = shfl1(f, lane ^ 1);
+                if (out_on) {
+                    const float2 *cf = coef_dd + int64_t(r) * (2 * ncond + 1);
+                    const float2 zr = cf[2 * cd], zi = cf[2 * cd + 1], cl = cf[2 * ncond];
+                    // re = zr gr - zi gi - cl fi,  im = zr gi + zi gr + cl fr
+                    const DD o = dd_add(dd_mul(DD{zi.x, zi.y}, to_dd(go)), dd_mul(DD{cl.x, cl.y}, to_dd(fo)));
+                    const DD y = dd_add(dd_mul(DD{zr.x, zr.y}, g), im ? o : dd_neg(o));
+                    reinterpret_cast<float2 *>(y_tri + (int64_t(r) * nt + t) * 3 + k)[im] = make_float2(y.hi, y.lo);
+                }
+            } else {
+                const double g = ::fma(gm[3 * k + 2], x2, ::fma(gm[3 * k + 1], x1, gm[3 * k] * x0));
+                const double go = shfl1(g, lane ^ 1), fo = shfl1(f, lane ^ 1);
+                if (out_on) {
+                    const double *cf = coef + int64_t(r) * (2 * ncond + 1);
+                    const double zr = cf[2 * cd], zi = cf[2 * cd + 1], cl = cf[2 * ncond];
+                    const double o = ::fma(cl, fo, zi * go);
+                    reinterpret_cast<double *>(y_tri + (int64_t(r) * nt + t) * 3 + k)[im] =
+                        ::fma(zr, g, im ? o : -o);
+                }
+            }
+        }
+    }
 }
 
 // The lossy kernel (pfft_params.kernel = SIE_KERNEL_LOSSY): as k_tri_gather with
@@ -828,28 +1027,72 @@ int scratch_reserve(pfft_plan *p, int32_t nrhs, int prec) {
     return SIE_OK;
 }
 
-// Block-sparse stages for one slab shape: V complex per load, J loads per lane.
+// block records by precision: projection (rows = nodes), interpolation (rows = triangles), near field
+template <typename T> const Rec<T> *rec_pn(const pfft_plan *p) {
+    if constexpr (is_df<T>) return p->d_pn_recdf;
+    else if constexpr (is_f64<T>) return p->d_pn_rec64;
+    else return p->d_pn_rec32;
+}
+template <typename T> const Rec<T> *rec_pt(const pfft_plan *p) {
+    if constexpr (is_df<T>) return p->d_pt_recdf;
+    else if constexpr (is_f64<T>) return p->d_pt_rec64;
+    else return p->d_pt_rec32;
+}
+template <typename T> const Rec<T> *rec_near(const pfft_plan *p) {
+    if constexpr (is_df<T>) return p->d_near_recdf;
+    else if constexpr (is_f64<T>) return p->d_near_rec64;
+    else return p->d_near_rec32;
+}
+
+// Block-sparse stages by real columns (FP64, double-float): J column sets per
+// lane, G groups of lanes per row.
+template <typename T, int J, int G> struct Cols {
+    static int project(pfft_plan *p, int32_t R, cudaStream_t st) {
+        constexpr int GP = G < kProjSeg ? G : kProjSeg;
+        const int nodes = kProjNodes * (GP == 1 ? 1 : 32 / (GP * 2 * R));
+        const dim3 grid(unsigned((p->Ng + nodes - 1) / nodes), unsigned((2 * R + 32 * J - 1) / (32 * J)));
+        const size_t smem = size_t(nodes) * (GP == 1 ? proj_cols_pitch<T, J>() : 6 * R + 2) * sizeof(T);
+        k_project_cols<T, J, GP><<<grid, 32 * kProjNodes, smem, st>>>(p->d_pn_ptr, rec_pn<T>(p),
+                                                                      (const T *)p->scr.cT, p->Ng, R,
+                                                                      (C<T> *)p->scr.grid);
+        SIE_LAUNCH_CHECK(p);
+        return SIE_OK;
+    }
+    static int tri_gather(pfft_plan *p, int32_t R, cudaStream_t st) {
+        const int32_t nslab = (2 * R + 32 * J - 1) / (32 * J);
+        const int rpw = G == 1 ? 1 : 32 / (G * 2 * R);
+        const int64_t warps = (p->nt + rpw - 1) / rpw * nslab;
+        k_tri_cols<T, J, G><<<unsigned((warps * 32 + 255) / 256), 256, 0, st>>>(
+            p->d_near_ptr, rec_near<T>(p), p->d_pt_ptr, rec_pt<T>(p), (const T *)p->scr.cT, (const T *)p->scr.phiT,
+            p->d_gram, p->d_cond, p->scr.coef, coef_dd(p), p->ncond, p->nt, R, nslab, (TourE<T> *)p->scr.y_tri);
+        SIE_LAUNCH_CHECK(p);
+        return SIE_OK;
+    }
+};
+// C = 2R columns: up to 16 of them the most groups that fit a warp (R <= 2: 8,
+// R <= 4: 4, R <= 8: 2); above, the J of the fewest equal slabs of at most 128.
+#define SIE_COLS_DISPATCH(T, R, CALL)                                         \
+    do {                                                                     \
+        if ((R) <= 2) return Cols<T, 1, 8>::CALL;                            \
+        if ((R) <= 4) return Cols<T, 1, 4>::CALL;                            \
+        if ((R) <= 8) return Cols<T, 1, 2>::CALL;                            \
+        const int32_t sets = (2 * (R) + 31) / 32, slabs = (sets + 3) / 4;    \
+        switch ((sets + slabs - 1) / slabs) {                                \
+            case 1: return Cols<T, 1, 1>::CALL;                              \
+            case 2: return Cols<T, 2, 1>::CALL;                              \
+            case 3: return Cols<T, 3, 1>::CALL;                              \
+            default: return Cols<T, 4, 1>::CALL;                             \
+        }                                                                    \
+    } while (0)
+
+// Block-sparse stages for one slab shape: V complex per load, J loads per lane
+// (mixed form; FP64 for the lossy kernel's gather).
 template <typename T, int V, int J> struct Blocks {
     static constexpr int SLAB = 32 * V * J;
-    static const Rec<T> *pn(const pfft_plan *p) {
-        if constexpr (is_df<T>) return p->d_pn_recdf;
-        else if constexpr (is_f64<T>) return p->d_pn_rec64;
-        else return p->d_pn_rec32;
-    }
-    static const Rec<T> *pt(const pfft_plan *p) {
-        if constexpr (is_df<T>) return p->d_pt_recdf;
-        else if constexpr (is_f64<T>) return p->d_pt_rec64;
-        else return p->d_pt_rec32;
-    }
-    static const Rec<T> *nr(const pfft_plan *p) {
-        if constexpr (is_df<T>) return p->d_near_recdf;
-        else if constexpr (is_f64<T>) return p->d_near_rec64;
-        else return p->d_near_rec32;
-    }
     static int project(pfft_plan *p, int32_t R, cudaStream_t st) {
         const dim3 grid(unsigned((p->Ng + kProjNodes - 1) / kProjNodes), unsigned((R + SLAB - 1) / SLAB));
         k_project<T, V, J><<<grid, 32 * kProjNodes, proj_smem<T, V, J>(), st>>>(
-            p->d_pn_ptr, pn(p), (const C<T> *)p->scr.cT, p->Ng, R, (C<T> *)p->scr.grid);
+            p->d_pn_ptr, rec_pn<T>(p), (const C<T> *)p->scr.cT, p->Ng, R, (C<T> *)p->scr.grid);
         SIE_LAUNCH_CHECK(p);
         return SIE_OK;
     }
@@ -857,7 +1100,7 @@ template <typename T, int V, int J> struct Blocks {
         const int32_t nslab = (R + SLAB - 1) / SLAB;
         const int64_t warps = p->nt * nslab;
         k_far_gather<T, V, J><<<unsigned((warps * 32 + 255) / 256), 256, 0, st>>>(
-            p->d_pt_ptr, pt(p), (const C<T> *)p->scr.phiT, p->nt, R, nslab, (C<T> *)p->scr.ffar);
+            p->d_pt_ptr, rec_pt<T>(p), (const C<T> *)p->scr.phiT, p->nt, R, nslab, (C<T> *)p->scr.ffar);
         SIE_LAUNCH_CHECK(p);
         return SIE_OK;
     }
@@ -868,7 +1111,7 @@ template <typename T, int V, int J> struct Blocks {
         const int prec = is_f64<T> ? SIE_PREC_FP64 : SIE_PREC_MIXED;
         k_tri_gather_lossy<T, J><<<unsigned((warps * 32 + 255) / 256), 256, 0, st>>>(
             p->d_near_ptr, p->d_near_col, reinterpret_cast<const C<T> *const *>(lossy_ltab(p, prec)),
-            lossy_rslot(p), p->d_pt_ptr, pt(p), (const C<T> *)p->scr.cT, (const C<T> *)p->scr.phiT, p->d_gram,
+            lossy_rslot(p), p->d_pt_ptr, rec_pt<T>(p), (const C<T> *)p->scr.cT, (const C<T> *)p->scr.phiT, p->d_gram,
             p->d_cond, p->scr.coef, coef_dd(p), p->ncond, p->nt, R, nslab, (TourE<T> *)p->scr.y_tri);
         SIE_LAUNCH_CHECK(p);
         return SIE_OK;
@@ -877,7 +1120,7 @@ template <typename T, int V, int J> struct Blocks {
         const int32_t nslab = (R + SLAB - 1) / SLAB;
         const int64_t warps = p->nt * nslab;
         k_tri_gather<T, V, J><<<unsigned((warps * 32 + 255) / 256), 256, 0, st>>>(
-            p->d_near_ptr, nr(p), p->d_pt_ptr, pt(p), (const C<T> *)p->scr.cT, (const C<T> *)p->scr.phiT,
+            p->d_near_ptr, rec_near<T>(p), p->d_pt_ptr, rec_pt<T>(p), (const C<T> *)p->scr.cT, (const C<T> *)p->scr.phiT,
             p->d_gram, p->d_cond, p->scr.coef, coef_dd(p), p->ncond, p->nt, R, nslab, (TourE<T> *)p->scr.y_tri);
         SIE_LAUNCH_CHECK(p);
         return SIE_OK;
@@ -888,19 +1131,11 @@ template <typename T, int V, int J> struct Blocks {
 // and 32 V J right-hand sides, V complex per load (FP32: two per 16-byte load
 // when R is even, so that rows of [.][3][R] start on 16-byte boundaries), J
 // loads per lane; the smallest slab that covers R keeps every lane busy.
-#define SIE_SLAB_DISPATCH(T, R, CALL)                                                     \
+#define SIE_SLAB_DISPATCH(R, CALL)                                                        \
     do {                                                                                 \
-        if constexpr (is_df<T>) {                                                         \
-            if ((R) <= 32) return Blocks<df, 1, 1>::CALL;                                 \
-            return Blocks<df, 1, 2>::CALL;                                                \
-        } else if constexpr (is_f64<T>) {                                                 \
-            if ((R) <= 32) return Blocks<double, 1, 1>::CALL;                             \
-            return Blocks<double, 1, 2>::CALL;                                            \
-        } else {                                                                          \
-            if ((R) <= 32) return Blocks<float, 1, 1>::CALL;                              \
-            if ((R) <= 64) return (R) % 2 == 0 ? Blocks<float, 2, 1>::CALL : Blocks<float, 1, 2>::CALL; \
-            return (R) % 2 == 0 ? Blocks<float, 2, 2>::CALL : Blocks<float, 1, 4>::CALL;  \
-        }                                                                                 \
+        if ((R) <= 32) return Blocks<float, 1, 1>::CALL;                                  \
+        if ((R) <= 64) return (R) % 2 == 0 ? Blocks<float, 2, 1>::CALL : Blocks<float, 1, 2>::CALL; \
+        return (R) % 2 == 0 ? Blocks<float, 2, 2>::CALL : Blocks<float, 1, 4>::CALL;      \
     } while (0)
 // The far-field gather keeps slabs at most 64 wide in FP32: its 128-wide form
 // needs 80 registers a thread, which caps residency at 3 CTAs per SM for this
@@ -908,12 +1143,10 @@ template <typename T, int V, int J> struct Blocks {
 // twice but keep 4 CTAs resident (measured: 0.77 -> 0.66 ms on the bond-wire
 // step; the projection, whose block records dominate its loads, is faster 128
 // wide).
-#define SIE_SLAB_DISPATCH_NARROW(T, R, CALL)                                              \
+#define SIE_SLAB_DISPATCH_NARROW(R, CALL)                                                 \
     do {                                                                                 \
-        if constexpr (is_f32<T>) {                                                        \
-            if ((R) > 32) return (R) % 2 == 0 ? Blocks<float, 2, 1>::CALL : Blocks<float, 1, 2>::CALL; \
-        }                                                                                 \
-        SIE_SLAB_DISPATCH(T, R, CALL);                                                    \
+        if ((R) > 32) return (R) % 2 == 0 ? Blocks<float, 2, 1>::CALL : Blocks<float, 1, 2>::CALL; \
+        SIE_SLAB_DISPATCH(R, CALL);                                                       \
     } while (0)
 template <typename T> int run_project(pfft_plan *p, int32_t R, cudaStream_t st) {
     if constexpr (is_f32<T>) {
@@ -931,16 +1164,19 @@ template <typename T> int run_project(pfft_plan *p, int32_t R, cudaStream_t st) 
             SIE_LAUNCH_CHECK(p);
             return SIE_OK;
         }
+        if (p->kt.proj_slab == 64) SIE_SLAB_DISPATCH_NARROW(R, project(p, R, st));
+        SIE_SLAB_DISPATCH(R, project(p, R, st));
+    } else {
+        SIE_COLS_DISPATCH(T, R, project(p, R, st));
     }
-    if (p->kt.proj_slab == 64) SIE_SLAB_DISPATCH_NARROW(T, R, project(p, R, st));
-    SIE_SLAB_DISPATCH(T, R, project(p, R, st));
 }
 int run_far_gather(pfft_plan *p, int32_t R, cudaStream_t st) {
-    if (p->kt.far_slab == 128) SIE_SLAB_DISPATCH(float, R, far_gather(p, R, st));
-    SIE_SLAB_DISPATCH_NARROW(float, R, far_gather(p, R, st));
+    if (p->kt.far_slab == 128) SIE_SLAB_DISPATCH(R, far_gather(p, R, st));
+    SIE_SLAB_DISPATCH_NARROW(R, far_gather(p, R, st));
 }
 template <typename T> int run_tri_gather(pfft_plan *p, int32_t R, cudaStream_t st) {
-    SIE_SLAB_DISPATCH(T, R, tri_gather(p, R, st));
+    if constexpr (is_f32<T>) SIE_SLAB_DISPATCH(R, tri_gather(p, R, st));
+    else SIE_COLS_DISPATCH(T, R, tri_gather(p, R, st));
 }
 template <typename T> int run_tri_gather_lossy(pfft_plan *p, int32_t R, cudaStream_t st) {
     if (R <= 32) return Blocks<T, 1, 1>::tri_gather_lossy(p, R, st);
