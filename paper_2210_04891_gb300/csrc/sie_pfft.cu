@@ -218,8 +218,9 @@ __device__ __forceinline__ C<T> branch_current(int32_t b, int64_t r, const doubl
 }
 
 // Local currents c_T[k] = s_k alpha_{b(T,k)}: one thread per (T, r) for the
-// three local edges, written as cT [T][3][R] (right-hand sides innermost).
-template <typename T>
+// three local edges, written as cT [T][3][R] (right-hand sides innermost), or
+// with SMALL (FP32) as float4 [T][2R] (components innermost, re and im columns).
+template <typename T, bool SMALL>
 __global__ void k_alpha_tri(const double2 *__restrict__ x, int64_t nl, const TourE<T> *__restrict__ P, int64_t nslots,
                             const int32_t *__restrict__ tb, const int8_t *__restrict__ ts,
                             const int32_t *__restrict__ loop_of_branch, const int32_t *__restrict__ twig_node,
@@ -229,6 +230,7 @@ __global__ void k_alpha_tri(const double2 *__restrict__ x, int64_t nl, const Tou
     int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= nt * nrhs) return;
     const int64_t t = i / nrhs, r = i % nrhs;
+    C<T> c[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const int64_t tk = t * 3 + k;
@@ -241,7 +243,14 @@ __global__ void k_alpha_tri(const double2 *__restrict__ x, int64_t nl, const Tou
                 a = to_c(x[r * nb + b], C<T>{});
             if (ts[tk] < 0) { a.x = -a.x; a.y = -a.y; }
         }
-        cT[tk * nrhs + r] = a;
+        if constexpr (SMALL) c[k] = a;
+        else cT[tk * nrhs + r] = a;
+    }
+    if constexpr (SMALL) {
+        static_assert(is_f32<T>, "component-inner currents in FP32 only");
+        float4 *o = reinterpret_cast<float4 *>(cT) + (t * nrhs + r) * 2;
+        o[0] = make_float4(c[0].x, c[1].x, c[2].x, 0.f);
+        o[1] = make_float4(c[0].y, c[1].y, c[2].y, 0.f);
     }
 }
 
@@ -494,7 +503,8 @@ __device__ __forceinline__ void gather_cols(const Rec<T> *__restrict__ rec, int6
 // columns).  FP64, bond wires: 48 right-hand sides 3.82 ms (6.29 with a complex
 // right-hand side per lane), 20k triangles and 8: 0.235 (1.19) ms.
 constexpr int kProjSeg = 4, kTriSeg = 8;   // runs per row (a node has about 20 records, a triangle 300)
-template <typename T, int J> __host__ __device__ constexpr int proj_cols_pitch() { return 3 * 32 * J + 2; }   // 2 x odd: distinct banks
+// shared pitch of a node, 2 x odd: the 8-node reads of the store hit distinct banks
+template <typename T, int J> __host__ __device__ constexpr int proj_cols_pitch() { return 3 * 32 * J + 2; }
 template <typename T, int J, int G>
 __global__ void __launch_bounds__(256) k_project_cols(const int64_t *__restrict__ ptr, const Rec<T> *__restrict__ rec,
                                                       const T *__restrict__ cT, int64_t Ng, int32_t R,
@@ -530,6 +540,174 @@ __global__ void __launch_bounds__(256) k_project_cols(const int64_t *__restrict_
             grid[(int64_t(d) * R + slab0 / 2 + rl) * Ng + nn] =
                 *reinterpret_cast<const C<T> *>(sm + nd * pitch + d * dstep + 2 * rl);
     }
+}
+
+// ---- FP32 gathers of few right-hand sides (C = 2R <= 32 columns): a lane owns
+// a real column of a row, up to 5 right-hand sides one output component of it
+// (COMP), and a warp takes several rows, where the wider form gives a warp one
+// row and leaves 32 - R lanes idle.  Each lane sums its row's records in order
+// with the wider form's expression, so the result is the same bit for bit at
+// every number of right-hand sides.
+// With little arithmetic per record these kernels are bound by their loads: by
+// latency on a small mesh (a row is a chain of record, then the operand it
+// names: U records are in flight and the next U are fetched a chunk ahead,
+// which leaves one round trip per chunk), by L1 wavefronts on a larger one (a
+// warp's load takes one per row and 128 bytes, however few lanes it serves).
+// Hence the layouts: a lane's coefficients and column are one 16-byte load, its
+// operand (the three components of a column, float4 [row][C]) another.
+constexpr int kSmallWarps = 2;   // warps per block: a small mesh still reaches every SM
+
+template <int U>   // COMP: output component a of column c
+__device__ __forceinline__ void gather_row(const Rec<float> *__restrict__ rec, int64_t e0, int64_t e1,
+                                           const float4 *__restrict__ X, int32_t C, int32_t c, int a,
+                                           float (&acc)[1]) {
+    const int n = int(e1 - e0);
+    if (n <= 0) return;
+    const float4 *v = reinterpret_cast<const float4 *>(rec + e0) + a;
+    X += c;
+    float4 bn[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) bn[u] = __ldg(v + 3 * int64_t(min(u, n - 1)));
+    for (int i = 0; i < n; i += U) {
+        float4 b[U], x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            b[u] = bn[u];
+            x[u] = __ldg(X + int64_t(__float_as_int(b[u].w)) * C);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) bn[u] = __ldg(v + 3 * int64_t(min(i + U + u, n - 1)));
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u < n) acc[0] += b[u].x * x[u].x + b[u].y * x[u].y + b[u].z * x[u].z;
+    }
+}
+template <int U>   // all three components of column c
+__device__ __forceinline__ void gather_row(const Rec<float> *__restrict__ rec, int64_t e0, int64_t e1,
+                                           const float4 *__restrict__ X, int32_t C, int32_t c, int,
+                                           float (&acc)[3]) {
+    const int n = int(e1 - e0);
+    if (n <= 0) return;
+    const float4 *v = reinterpret_cast<const float4 *>(rec + e0);
+    X += c;
+    float4 bn[U];   // the next chunk's first rows: coefficients and column
+#pragma unroll
+    for (int u = 0; u < U; ++u) bn[u] = __ldg(v + 3 * int64_t(min(u, n - 1)));
+    for (int i = 0; i < n; i += U) {
+        float4 b0[U], b1[U], b2[U], x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            b0[u] = bn[u];
+            x[u] = __ldg(X + int64_t(__float_as_int(b0[u].w)) * C);
+            const float4 *r = v + 3 * int64_t(min(i + u, n - 1));
+            b1[u] = __ldg(r + 1);
+            b2[u] = __ldg(r + 2);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) bn[u] = __ldg(v + 3 * int64_t(min(i + U + u, n - 1)));
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u < n) {
+                acc[0] += b0[u].x * x[u].x + b0[u].y * x[u].y + b0[u].z * x[u].z;
+                acc[1] += b1[u].x * x[u].x + b1[u].y * x[u].y + b1[u].z * x[u].z;
+                acc[2] += b2[u].x * x[u].x + b2[u].y * x[u].y + b2[u].z * x[u].z;
+            }
+    }
+}
+// lane of a warp of rpw rows: row, output component (0 without COMP) and column
+template <bool COMP> struct SmallLane {
+    int row, a;
+    int32_t c;
+    __device__ __forceinline__ SmallLane(int32_t C, int lane) {
+        const int per = COMP ? 3 * C : C;
+        row = lane / per;
+        a = (lane - row * per) / C;
+        c = lane - row * per - a * C;
+    }
+};
+
+// Grid currents (k_project) of few right-hand sides: rpw nodes per warp.
+template <bool COMP>
+__global__ void __launch_bounds__(32 * kSmallWarps)
+    k_project_small(const int64_t *__restrict__ ptr, const Rec<float> *__restrict__ rec, const float4 *__restrict__ cT,
+                    int64_t Ng, int32_t R, int rpw, float2 *__restrict__ grid) {
+    constexpr int NA = COMP ? 1 : 3;
+    extern __shared__ __align__(16) float smf[];   // [nodes][pitch]
+    const int w = threadIdx.x >> 5;
+    const int32_t Cn = 2 * R;
+    const SmallLane<COMP> l(Cn, threadIdx.x & 31);
+    const int nodes = kSmallWarps * rpw, pitch = 3 * Cn + 2;
+    const int64_t n0 = int64_t(blockIdx.x) * nodes, n = n0 + w * rpw + l.row;
+    if (l.row < rpw) {
+        float acc[NA] = {};
+        if (n < Ng) gather_row<4>(rec, ptr[n], ptr[n + 1], cT, Cn, l.c, l.a, acc);
+#pragma unroll
+        for (int a = 0; a < NA; ++a) smf[(w * rpw + l.row) * pitch + (l.a + a) * Cn + l.c] = acc[a];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * R * nodes; i += blockDim.x) {
+        const int q = i / nodes, nd = i - q * nodes;   // q = d R + r
+        if (n0 + nd < Ng)
+            grid[int64_t(q) * Ng + n0 + nd] = *reinterpret_cast<const float2 *>(smf + nd * pitch + 2 * q);
+    }
+}
+
+// k_tri_gather of few right-hand sides (mixed form): re and im of a right-hand
+// side sit in neighbouring lanes, each forming its half of Eq. Zb.
+template <bool COMP>
+__global__ void __launch_bounds__(32 * kSmallWarps)
+    k_tri_small(const int64_t *__restrict__ near_ptr, const Rec<float> *__restrict__ near_rec,
+                const int64_t *__restrict__ pt_ptr, const Rec<float> *__restrict__ pt_rec,
+                const float4 *__restrict__ cT, const float4 *__restrict__ phiT, const double *__restrict__ gram,
+                const int32_t *__restrict__ cond, const float2 *__restrict__ coef_dd, int ncond, int64_t nt,
+                int32_t R, int rpw, float4 *__restrict__ y_tri) {
+    constexpr int NA = COMP ? 1 : 3, U = COMP ? 8 : 4;
+    const int64_t gw = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const int32_t Cn = 2 * R;
+    const SmallLane<COMP> l(Cn, lane);
+    const bool act = l.row < rpw && gw * rpw + l.row < nt;
+    const int64_t t = act ? gw * rpw + l.row : 0;
+    float acc[NA] = {};
+    if (act) {
+        gather_row<U>(near_rec, near_ptr[t], near_ptr[t + 1], cT, Cn, l.c, l.a, acc);
+        gather_row<U>(pt_rec, pt_ptr[t], pt_ptr[t + 1], phiT, Cn, l.c, l.a, acc);
+    }
+    const float4 x = cT[t * Cn + l.c];
+    const int cd = cond[t], im = l.c & 1;
+    const int32_t r = l.c >> 1;
+    const float2 *cf = coef_dd + int64_t(r) * (2 * ncond + 1);
+    const float2 zr = cf[2 * cd], zi = cf[2 * cd + 1], cl = cf[2 * ncond];
+    const DD Zr{zr.x, zr.y}, Zi{zi.x, zi.y}, Cl{cl.x, cl.y};
+#pragma unroll
+    for (int a = 0; a < NA; ++a) {
+        const int k = l.a + a;
+        const double *gm = gram + 9 * t + 3 * k;
+        const float G0 = float(__ldg(gm)), G1 = float(__ldg(gm + 1)), G2 = float(__ldg(gm + 2));
+        const float g = G0 * x.x + G1 * x.y + G2 * x.z;
+        const float go = shfl1(g, lane ^ 1), fo = shfl1(acc[a], lane ^ 1);
+        // re = zr gr - zi gi - cl fi,  im = zr gi + zi gr + cl fr (the sums of dd_zb)
+        const DD zg = dd_mul(Zi, go), cfo = dd_mul(Cl, DD{fo, 0.f});
+        const DD y = dd_add(dd_add(dd_mul(Zr, g), im ? zg : dd_neg(zg)), im ? cfo : dd_neg(cfo));
+        if (act) reinterpret_cast<float2 *>(y_tri + (int64_t(r) * nt + t) * 3 + k)[im] = make_float2(y.hi, y.lo);
+    }
+}
+
+// Grid potentials as float4 [node][2R] (k_regroup for few right-hand sides): one
+// thread per (right-hand side, node of a tile with stencil nodes).
+__global__ void __launch_bounds__(256) k_regroup_small(const float2 *__restrict__ grid,
+                                                       const int32_t *__restrict__ tiles, int64_t n_tiles, int64_t Ng,
+                                                       int32_t R, float4 *__restrict__ phiT) {
+    const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    if (w >= n_tiles * R) return;
+    const int64_t r = w % R, n = int64_t(tiles[w / R]) * 32 + (threadIdx.x & 31);
+    if (n >= Ng) return;
+    float2 v[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) v[d] = grid[(int64_t(d) * R + r) * Ng + n];
+    float4 *o = phiT + (n * R + r) * 2;
+    o[0] = make_float4(v[0].x, v[1].x, v[2].x, 0.f);
+    o[1] = make_float4(v[0].y, v[1].y, v[2].y, 0.f);
 }
 
 // Grid currents (Eq. Projection) of the mixed form by node chunks whose
@@ -998,15 +1176,18 @@ int scratch_reserve(pfft_plan *p, int32_t nrhs, int prec) {
         if (a) cudaFree(a);
     s = Scratch{};
     constexpr int kBufs = 9;
+    // bytes per row of the right-hand-sides-inner operands, and of the float4
+    // columns that few right-hand sides use instead
+    const size_t row = std::max(size_t(R) * 3 * cs, size_t(std::min<int64_t>(R, kSmallRhs)) * 2 * sizeof(float4));
     const size_t sizes[kBufs] = {
         size_t(R) * 2 * p->nn * sizeof(double2),
         size_t(R) * 3 * p->Ng * cs,
         size_t(R) * 3 * p->Mx * (p->Ny + (p->large_plane ? p->My : 0)) * p->Nz * cs,
-        size_t(R) * 3 * p->Ng * cs,
+        row * p->Ng,
         size_t(R) * p->nt * 3 * sizeof(double2),
         size_t(R) * (p->nb + p->np) * sizeof(double2),
         size_t(R) * (2 * p->ncond + 1) * (sizeof(double) + sizeof(float2)),
-        size_t(R) * p->nt * 3 * cs,
+        row * p->nt,
         with_far ? size_t(R) * p->nt * 3 * sizeof(float2) : 0};
     void **dst[kBufs] = {&s.tour, &s.grid, &s.spec, &s.phiT, &s.y_tri, &s.y_br, (void **)&s.coef, &s.cT,
                          &s.ffar};
@@ -1148,6 +1329,45 @@ template <typename T, int V, int J> struct Blocks {
         if ((R) > 32) return (R) % 2 == 0 ? Blocks<float, 2, 1>::CALL : Blocks<float, 1, 2>::CALL; \
         SIE_SLAB_DISPATCH(R, CALL);                                                       \
     } while (0)
+// Few-column FP32 gathers: the static kernel with at most kSmallRhs right-hand
+// sides, unless the tuning asks for a path that reads the [row][3][R] operands.
+bool small_rhs(const pfft_plan *p, int32_t R) {
+    return R <= kSmallRhs && p->params.kernel == SIE_KERNEL_STATIC && !(p->kt.near == 1 && R % 2 == 0) &&
+           p->kt.proj_slab != kChunkRhs;
+}
+// A lane per output component (latency) up to kCompRows rows, a lane per column
+// (fewer load wavefronts) above; rows per warp: as many as fit, fewer while that
+// keeps more warps on the chip.
+bool small_comp(int64_t rows, int32_t R) {
+    constexpr int64_t kCompRows = 152 * 32;
+    return R <= 5 && rows <= kCompRows;
+}
+int small_rows(int64_t rows, int32_t R) {
+    constexpr int64_t kFill = 152 * 16;
+    const int64_t fit = 32 / ((small_comp(rows, R) ? 6 : 2) * R);
+    return int(std::max<int64_t>(1, std::min(fit, rows / kFill)));
+}
+int project_small(pfft_plan *p, int32_t R, cudaStream_t st) {
+    const int rpw = small_rows(p->Ng, R), nodes = kSmallWarps * rpw;
+    const unsigned blocks = unsigned((p->Ng + nodes - 1) / nodes);
+    const size_t smem = size_t(nodes) * (6 * R + 2) * sizeof(float);
+    const auto fn = small_comp(p->Ng, R) ? k_project_small<true> : k_project_small<false>;
+    fn<<<blocks, 32 * kSmallWarps, smem, st>>>(p->d_pn_ptr, p->d_pn_rec32, (const float4 *)p->scr.cT, p->Ng, R, rpw,
+                                               (float2 *)p->scr.grid);
+    SIE_LAUNCH_CHECK(p);
+    return SIE_OK;
+}
+int tri_gather_small(pfft_plan *p, int32_t R, cudaStream_t st) {
+    const int rpw = small_rows(p->nt, R);
+    const int64_t rows = int64_t(kSmallWarps) * rpw;
+    const auto fn = small_comp(p->nt, R) ? k_tri_small<true> : k_tri_small<false>;
+    fn<<<unsigned((p->nt + rows - 1) / rows), 32 * kSmallWarps, 0, st>>>(
+        p->d_near_ptr, p->d_near_rec32, p->d_pt_ptr, p->d_pt_rec32, (const float4 *)p->scr.cT,
+        (const float4 *)p->scr.phiT, p->d_gram, p->d_cond, coef_dd(p), p->ncond, p->nt, R, rpw,
+        (float4 *)p->scr.y_tri);
+    SIE_LAUNCH_CHECK(p);
+    return SIE_OK;
+}
 template <typename T> int run_project(pfft_plan *p, int32_t R, cudaStream_t st) {
     if constexpr (is_f32<T>) {
         // mixed form: staged node chunks when asked for (pfft_plan_set_kernel_tuning,
@@ -1203,12 +1423,16 @@ int matvec_t(pfft_plan *p, const double2 *x, double2 *y, int32_t R, int space, c
         k_scan_rows<E><<<R, 1024, 0, st>>>(tour, nslots);
         SIE_LAUNCH_CHECK(p);
     }
-    k_alpha_tri<T><<<nblk(p->nt * R), 256, 0, st>>>(x, p->nl, tour, nslots, p->d_tb, p->d_ts, p->d_loop_of_branch,
-                                                     p->d_twig_node, p->d_head, p->d_enter, p->d_exit, p->nt, R, space,
-                                                     p->nb, (C<T> *)s.cT);
+    const bool small = is_f32<T> && small_rhs(p, R);
+    auto alpha = k_alpha_tri<T, false>;
+    if constexpr (is_f32<T>)
+        if (small) alpha = k_alpha_tri<T, true>;
+    alpha<<<nblk(p->nt * R), 256, 0, st>>>(x, p->nl, tour, nslots, p->d_tb, p->d_ts, p->d_loop_of_branch,
+                                           p->d_twig_node, p->d_head, p->d_enter, p->d_exit, p->nt, R, space, p->nb,
+                                           (C<T> *)s.cT);
     SIE_LAUNCH_CHECK(p);
     tm.reset(new StageTimer(p, SIE_STAGE_PROJECT, st));
-    int rc = run_project<T>(p, R, st);
+    int rc = small ? project_small(p, R, st) : run_project<T>(p, R, st);
     if (rc) return rc;
     tm.reset();
     const int prec = is_df<T> ? SIE_PREC_DF : is_f64<T> ? SIE_PREC_FP64 : SIE_PREC_MIXED;
@@ -1216,7 +1440,11 @@ int matvec_t(pfft_plan *p, const double2 *x, double2 *y, int32_t R, int space, c
     rc = fft_conv(p, s.grid, s.spec, R, prec, st, lossy ? lossy_sel(p, prec) : nullptr);
     if (rc) return rc;
     tm.reset(new StageTimer(p, SIE_STAGE_INTERP, st));
-    {
+    if (small) {
+        k_regroup_small<<<nblk(p->n_tiles * R * 32), 256, 0, st>>>((const float2 *)s.grid, p->d_tiles, p->n_tiles,
+                                                                   p->Ng, R, (float4 *)s.phiT);
+        SIE_LAUNCH_CHECK(p);
+    } else {
         const int32_t B = 3 * R;
         const dim3 grid(unsigned(p->n_tiles), unsigned((B + 31) / 32));
         k_regroup<T><<<grid, 256, 0, st>>>((const C<T> *)s.grid, p->d_tiles, p->Ng, B, (C<T> *)s.phiT);
@@ -1234,6 +1462,9 @@ int matvec_t(pfft_plan *p, const double2 *x, double2 *y, int32_t R, int space, c
         // complex near blocks per frequency: one CUDA-core gather (near + interpolation + y_T)
         tm.reset(new StageTimer(p, SIE_STAGE_NEAR, st));
         rc = run_tri_gather_lossy<T>(p, R, st);
+    } else if (small) {
+        tm.reset(new StageTimer(p, SIE_STAGE_NEAR, st));
+        rc = tri_gather_small(p, R, st);        // near + interpolation + y_T in one gather
     } else if (is_f32<T> && R % 2 == 0 && p->kt.near != 2 && (R >= kNearMmaMinRhs || p->kt.near == 1)) {
         rc = run_far_gather(p, R, st);          // interpolation (step 3) on the CUDA cores
         if (rc) return rc;

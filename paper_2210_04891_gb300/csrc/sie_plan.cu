@@ -400,15 +400,10 @@ __global__ void k_pack_near(const int32_t *__restrict__ col, const double *__res
     int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (e >= n) return;
     Rec<double> a{};
-    Rec<float> b{};
-    for (int i = 0; i < 9; ++i) {
-        a.b[i] = Ld[9 * e + i];
-        b.b[i] = float(a.b[i]);
-    }
+    for (int i = 0; i < 9; ++i) a.b[i] = Ld[9 * e + i];
     a.col = col[e];
-    b.col = col[e];
     r64[e] = a;
-    r32[e] = b;
+    r32[e] = make_rec(a.b, col[e]);
 }
 
 bool is_pow2(int n) { return n >= 2 && (n & (n - 1)) == 0; }
@@ -840,14 +835,8 @@ extern "C" int pfft_plan_create(const sie_mesh *m, const sie_loops *L, const pff
                 b.col = pt_node[e];
             }
         for (int64_t e = 0; e < n_pair; ++e) {
-            pn_rec32[e] = Rec<float>{};
-            pt_rec32[e] = Rec<float>{};
-            for (int i = 0; i < 9; ++i) {
-                pn_rec32[e].b[i] = float(pn_rec64[e].b[i]);
-                pt_rec32[e].b[i] = float(pt_rec64[e].b[i]);
-            }
-            pn_rec32[e].col = int32_t(pn_rec64[e].col);
-            pt_rec32[e].col = int32_t(pt_rec64[e].col);
+            pn_rec32[e] = make_rec(pn_rec64[e].b, int32_t(pn_rec64[e].col));
+            pt_rec32[e] = make_rec(pt_rec64[e].b, int32_t(pt_rec64[e].col));
         }
     }
     std::vector<int32_t> tiles;

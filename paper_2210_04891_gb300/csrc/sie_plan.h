@@ -20,6 +20,10 @@ template <typename T> struct DevBuf {
 // triangles staged per chunk, kChunkRhs right-hand sides per slab.
 constexpr int kChunkTri = 64;
 constexpr int kChunkRhs = 32;
+// Largest right-hand-side count of the few-column FP32 gathers (2R columns fill
+// a warp).  Their dense operands are float4 [row][2R], the three components of
+// a real column side by side, so that a lane reads its operand in one load.
+constexpr int kSmallRhs = 16;
 
 struct PrecondState;   // sie_solve.cu
 struct LossyCache;     // sie_lossy.cu
@@ -35,12 +39,14 @@ struct Scratch {
     void *spec = nullptr;      // complex T [3R][Mx][Ny][Nz]  grids transformed along x, then (large
                                // planes) [3R][Mx][My][Nz] the same transformed along y
     void *phiT = nullptr;      // complex T [Ng][3][R]   grid potentials, right-hand sides innermost
+                               // (few right-hand sides in FP32: float4 [Ng][2R], see kSmallRhs)
     void *y_tri = nullptr;     // [R][nt][3]
     void *y_br = nullptr;      // [R][nb + np]
     // per RHS: Z_s per conductor (re, im), c_L (im) -> double [R][2 ncond + 1],
     // followed by the same table as double-float (hi, lo) pairs, see coef_dd()
     double *coef = nullptr;
     void *cT = nullptr;        // complex T [nt][3][R]  local currents, right-hand sides innermost
+                               // (few right-hand sides in FP32: float4 [nt][2R], see kSmallRhs)
     void *ffar = nullptr;      // complex64 [nt][3][R]  interpolated far field (mixed form)
     size_t bytes = 0;
 };

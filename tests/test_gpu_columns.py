@@ -1,11 +1,13 @@
-"""The FP64 and double-float gathers by real columns (projection, near field,
-interpolation) at every team shape: groups of lanes per row for up to 8
-right-hand sides, one to four column sets per lane above, ragged last slabs.
+"""The gathers by real columns (projection, near field, interpolation) at every
+team shape: FP64 and double-float with groups of lanes per row for up to 8
+right-hand sides, one to four column sets per lane above, ragged last slabs;
+FP32 with several rows per warp for up to 16 right-hand sides, one row above.
 
-Every right-hand side is compared with the oracle pFFT (FP64 1e-10, the parity
-bar of both forms), and must equal, bit for bit, the product of that
-right-hand side alone: the order of a row's sum does not depend on how many
-right-hand sides share the call.
+Every right-hand side is compared with the oracle pFFT (1e-10 for FP64 and
+double-float, 1e-5 for the mixed form: their parity bars), and must equal, bit
+for bit, the product of that right-hand side alone: the order of a row's sum
+does not depend on how many right-hand sides share the call (mixed form: below
+the 96 at which the near field changes to the tensor cores).
 """
 import numpy as np
 import pytest
@@ -17,7 +19,7 @@ from oracle.pfft import PfftSystem, PfftParams
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from paper_2210_04891_gb300 import api, SPACE_LOOP, PREC_FP64, PREC_DF  # noqa: E402
+from paper_2210_04891_gb300 import api, SPACE_LOOP, PREC_FP64, PREC_MIXED, PREC_DF  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -33,7 +35,7 @@ def system():
     ref = np.stack([S.matvec(x[r], om[r]) for r in range(130)])
     xt = torch.from_numpy(x).cuda()
     alone = {prec: torch.cat([api.pfft_matvec(P, xt[r:r + 1], om[r:r + 1], SPACE_LOOP, prec) for r in range(130)])
-             for prec in (PREC_FP64, PREC_DF)}
+             for prec in (PREC_FP64, PREC_DF, PREC_MIXED)}
     return P, om, xt, ref, alone
 
 
@@ -43,5 +45,17 @@ def test_columns_match_oracle_and_single_right_hand_side(system, R, prec):
     P, om, xt, ref, alone = system
     y = api.pfft_matvec(P, xt[:R].contiguous(), om[:R], SPACE_LOOP, prec)
     assert torch.equal(y, alone[prec][:R])
-    err = np.linalg.norm(y.cpu().numpy() - ref[:R], axis=1) / np.linalg.norm(ref[:R], axis=1)
-    assert err.max() < 1e-10
+    check(y, ref[:R], 1e-10)
+
+
+@pytest.mark.parametrize("R", [1, 2, 3, 4, 5, 6, 8, 10, 11, 15, 16, 17, 31, 32, 33, 48, 65, 95])
+def test_mixed_columns_match_oracle_and_single_right_hand_side(system, R):
+    P, om, xt, ref, alone = system
+    y = api.pfft_matvec(P, xt[:R].contiguous(), om[:R], SPACE_LOOP, PREC_MIXED)
+    assert torch.equal(y, alone[PREC_MIXED][:R])
+    check(y, ref[:R], 1e-5)
+
+
+def check(y, ref, tol):
+    err = np.linalg.norm(y.cpu().numpy() - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert err.max() < tol
