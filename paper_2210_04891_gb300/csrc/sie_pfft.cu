@@ -409,14 +409,22 @@ __device__ __forceinline__ df col_sum(df a, df b) { return df_qadd(a, b); }
 __device__ __forceinline__ double col_val(double a) { return a; }
 __device__ __forceinline__ df col_val(df a) { return df_norm(a); }
 
-// Lane of a row's team: G groups of C lanes, 32 / (G C) rows per warp (one
-// group and J column sets when C > 16).
+// Lane of a row's team: G groups of C lanes, 32 / (G C) rows per warp while C <= 16
+// (J = 1); above, one row, one group and J column sets.
 template <int J, int G> struct ColLane {
     int row, rpw, g;   // row of the warp's rpw rows, group
     int32_t c[J];      // columns (lanes beyond the last column repeat a valid one)
     bool col[J], on;   // column exists; lane belongs to a row
     __device__ __forceinline__ ColLane(int32_t C, int32_t slab0, int lane) {
-        if constexpr (G == 1) {
+        static_assert(J == 1 || G == 1, "one column per lane in a group");
+        if (J == 1 && C <= 16) {
+            rpw = 32 / (G * C);
+            row = lane / (G * C);
+            g = (lane - row * G * C) / C;
+            c[0] = lane - (row * G + g) * C;
+            on = row < rpw;
+            col[0] = on;
+        } else {
             row = g = 0;
             rpw = 1;
             on = true;
@@ -425,21 +433,15 @@ template <int J, int G> struct ColLane {
                 col[j] = slab0 + lane + 32 * j < C;
                 c[j] = col[j] ? slab0 + lane + 32 * j : slab0 + (lane & 1);
             }
-        } else {
-            static_assert(J == 1, "one column per lane in a group");
-            rpw = 32 / (G * C);
-            row = lane / (G * C);
-            g = (lane - row * G * C) / C;
-            c[0] = lane - (row * G + g) * C;
-            on = row < rpw;
-            col[0] = on;
         }
     }
 };
+// rows per warp of such a team
+template <int J, int G> int cols_rpw(int32_t R) { return J == 1 && R <= 8 ? 32 / (G * 2 * R) : 1; }
 
 // v[a][j] = sum over row [e0, e1) of sum_b rec.b[3a+b] X[col][b][c[j]], in the
 // order described above, in the lanes of group 0.  Every lane of the warp calls.
-template <typename T, int J, int G, int SEG>
+template <typename T, int J, int G, int SEG, int UNR>
 __device__ __forceinline__ void gather_cols(const Rec<T> *__restrict__ rec, int64_t e0, int64_t e1,
                                             const T *__restrict__ X, int32_t C, const ColLane<J, G> &l, int lane,
                                             T (&v)[3][J]) {
@@ -457,7 +459,7 @@ __device__ __forceinline__ void gather_cols(const Rec<T> *__restrict__ rec, int6
             for (int j = 0; j < J; ++j) acc[a][j] = T(0.0);
         const int s = l.g * PER + q;
         const int64_t b0 = e0 + len * s / SEG, b1 = e0 + len * (s + 1) / SEG;
-#pragma unroll 2
+#pragma unroll UNR
         for (int64_t e = b0; e < b1; ++e) {
             T b[9];
             const int64_t col = load_rec<T>(rec + e, b);
@@ -499,10 +501,13 @@ __device__ __forceinline__ void gather_cols(const Rec<T> *__restrict__ rec, int6
 }
 
 // Grid currents as k_project, by real columns: a warp takes its rpw nodes, a
-// block kProjNodes of them (8 warps' worth), grid (node blocks, slabs of 32 J
-// columns).  FP64, bond wires: 48 right-hand sides 3.82 ms (6.29 with a complex
-// right-hand side per lane), 20k triangles and 8: 0.235 (1.19) ms.
-constexpr int kProjSeg = 4, kTriSeg = 8;   // runs per row (a node has about 20 records, a triangle 300)
+// block 8 warps' worth, grid (node blocks, slabs of 32 J columns).  A node has
+// some 20 records: four runs in FP64, which is bound by its pipe (bond wires, 48
+// right-hand sides: 3.84 ms, 6.29 with a complex right-hand side per lane; bar, one:
+// 16 us, 30 in one run), one in double-float, where starting a run shows (same
+// sizes: 1.18 ms in one run, 1.70 in four, 1.51 with complex lanes).
+template <typename T> constexpr int kProjSeg = is_f64<T> ? 4 : 1;
+constexpr int kTriSeg = 8;   // runs per triangle (about 300 near, 60 grid records)
 // shared pitch of a node, 2 x odd: the 8-node reads of the store hit distinct banks
 template <typename T, int J> __host__ __device__ constexpr int proj_cols_pitch() { return 3 * 32 * J + 2; }
 template <typename T, int J, int G>
@@ -516,13 +521,11 @@ __global__ void __launch_bounds__(256) k_project_cols(const int64_t *__restrict_
     const int32_t Cn = 2 * R, slab0 = int32_t(blockIdx.y) * SLAB;
     const ColLane<J, G> l(Cn, slab0, lane);
     const int nodes = kProjNodes * l.rpw;
-    // several nodes per warp: their columns fit one pitch of the single-node form
-    const int pitch = G == 1 ? ROWS : 3 * Cn + 2;
+    const int dstep = l.rpw > 1 ? Cn : SLAB, pitch = l.rpw > 1 ? 3 * Cn + 2 : ROWS;
     const int64_t n0 = int64_t(blockIdx.x) * nodes, n = n0 + w * l.rpw + l.row;
     T v[3][J];
     const bool act = l.on && n < Ng;
-    gather_cols<T, J, G, kProjSeg>(rec, act ? ptr[n] : 0, act ? ptr[n + 1] : 0, cT, Cn, l, lane, v);
-    const int dstep = G == 1 ? SLAB : Cn;
+    gather_cols<T, J, G, kProjSeg<T>, 1>(rec, act ? ptr[n] : 0, act ? ptr[n + 1] : 0, cT, Cn, l, lane, v);
     if (l.on && l.g == 0) {
 #pragma unroll
         for (int a = 0; a < 3; ++a)
@@ -931,8 +934,8 @@ __global__ void __launch_bounds__(256)
     const bool act = l.on && t0 + l.row < nt;
     const int64_t t = act ? t0 + l.row : t0;
     T acc[3][J], far[3][J];
-    gather_cols<T, J, G, kTriSeg>(near_rec, near_ptr[t], near_ptr[t + 1], cT, Cn, l, lane, acc);
-    gather_cols<T, J, G, kTriSeg>(pt_rec, pt_ptr[t], pt_ptr[t + 1], phiT, Cn, l, lane, far);
+    gather_cols<T, J, G, kTriSeg, 2>(near_rec, near_ptr[t], near_ptr[t + 1], cT, Cn, l, lane, acc);
+    gather_cols<T, J, G, kTriSeg, 2>(pt_rec, pt_ptr[t], pt_ptr[t + 1], phiT, Cn, l, lane, far);
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -1229,19 +1232,18 @@ template <typename T> const Rec<T> *rec_near(const pfft_plan *p) {
 // lane, G groups of lanes per row.
 template <typename T, int J, int G> struct Cols {
     static int project(pfft_plan *p, int32_t R, cudaStream_t st) {
-        constexpr int GP = G < kProjSeg ? G : kProjSeg;
-        const int nodes = kProjNodes * (GP == 1 ? 1 : 32 / (GP * 2 * R));
+        constexpr int GP = G < kProjSeg<T> ? G : kProjSeg<T>;
+        const int rpw = cols_rpw<J, GP>(R), nodes = kProjNodes * rpw;
         const dim3 grid(unsigned((p->Ng + nodes - 1) / nodes), unsigned((2 * R + 32 * J - 1) / (32 * J)));
-        const size_t smem = size_t(nodes) * (GP == 1 ? proj_cols_pitch<T, J>() : 6 * R + 2) * sizeof(T);
-        k_project_cols<T, J, GP><<<grid, 32 * kProjNodes, smem, st>>>(p->d_pn_ptr, rec_pn<T>(p),
-                                                                      (const T *)p->scr.cT, p->Ng, R,
-                                                                      (C<T> *)p->scr.grid);
+        const size_t smem = size_t(nodes) * (rpw > 1 ? 6 * R + 2 : proj_cols_pitch<T, J>()) * sizeof(T);
+        k_project_cols<T, J, GP><<<grid, 32 * kProjNodes, smem, st>>>(p->d_pn_ptr, rec_pn<T>(p), (const T *)p->scr.cT,
+                                                                  p->Ng, R, (C<T> *)p->scr.grid);
         SIE_LAUNCH_CHECK(p);
         return SIE_OK;
     }
     static int tri_gather(pfft_plan *p, int32_t R, cudaStream_t st) {
         const int32_t nslab = (2 * R + 32 * J - 1) / (32 * J);
-        const int rpw = G == 1 ? 1 : 32 / (G * 2 * R);
+        const int rpw = cols_rpw<J, G>(R);
         const int64_t warps = (p->nt + rpw - 1) / rpw * nslab;
         k_tri_cols<T, J, G><<<unsigned((warps * 32 + 255) / 256), 256, 0, st>>>(
             p->d_near_ptr, rec_near<T>(p), p->d_pt_ptr, rec_pt<T>(p), (const T *)p->scr.cT, (const T *)p->scr.phiT,
@@ -1250,20 +1252,28 @@ template <typename T, int J, int G> struct Cols {
         return SIE_OK;
     }
 };
-// C = 2R columns: up to 16 of them the most groups that fit a warp (R <= 2: 8,
-// R <= 4: 4, R <= 8: 2); above, the J of the fewest equal slabs of at most 128.
-#define SIE_COLS_DISPATCH(T, R, CALL)                                         \
-    do {                                                                     \
-        if ((R) <= 2) return Cols<T, 1, 8>::CALL;                            \
-        if ((R) <= 4) return Cols<T, 1, 4>::CALL;                            \
-        if ((R) <= 8) return Cols<T, 1, 2>::CALL;                            \
-        const int32_t sets = (2 * (R) + 31) / 32, slabs = (sets + 3) / 4;    \
-        switch ((sets + slabs - 1) / slabs) {                                \
-            case 1: return Cols<T, 1, 1>::CALL;                              \
-            case 2: return Cols<T, 2, 1>::CALL;                              \
-            case 3: return Cols<T, 3, 1>::CALL;                              \
-            default: return Cols<T, 4, 1>::CALL;                             \
-        }                                                                    \
+// Column sets per lane above 16 right-hand sides.  FP64 takes one: its pipe needs
+// 144 cycles per record and set, so reading a record once per set costs nothing
+// (bond wires, 48 right-hand sides, near field: 20.2 ms with one, 20.4 with three).  In
+// double-float a set's arithmetic (27 cycles) is of the order of the record's
+// loads: three or two sets, whichever wastes fewer lanes (6.62, 8.31 and 5.93 ms
+// with one, two and three sets, two having a quarter of its lanes idle there).
+template <typename T> int col_sets(int32_t R) {
+    const int sets = (2 * R + 31) / 32;
+    if (is_f64<T> || sets == 1) return 1;
+    return (sets + 2) / 3 * 3 <= (sets + 1) / 2 * 2 ? 3 : 2;
+}
+// Up to 8 right-hand sides the most groups that fit a warp.
+#define SIE_COLS_DISPATCH(T, R, CALL)                                       \
+    do {                                                                   \
+        if ((R) <= 2) return Cols<T, 1, 8>::CALL;                          \
+        if ((R) <= 4) return Cols<T, 1, 4>::CALL;                          \
+        if ((R) <= 8) return Cols<T, 1, 2>::CALL;                          \
+        if constexpr (is_df<T>) {                                          \
+            if (col_sets<T>(R) == 2) return Cols<T, 2, 1>::CALL;           \
+            if (col_sets<T>(R) == 3) return Cols<T, 3, 1>::CALL;           \
+        }                                                                  \
+        return Cols<T, 1, 1>::CALL;                                        \
     } while (0)
 
 // Block-sparse stages for one slab shape: V complex per load, J loads per lane
