@@ -46,6 +46,39 @@ template <> __host__ __device__ __forceinline__ cdf cadd<cdf>(cdf a, cdf b) {
 template <> __host__ __device__ __forceinline__ cdf csub<cdf>(cdf a, cdf b) {
     return cdf{df_qadd(a.x, -b.x), df_qadd(a.y, -b.y)};
 }
+// a times conj(b)
+template <typename V> __host__ __device__ __forceinline__ V cmulc(V a, V b) {
+    V z;
+    z.x = a.x * b.x + a.y * b.y;
+    z.y = a.y * b.x - a.x * b.y;
+    return z;
+}
+// Double-float a c + b d, a fused product sum: both high products exact (FMA
+// two-product), one two-sum of them, every error and cross product in the low
+// part, unnormalised as the sums above.  16 FP32 operations against 27 for two
+// normalised products and a normalised sum.
+__host__ __device__ __forceinline__ df df_dot2(df a, df c, df b, df d) {
+    const float p = a.hi * c.hi, q = b.hi * d.hi;
+    const float s = p + q, bb = s - p;
+    float l = fmaf(a.hi, c.hi, -p) + fmaf(b.hi, d.hi, -q);
+    l += (p - (s - bb)) + (q - bb);
+    l = fmaf(a.hi, c.lo, fmaf(a.lo, c.hi, l));
+    return df(s, fmaf(b.hi, d.lo, fmaf(b.lo, d.hi, l)));
+}
+template <> __host__ __device__ __forceinline__ cdf cmul<cdf>(cdf a, cdf b) {
+    return cdf{df_dot2(a.x, b.x, a.y, -b.y), df_dot2(a.x, b.y, a.y, b.x)};
+}
+template <> __host__ __device__ __forceinline__ cdf cmulc<cdf>(cdf a, cdf b) {
+    return cdf{df_dot2(a.x, b.x, a.y, b.y), df_dot2(a.y, b.x, a.x, -b.y)};
+}
+// times a real double-float, unnormalised
+__host__ __device__ __forceinline__ df df_scale(df a, df h) {
+    const float p = a.hi * h.hi;
+    return df(p, fmaf(a.hi, h.lo, fmaf(a.lo, h.hi, fmaf(a.hi, h.hi, -p))));
+}
+template <> __host__ __device__ __forceinline__ cdf cscale<cdf, df>(cdf a, df h) {
+    return cdf{df_scale(a.x, h), df_scale(a.y, h)};
+}
 // multiply by -i (forward) or +i (inverse)
 template <typename V> __device__ __forceinline__ V mul_mi(V a, bool inv) {
     V z;

@@ -11,6 +11,8 @@
 // single buffer suffices.  Twiddles come from a table W[m] = exp(-2 pi i m / M).
 #pragma once
 
+#include <type_traits>
+
 #include "sie_common.cuh"
 
 namespace sie {
@@ -247,8 +249,12 @@ __device__ __forceinline__ C<T> twiddle_mul(C<T> b, int t) {
         if (INV) { r.x = -b.y; r.y = b.x; } else { r.x = b.y; r.y = -b.x; }
     } else {
         const T c = T(c16(t)), sn = INV ? T(s16(t)) : T(-s16(t));
-        r.x = b.x * c - b.y * sn;
-        r.y = b.x * sn + b.y * c;
+        if constexpr (std::is_same<T, df>::value) {
+            r = cmul(b, cdf{c, sn});
+        } else {
+            r.x = b.x * c - b.y * sn;
+            r.y = b.x * sn + b.y * c;
+        }
     }
     if (neg) { r.x = -r.x; r.y = -r.y; }
     return r;
@@ -270,10 +276,14 @@ template <typename T, bool INV>
 __device__ __forceinline__ C<T> twiddle32(C<T> b, int t) {
     if ((t & 1) == 0) return twiddle_mul<T, INV>(b, t >> 1);
     const T c = T(c32(t)), sn = INV ? T(s32(t)) : T(-s32(t));
-    C<T> r;
-    r.x = b.x * c - b.y * sn;
-    r.y = b.x * sn + b.y * c;
-    return r;
+    if constexpr (std::is_same<T, df>::value) {
+        return cmul(b, cdf{c, sn});
+    } else {
+        C<T> r;
+        r.x = b.x * c - b.y * sn;
+        r.y = b.x * sn + b.y * c;
+        return r;
+    }
 }
 
 template <typename T, int N, bool INV, int NA>
@@ -336,6 +346,215 @@ __device__ __forceinline__ void dft_reg(C<T> (&v)[NA]) {
     }
 }
 
+// ---- The four short transforms of a four-step pass pair, by precision.
+//   fwd1: DFT_N1 over j1 of inputs that are zero for j1 >= N1 / 2;
+//   fwd2: DFT_N2 over j2;  inv1: inverse DFT_N2 over k2;
+//   inv2: inverse DFT_N1 over k1, of which the outputs p1 < N1 / 2 are kept.
+// The twiddles W_M^(j2 k1) between them are where they cost least.
+//
+// FP32: on the outputs of fwd1 and inv1 (tables tf, ti below); every input and
+// output of the short transforms is computed.
+template <typename T, int N1, int N2> struct FourStep {
+    template <int NA> static __device__ __forceinline__ void fwd1(C<T> (&v)[NA], int j2, const C<T> *tf) {
+#pragma unroll
+        for (int j1 = N1 / 2; j1 < N1; ++j1) v[j1] = mk<T>(T(0), T(0));
+        dft_reg<T, N1, false>(v);
+        const C<T> *t = tf + j2 * N1;
+#pragma unroll
+        for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmul(v[k1], t[k1]);
+    }
+    template <int NA> static __device__ __forceinline__ void fwd2(C<T> (&v)[NA], int, const C<T> *) {
+        dft_reg<T, N2, false>(v);
+    }
+    template <int NA> static __device__ __forceinline__ void inv1(C<T> (&v)[NA], int k1, const C<T> *ti) {
+        dft_reg<T, N2, true>(v);
+        const C<T> *t = ti + k1 * N2;
+#pragma unroll
+        for (int p2 = 1; p2 < N2; ++p2) v[p2] = cmulc(v[p2], t[p2]);
+    }
+    template <int NA> static __device__ __forceinline__ void inv2(C<T> (&v)[NA], int, const C<T> *) {
+        dft_reg<T, N1, true>(v);
+    }
+};
+
+// Double-float: the same places, with the short transforms pruned and products
+// fused (bond wires, 48 right-hand sides: (y, z) planes 9.73 -> 6.92 ms).  Zero-padded:
+// the even outputs are DFT_N/2 of the inputs, the odd ones that of v[j] W_N^j.
+// Cropped: out[p] = E[p] + W_N^-p O[p], E and O the half transforms of the even
+// and odd inputs.
+template <int N, int NA> __device__ __forceinline__ void df_dft_zpad(cdf (&v)[NA]) {
+    constexpr int H = N / 2;
+    if constexpr (N == 2) {
+        v[1] = v[0];
+    } else {
+        cdf e[H], o[H];
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            e[j] = v[j];
+            o[j] = j ? twiddle_mul<df, false>(v[j], j * (16 / N)) : v[j];
+        }
+        dft_reg<df, H, false>(e);
+        dft_reg<df, H, false>(o);
+#pragma unroll
+        for (int m = 0; m < H; ++m) {
+            v[2 * m] = e[m];
+            v[2 * m + 1] = o[m];
+        }
+    }
+}
+template <int N, int NA> __device__ __forceinline__ void df_idft_half(cdf (&v)[NA]) {
+    constexpr int H = N / 2;
+    if constexpr (N == 2) {
+        v[0] = cadd(v[0], v[1]);
+    } else {
+        cdf e[H], o[H];
+#pragma unroll
+        for (int m = 0; m < H; ++m) {
+            e[m] = v[2 * m];
+            o[m] = v[2 * m + 1];
+        }
+        dft_reg<df, H, true>(e);
+        dft_reg<df, H, true>(o);
+#pragma unroll
+        for (int p = 0; p < H; ++p) v[p] = cadd(e[p], p ? twiddle_mul<df, true>(o[p], p * (16 / N)) : o[p]);
+    }
+}
+template <int N1, int N2> struct FourStep<df, N1, N2> {
+    template <int NA> static __device__ __forceinline__ void fwd1(cdf (&v)[NA], int j2, const cdf *tf) {
+        df_dft_zpad<N1>(v);
+        const cdf *t = tf + j2 * N1;
+#pragma unroll
+        for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmul(v[k1], t[k1]);
+    }
+    template <int NA> static __device__ __forceinline__ void fwd2(cdf (&v)[NA], int, const cdf *) {
+        dft_reg<df, N2, false>(v);
+    }
+    template <int NA> static __device__ __forceinline__ void inv1(cdf (&v)[NA], int k1, const cdf *ti) {
+        dft_reg<df, N2, true>(v);
+        const cdf *t = ti + k1 * N2;
+#pragma unroll
+        for (int p2 = 1; p2 < N2; ++p2) v[p2] = cmulc(v[p2], t[p2]);
+    }
+    template <int NA> static __device__ __forceinline__ void inv2(cdf (&v)[NA], int, const cdf *) {
+        df_idft_half<N1>(v);
+    }
+};
+
+// FP64: bound by the FP64 pipe, where an add, a product and an FMA cost the same.
+// Radix-2 decimation in time takes six FMAs per butterfly whatever its twiddle
+// (a + w b: four; a - w b = 2 a - (a + w b): two), so the twiddles W_M^(j2 k1)
+// ride in the butterflies of the second transform (fwd2, inv2) for nothing:
+// input j of a length-N transform carries theta^j, theta = W_M^k1, and the level
+// of length n uses theta^(N/n) W_n^k, k < n / 4 (the rest are -i times those),
+// read from the axis's table of roots W_M^m.  Zero-padded inputs remove the
+// first level, cropped outputs half of the last.  Per 8 + 16-point pair of a
+// 128-point axis, FP64 operations: zero-padded DFT_8 36, twiddled DFT_16 192,
+// inverse DFT_16 148, twiddled cropped DFT_8 64 (radix-4 with separate twiddles
+// and no pruning: 84, 160, 220, 56).  Bond wires, 48 right-hand sides: (y, z)
+// planes 32.0 -> 26.8 ms, x pencils 3.35 -> 2.60 and 3.21 -> 2.74 ms.
+__host__ __device__ constexpr double cr32(int t) { return t % 2 ? c32(t) : c16(t / 2); }   // cos 2 pi t / 32
+__host__ __device__ constexpr double sr32(int t) { return t % 2 ? s32(t) : s16(t / 2); }   // t in [0, 16)
+
+// Inputs v[S0 + ST j], j < N, outputs o[k] natural order (k < N / 2 with HALF).
+// TW: w[n / 4 + k] (n = 2: w[0]) as above.  ZP: inputs j >= N / 2 of the whole
+// transform are zero.  SC: inputs times the real h.
+template <int N, bool INV, bool TW, bool ZP, bool HALF, bool SC, int S0, int ST, int NA, int NW, int NH, int NO>
+__device__ __forceinline__ void dit(const double2 (&v)[NA], const double2 (&w)[NW], const double (&h)[NH],
+                                    double2 (&o)[NO]) {
+    constexpr int H = N / 2;
+    if constexpr (N == 1) {
+        o[0] = v[S0];
+    } else if constexpr (N == 2 && ZP) {
+        o[0] = o[1] = v[S0];
+    } else if constexpr (N == 2 && SC) {
+        const double hb = h[S0 + ST];
+        const double2 a = cscale(v[S0], h[S0]), b = v[S0 + ST];
+        o[0] = make_double2(__fma_rn(b.x, hb, a.x), __fma_rn(b.y, hb, a.y));
+        o[1] = make_double2(__fma_rn(-b.x, hb, a.x), __fma_rn(-b.y, hb, a.y));
+    } else {
+        double2 e[H], d[H];
+        dit<H, INV, TW, ZP, false, SC, S0, 2 * ST>(v, w, h, e);
+        dit<H, INV, TW, ZP, false, SC, S0 + ST, 2 * ST>(v, w, h, d);
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            constexpr int Q = N >= 4 ? N / 4 : 1;
+            if (!TW && k == 0) {
+                o[0] = cadd(e[0], d[0]);
+                if (!HALF) o[H] = csub(e[0], d[0]);
+            } else if (!TW && k == Q) {            // -i (forward), +i (inverse)
+                const double2 t = INV ? make_double2(-d[k].y, d[k].x) : make_double2(d[k].y, -d[k].x);
+                o[k] = cadd(e[k], t);
+                if (!HALF) o[k + H] = csub(e[k], t);
+            } else {
+                double wx, wy;
+                if constexpr (TW) {
+                    const double2 t = w[N / 4 + k % Q];
+                    if (k < Q) { wx = t.x; wy = t.y; }
+                    else if (INV) { wx = -t.y; wy = t.x; }
+                    else { wx = t.y; wy = -t.x; }
+                } else {
+                    wx = cr32(k * (32 / N));
+                    wy = INV ? sr32(k * (32 / N)) : -sr32(k * (32 / N));
+                }
+                const double2 a = e[k], b = d[k];
+                const double2 r = make_double2(__fma_rn(-wy, b.y, __fma_rn(wx, b.x, a.x)),
+                                               __fma_rn(wy, b.x, __fma_rn(wx, b.y, a.y)));
+                o[k] = r;
+                if (!HALF) o[k + H] = make_double2(__fma_rn(2.0, a.x, -r.x), __fma_rn(2.0, a.y, -r.y));
+            }
+        }
+    }
+}
+// twiddles of a length-N transform whose input j carries W_M^(q j) (conjugated with INV)
+template <int N, int M, bool INV, int NW>
+__device__ __forceinline__ void dit_twiddles(int q, const double2 *__restrict__ root, double2 (&w)[NW]) {
+#pragma unroll
+    for (int n = 2; n <= N; n *= 2)
+#pragma unroll
+        for (int k = 0; k < (n >= 4 ? n / 4 : 1); ++k) {
+            double2 t = __ldg(root + q * (N / n) + k * (M / n));
+            if (INV) t.y = -t.y;
+            w[n / 4 + k] = t;
+        }
+}
+template <int N1, int N2> struct FourStep<double, N1, N2> {
+    static constexpr int M = N1 * N2;
+    template <int N, bool INV, bool TW, bool ZP, bool HALF, bool SC, int NA, int NW, int NH>
+    static __device__ __forceinline__ void go(double2 (&v)[NA], const double2 (&w)[NW], const double (&h)[NH]) {
+        double2 o[N];
+        dit<N, INV, TW, ZP, HALF, SC, 0, 1>(v, w, h, o);
+#pragma unroll
+        for (int i = 0; i < (HALF ? N / 2 : N); ++i) v[i] = o[i];
+    }
+    template <int NA> static __device__ __forceinline__ void fwd1(double2 (&v)[NA], int, const double2 *) {
+        const double2 w[1] = {};
+        const double h[1] = {};
+        go<N1, false, false, true, false, false>(v, w, h);
+    }
+    template <int NA> static __device__ __forceinline__ void fwd2(double2 (&v)[NA], int k1, const double2 *root) {
+        double2 w[N2 / 2];
+        const double h[1] = {};
+        dit_twiddles<N2, M, false>(k1, root, w);
+        go<N2, false, true, false, false, false>(v, w, h);
+    }
+    template <int NA> static __device__ __forceinline__ void inv1(double2 (&v)[NA], int, const double2 *) {
+        const double2 w[1] = {};
+        const double h[1] = {};
+        go<N2, true, false, false, false, false>(v, w, h);
+    }
+    // inverse of v times the real h
+    template <int NA> static __device__ __forceinline__ void inv1_scaled(double2 (&v)[NA], const double (&h)[N2]) {
+        const double2 w[1] = {};
+        go<N2, true, false, false, false, true>(v, w, h);
+    }
+    template <int NA> static __device__ __forceinline__ void inv2(double2 (&v)[NA], int p2, const double2 *root) {
+        double2 w[N1 > 2 ? N1 / 2 : 1];
+        const double h[1] = {};
+        dit_twiddles<N1, M, true>(p2, root, w);
+        go<N1, true, true, false, true, false>(v, w, h);
+    }
+};
+
 // M -> (N1, N2): 8 = 2x4, 16 = 4x4, 32 = 4x8, 64 = 8x8, 128 = 8x16, 256 = 16x16
 inline void split4(int M, int &N1, int &N2) {
     int lg = 0;
@@ -377,7 +596,8 @@ template <int N1, int N2> struct Pencil {
 
 // Four-step twiddle tables of an axis of length M = N1 N2 (built at plan
 // creation): tf[j2 * N1 + k1] = W_M^(j2 k1) for the forward pass 1 and
-// ti[k1 * N2 + p2] = W_M^(k1 p2) for the inverse pass A (used conjugated).
+// ti[k1 * N2 + p2] = W_M^(k1 p2) for the inverse pass A (used conjugated); in
+// FP64 both are the table of roots root[m] = W_M^m instead (see FourStep).
 
 // ---- x pencils.  Buffers [batch][rows][ncols], row x at x * ncols; one CTA
 // per (batch, KT consecutive columns), KT * max(N1, N2) threads, a shared
@@ -402,18 +622,17 @@ __global__ void __launch_bounds__(256) k_fft_xf(const C<T> *__restrict__ in, C<T
         const int j2 = q;
         const C<T> *src = in + int64_t(b) * (M / 2) * ncols + c0 + line + int64_t(j2) * ncols;
 #pragma unroll
-        for (int j1 = 0; j1 < N1; ++j1) v[j1] = j1 < H1 ? src[j1 * stride] : mk<T>(T(0), T(0));
-        dft_reg<T, N1, false>(v);
-        const C<T> *t = tf + j2 * N1;
+        for (int j1 = 0; j1 < H1; ++j1) v[j1] = src[j1 * stride];
+        FourStep<T, N1, N2>::fwd1(v, j2, tf);
 #pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) Sl[k1 * N2 + j2] = k1 ? cmul(v[k1], t[k1]) : v[0];
+        for (int k1 = 0; k1 < N1; ++k1) Sl[k1 * N2 + j2] = v[k1];
     }
     __syncthreads();
     if (q < N1) {                      // pass 2: k1 = q, DFT over j2 -> X[k1 + N1 k2]
         const int k1 = q;
 #pragma unroll
         for (int j2 = 0; j2 < N2; ++j2) v[j2] = Sl[k1 * N2 + j2];
-        dft_reg<T, N2, false>(v);
+        FourStep<T, N1, N2>::fwd2(v, k1, tf);
         C<T> *dst = out + int64_t(b) * M * ncols + c0 + line + int64_t(k1) * ncols;
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) dst[N1 * k2 * int64_t(ncols)] = v[k2];
@@ -437,25 +656,16 @@ __global__ void __launch_bounds__(256) k_fft_xi(const C<T> *__restrict__ in, C<T
         const C<T> *src = in + int64_t(b) * M * ncols + c0 + line + int64_t(k1) * ncols;
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) v[k2] = src[N1 * k2 * int64_t(ncols)];
-        dft_reg<T, N2, true>(v);
-        const C<T> *t = ti + k1 * N2;
+        FourStep<T, N1, N2>::inv1(v, k1, ti);
 #pragma unroll
-        for (int p2 = 0; p2 < N2; ++p2) {
-            C<T> r = v[p2];
-            if (p2) {
-                const C<T> w = t[p2];
-                r.x = v[p2].x * w.x + v[p2].y * w.y;
-                r.y = v[p2].y * w.x - v[p2].x * w.y;
-            }
-            Sl[p2 * N1 + k1] = r;
-        }
+        for (int p2 = 0; p2 < N2; ++p2) Sl[p2 * N1 + k1] = v[p2];
     }
     __syncthreads();
     if (q < N2) {                      // pass B: p2 = q, inverse DFT over k1, x = p2 + N2 p1 < M/2
         const int p2 = q;
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) v[k1] = Sl[p2 * N1 + k1];
-        dft_reg<T, N1, true>(v);
+        FourStep<T, N1, N2>::inv2(v, p2, ti);
         C<T> *dst = out + int64_t(b) * (M / 2) * ncols + c0 + line + int64_t(p2) * ncols;
 #pragma unroll
         for (int p1 = 0; p1 < H1; ++p1) dst[p1 * int64_t(N2) * ncols] = v[p1];
@@ -504,18 +714,17 @@ __global__ void __launch_bounds__(256) k_fft_zconv(C<T> *__restrict__ buf, int l
     if (q < N2) {                      // forward pass 1: j2 = q, DFT over j1 (z = j2 + N2 j1 < N_z)
         const int j2 = q;
 #pragma unroll
-        for (int j1 = 0; j1 < N1; ++j1) v[j1] = j1 < H1 ? Sr[j2 + N2 * j1] : mk<T>(T(0), T(0));
-        dft_reg<T, N1, false>(v);
-        const C<T> *t = tf + j2 * N1;
+        for (int j1 = 0; j1 < H1; ++j1) v[j1] = Sr[j2 + N2 * j1];
+        FourStep<T, N1, N2>::fwd1(v, j2, tf);
 #pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) Sr[k1 * N2 + j2] = k1 ? cmul(v[k1], t[k1]) : v[0];
+        for (int k1 = 0; k1 < N1; ++k1) Sr[k1 * N2 + j2] = v[k1];
     }
     __syncthreads();
     const int k1 = q;
     if (q < N1) {                      // forward pass 2, kernel product, inverse pass A (in registers)
 #pragma unroll
         for (int j2 = 0; j2 < N2; ++j2) v[j2] = Sr[k1 * N2 + j2];
-        dft_reg<T, N2, false>(v);      // v[k2] = X[k1 + N1 k2]
+        FourStep<T, N1, N2>::fwd2(v, k1, tf);   // v[k2] = X[k1 + N1 k2]
         const int Mx = 1 << lgMx, My = 1 << lgMy;
         const int64_t row = row0 + r;
         const int ky = int(row & (My - 1)), kx = int((row >> lgMy) & (Mx - 1));
@@ -523,28 +732,19 @@ __global__ void __launch_bounds__(256) k_fft_zconv(C<T> *__restrict__ buf, int l
         const HT *Hr = Hg + (int64_t(fold_index(kx, Mx)) * (My / 2 + 1) + fold_index(ky, My)) * (Mz / 2 + 1);
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) v[k2] = kernel_mul<T>(v[k2], Hr[fold_index(k1 + N1 * k2, Mz)]);
-        dft_reg<T, N2, true>(v);
+        FourStep<T, N1, N2>::inv1(v, k1, ti);
     }
     __syncthreads();                   // every thread has read its pass-2 slots
     if (q < N1) {
-        const C<T> *t = ti + k1 * N2;
 #pragma unroll
-        for (int p2 = 0; p2 < N2; ++p2) {
-            C<T> o = v[p2];
-            if (p2) {
-                const C<T> w = t[p2];
-                o.x = v[p2].x * w.x + v[p2].y * w.y;
-                o.y = v[p2].y * w.x - v[p2].x * w.y;
-            }
-            Sr[p2 * N1 + k1] = o;
-        }
+        for (int p2 = 0; p2 < N2; ++p2) Sr[p2 * N1 + k1] = v[p2];
     }
     __syncthreads();
     const int p2 = q;
     if (q < N2) {                      // inverse pass B: p2 = q, DFT over k1, z = p2 + N2 p1 < N_z
 #pragma unroll
         for (int kk = 0; kk < N1; ++kk) v[kk] = Sr[p2 * N1 + kk];
-        dft_reg<T, N1, true>(v);
+        FourStep<T, N1, N2>::inv2(v, p2, ti);
     }
     __syncthreads();                   // every thread has read its pass-B slots
     if (q < N2) {
@@ -582,16 +782,15 @@ __device__ __forceinline__ void yz_f1(const C<T> *in, C<T> *P, int pitch, int Ny
         const int y = it >> LG2, j2 = it & (N2 - 1);
         const C<T> *src = in + y * Nz + j2;
 #pragma unroll
-        for (int j1 = 0; j1 < N1; ++j1) v[j1] = j1 < H1 ? src[N2 * j1] : mk<T>(T(0), T(0));
-        dft_reg<T, N1, false>(v);
-        const C<T> *t = tfz + j2 * N1;
+        for (int j1 = 0; j1 < H1; ++j1) v[j1] = src[N2 * j1];
+        FourStep<T, N1, N2>::fwd1(v, j2, tfz);
         C<T> *row = P + y * pitch + j2;
 #pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) row[k1 * N2] = k1 ? cmul(v[k1], t[k1]) : v[0];
+        for (int k1 = 0; k1 < N1; ++k1) row[k1 * N2] = v[k1];
     }
 }
 template <typename T, int N1, int N2>   // F2: z pass 2, P row slots -> Q natural rows
-__device__ __forceinline__ void yz_f2(const C<T> *P, C<T> *Q, int pitch, int lgNy) {
+__device__ __forceinline__ void yz_f2(const C<T> *P, C<T> *Q, int pitch, int lgNy, const C<T> *tfz) {
     C<T> v[FFT_NMAX];
     const int Ny = 1 << lgNy;
     for (int it = threadIdx.x; it < Ny * N1; it += blockDim.x) {
@@ -599,7 +798,7 @@ __device__ __forceinline__ void yz_f2(const C<T> *P, C<T> *Q, int pitch, int lgN
         const C<T> *row = P + y * pitch + k1 * N2;
 #pragma unroll
         for (int j2 = 0; j2 < N2; ++j2) v[j2] = row[j2];
-        dft_reg<T, N2, false>(v);
+        FourStep<T, N1, N2>::fwd2(v, k1, tfz);
         C<T> *out = Q + y * pitch + k1;
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) out[N1 * k2] = v[k2];
@@ -614,16 +813,15 @@ __device__ __forceinline__ void yz_f3(const C<T> *Q, C<T> *P, int pitch, int lgM
         const int kz = it & (Mz - 1), j2 = it >> lgMz;
         const C<T> *col = Q + j2 * pitch + kz;
 #pragma unroll
-        for (int j1 = 0; j1 < N1; ++j1) v[j1] = j1 < H1 ? col[N2 * j1 * pitch] : mk<T>(T(0), T(0));
-        dft_reg<T, N1, false>(v);
-        const C<T> *t = tfy + j2 * N1;
+        for (int j1 = 0; j1 < H1; ++j1) v[j1] = col[N2 * j1 * pitch];
+        FourStep<T, N1, N2>::fwd1(v, j2, tfy);
         C<T> *o = P + j2 * pitch + kz;
 #pragma unroll
-        for (int k1 = 0; k1 < N1; ++k1) o[k1 * N2 * pitch] = k1 ? cmul(v[k1], t[k1]) : v[0];
+        for (int k1 = 0; k1 < N1; ++k1) o[k1 * N2 * pitch] = v[k1];
     }
 }
 template <typename T, int N1, int N2>   // I2: y inverse pass B, P -> Q rows y < Ny
-__device__ __forceinline__ void yz_i2(const C<T> *P, C<T> *Q, int pitch, int lgMz) {
+__device__ __forceinline__ void yz_i2(const C<T> *P, C<T> *Q, int pitch, int lgMz, const C<T> *tiy) {
     constexpr int H1 = N1 / 2;
     C<T> v[FFT_NMAX];
     const int Mz = 1 << lgMz;
@@ -632,7 +830,7 @@ __device__ __forceinline__ void yz_i2(const C<T> *P, C<T> *Q, int pitch, int lgM
         const C<T> *src = P + p2 * N1 * pitch + kz;
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) v[k1] = src[k1 * pitch];
-        dft_reg<T, N1, true>(v);
+        FourStep<T, N1, N2>::inv2(v, p2, tiy);
         C<T> *o = Q + p2 * pitch + kz;
 #pragma unroll
         for (int p1 = 0; p1 < H1; ++p1) o[N2 * p1 * pitch] = v[p1];
@@ -650,23 +848,14 @@ __device__ __forceinline__ void yz_i3(const C<T> *Q, C<T> *P, int pitch, int lgN
         const C<T> *src = Q + y * pitch + k1;
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) v[k2] = src[N1 * k2];
-        dft_reg<T, N2, true>(v);
-        const C<T> *t = tiz + k1 * N2;
+        FourStep<T, N1, N2>::inv1(v, k1, tiz);
         C<T> *o = P + y * pitch + k1 * N2;
 #pragma unroll
-        for (int p2 = 0; p2 < N2; ++p2) {
-            C<T> r = v[p2];
-            if (p2) {
-                const C<T> w = t[p2];
-                r.x = v[p2].x * w.x + v[p2].y * w.y;
-                r.y = v[p2].y * w.x - v[p2].x * w.y;
-            }
-            o[p2] = r;
-        }
+        for (int p2 = 0; p2 < N2; ++p2) o[p2] = v[p2];
     }
 }
 template <typename T, int N1, int N2>   // I4: z inverse pass B, P row slots -> global, z < Nz
-__device__ __forceinline__ void yz_i4(const C<T> *P, C<T> *out, int pitch, int Ny) {
+__device__ __forceinline__ void yz_i4(const C<T> *P, C<T> *out, int pitch, int Ny, const C<T> *tiz) {
     constexpr int Mz = N1 * N2, Nz = Mz / 2, H1 = N1 / 2;
     constexpr int LG2 = N2 == 2 ? 1 : N2 == 4 ? 2 : N2 == 8 ? 3 : 4;
     C<T> v[FFT_NMAX];
@@ -675,7 +864,7 @@ __device__ __forceinline__ void yz_i4(const C<T> *P, C<T> *out, int pitch, int N
         const C<T> *src = P + y * pitch + p2;
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) v[k1] = src[k1 * N2];
-        dft_reg<T, N1, true>(v);
+        FourStep<T, N1, N2>::inv2(v, p2, tiz);
         C<T> *o = out + y * Nz + p2;
 #pragma unroll
         for (int p1 = 0; p1 < H1; ++p1) o[N2 * p1] = v[p1];
@@ -693,7 +882,7 @@ template <typename T> __device__ __forceinline__ C<T> hmul(C<T> v, C<T> h) { ret
 
 template <typename T, int N1, int N2, typename HT>
 __device__ __forceinline__ void yz_mid(C<T> *P, int pitch, int lgMz, const HT *__restrict__ Hk,
-                                       const C<T> *__restrict__ tiy) {
+                                       const C<T> *__restrict__ tfy, const C<T> *__restrict__ tiy) {
     constexpr int My = N1 * N2;
     const int Mz = 1 << lgMz, hz = Mz / 2 + 1;
     const int CW = blockDim.x / N1;
@@ -706,19 +895,17 @@ __device__ __forceinline__ void yz_mid(C<T> *P, int pitch, int lgMz, const HT *_
             const C<T> *col = P + k1 * N2 * pitch + kz;
 #pragma unroll
             for (int j2 = 0; j2 < N2; ++j2) v[j2] = col[j2 * pitch];
-            dft_reg<T, N2, false>(v);      // v[k2] = X[ky = k1 + N1 k2]
+            FourStep<T, N1, N2>::fwd2(v, k1, tfy);   // v[k2] = X[ky = k1 + N1 k2]
             const HT *h = Hk + fold_index(kz, Mz);
+            if constexpr (std::is_same<T, double>::value && std::is_same<HT, double>::value) {
+                double hv[N2];
 #pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) v[k2] = hmul<T>(v[k2], h[fold_index(k1 + N1 * k2, My) * hz]);
-            dft_reg<T, N2, true>(v);
-            const C<T> *t = tiy + k1 * N2;
+                for (int k2 = 0; k2 < N2; ++k2) hv[k2] = h[fold_index(k1 + N1 * k2, My) * hz];
+                FourStep<T, N1, N2>::inv1_scaled(v, hv);
+            } else {
 #pragma unroll
-            for (int p2 = 1; p2 < N2; ++p2) {
-                const C<T> w = t[p2];
-                C<T> r;
-                r.x = v[p2].x * w.x + v[p2].y * w.y;   // times conj(w)
-                r.y = v[p2].y * w.x - v[p2].x * w.y;
-                v[p2] = r;
+                for (int k2 = 0; k2 < N2; ++k2) v[k2] = hmul<T>(v[k2], h[fold_index(k1 + N1 * k2, My) * hz]);
+                FourStep<T, N1, N2>::inv1(v, k1, tiy);
             }
         }
         __syncthreads();
@@ -759,16 +946,16 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_fft_yzc(C<T> *__
     const HT *Hk = Hg + int64_t(fold_index(kx, Mx)) * (My / 2 + 1) * (Mz / 2 + 1);
     SIE_SPLIT_DISPATCH(Mz, (yz_f1<T, N1, N2>(plane, P, pitch, Ny, tfz)));
     __syncthreads();
-    SIE_SPLIT_DISPATCH(Mz, (yz_f2<T, N1, N2>(P, Qb, pitch, lgNy)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_f2<T, N1, N2>(P, Qb, pitch, lgNy, tfz)));
     __syncthreads();
     SIE_SPLIT_DISPATCH(My, (yz_f3<T, N1, N2>(Qb, P, pitch, lgMz, tfy)));
     __syncthreads();
-    SIE_SPLIT_DISPATCH(My, (yz_mid<T, N1, N2, HT>(P, pitch, lgMz, Hk, tiy)));
-    SIE_SPLIT_DISPATCH(My, (yz_i2<T, N1, N2>(P, Qb, pitch, lgMz)));
+    SIE_SPLIT_DISPATCH(My, (yz_mid<T, N1, N2, HT>(P, pitch, lgMz, Hk, tfy, tiy)));
+    SIE_SPLIT_DISPATCH(My, (yz_i2<T, N1, N2>(P, Qb, pitch, lgMz, tiy)));
     __syncthreads();
     SIE_SPLIT_DISPATCH(Mz, (yz_i3<T, N1, N2>(Qb, P, pitch, lgNy, tiz)));
     __syncthreads();
-    SIE_SPLIT_DISPATCH(Mz, (yz_i4<T, N1, N2>(P, plane, pitch, Ny)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_i4<T, N1, N2>(P, plane, pitch, Ny, tiz)));
 }
 
 }  // namespace sie

@@ -481,8 +481,8 @@ int set_smem(const void *fn, size_t bytes) {
 // Only the x-padded grid (2 N_g per grid) goes through device memory.
 template <typename T> struct Tables;
 template <> struct Tables<double> {
-    static const double2 *tf(const pfft_plan *p, int a) { return p->d_tf64[a]; }
-    static const double2 *ti(const pfft_plan *p, int a) { return p->d_ti64[a]; }
+    static const double2 *tf(const pfft_plan *p, int a) { return p->d_tw64[a]; }   // roots W_M^m
+    static const double2 *ti(const pfft_plan *p, int a) { return p->d_tw64[a]; }
     static const double *Hp(const pfft_plan *p) { return p->d_Hp64; }
     static const double2 *Hl(const pfft_plan *p) { return p->d_Hl64; }
 };
@@ -574,18 +574,30 @@ int launch_yzc(pfft_plan *p, C<T> *spec, int32_t ngrids, const HT *Hp, cudaStrea
         const int rc = plane_conv_f32(p, spec, ngrids, s, done);
         if (rc || done) return rc;
     }
-    // 512 threads for the FP32 static kernel (64 registers); the complex kernel value needs more
-    constexpr int NT = (sizeof(T) == 4 && sizeof(HT) == sizeof(T)) ? 512 : 256;
     const size_t plane_bytes = size_t(p->My + p->Ny) * (p->Mz + 1) * sizeof(C<T>);
-    int rc = set_smem((const void *)k_fft_yzc<T, NT, HT>, plane_bytes);
-    if (rc) return rc;
-    int lgMx = 0;
+    int lgMx = 0, n1y, n2y, n1z, n2z;
     while ((1 << lgMx) < p->Mx) ++lgMx;
-    k_fft_yzc<T, NT, HT><<<unsigned(ngrids * p->Mx), NT, plane_bytes, s>>>(spec, lgMx, p->My, p->Mz, Hp, Tb::tf(p, 1),
-                                                                        Tb::ti(p, 1), Tb::tf(p, 2), Tb::ti(p, 2),
-                                                                        Htab, gslot);
-    SIE_LAUNCH_CHECK(p);
-    return SIE_OK;
+    split4(p->My, n1y, n2y);
+    split4(p->Mz, n1z, n2z);
+    auto launch = [&](auto nt) -> int {
+        constexpr int NT = decltype(nt)::value;
+        if (int rc = set_smem((const void *)k_fft_yzc<T, NT, HT>, plane_bytes)) return rc;
+        k_fft_yzc<T, NT, HT><<<unsigned(ngrids * p->Mx), NT, plane_bytes, s>>>(
+            spec, lgMx, p->My, p->Mz, Hp, Tb::tf(p, 1), Tb::ti(p, 1), Tb::tf(p, 2), Tb::ti(p, 2), Htab, gslot);
+        SIE_LAUNCH_CHECK(p);
+        return SIE_OK;
+    };
+    if constexpr (sizeof(T) == 4) {
+        // 512 threads for the FP32 static kernel (64 registers); the complex kernel value needs more
+        return launch(std::integral_constant<int, sizeof(HT) == sizeof(T) ? 512 : 256>());
+    } else {
+        // a thread for every short transform of the widest pass, up to 256: planes of
+        // 16 x 16 take 64 threads, so that four times as many share an SM
+        const int items = std::max(p->Mz * n2y, p->Ny * n2z);
+        if (items <= 64) return launch(std::integral_constant<int, 64>());
+        if (items <= 128) return launch(std::integral_constant<int, 128>());
+        return launch(std::integral_constant<int, 256>());
+    }
 }
 
 template <typename T>
