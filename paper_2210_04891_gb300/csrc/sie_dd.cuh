@@ -57,6 +57,23 @@ __device__ __forceinline__ DD dd_from(double d) {
     return DD{hi, __double2float_rn(d - double(hi))};
 }
 
+// The same pair by integer arithmetic: hi is d rounded to nearest even at 24
+// bits, lo the exact remainder (29 bits and a sign) converted with one rounding.
+// FP64 conversions and subtractions run at 1/64 of the integer rate.  Exponents
+// outside the range where every part is a normal FP32 number (zero among them)
+// take dd_from.
+__device__ __forceinline__ DD dd_split(double d) {
+    const long long b = __double_as_longlong(d);
+    const unsigned e = unsigned(b >> 52) & 0x7ffu;
+    if (e - 950u > 198u) return dd_from(d);   // 2^-73 <= |d| < 2^126
+    const unsigned f = unsigned(b >> 29) & 0x7fffffu, rem = unsigned(b) & 0x1fffffffu;
+    const unsigned up = (rem + 0x0fffffffu + (f & 1u)) >> 29;   // above half, or half and odd
+    const unsigned sign = unsigned(b >> 32) & 0x80000000u;
+    const float lo = __int2float_rn(int(rem) - int(up << 29)) * __uint_as_float((e - 948u) << 23);
+    return DD{__uint_as_float((((e - 896u) << 23 | f) + up) | sign),
+              __uint_as_float(__float_as_uint(lo) ^ sign)};
+}
+
 __device__ __forceinline__ float4 cdd(DD re, DD im) { return make_float4(re.hi, re.lo, im.hi, im.lo); }
 __device__ __forceinline__ DD cdd_re(float4 v) { return DD{v.x, v.y}; }
 __device__ __forceinline__ DD cdd_im(float4 v) { return DD{v.z, v.w}; }

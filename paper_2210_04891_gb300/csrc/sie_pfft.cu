@@ -62,16 +62,16 @@ template <> __device__ __forceinline__ double2 ezero<double2>() { return make_do
 template <> __device__ __forceinline__ float4 ezero<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 // conversions: FP64 value -> element; element -> FP64, FP32 or another element type
 __device__ __forceinline__ void eset(double2 &e, double2 v) { e = v; }
-__device__ __forceinline__ void eset(float4 &e, double2 v) { e = cdd(dd_from(v.x), dd_from(v.y)); }
+__device__ __forceinline__ void eset(float4 &e, double2 v) { e = cdd(dd_split(v.x), dd_split(v.y)); }
 __device__ __forceinline__ void eset(double2 &e, float4 v) {
     e = make_double2(double(v.x) + double(v.y), double(v.z) + double(v.w));
 }
 __device__ __forceinline__ void eset(float4 &e, float4 v) { e = v; }
 __device__ __forceinline__ double2 to_c(double2 v, double2) { return v; }
-__device__ __forceinline__ float2 to_c(double2 v, float2) { return make_float2(float(v.x), float(v.y)); }
+__device__ __forceinline__ float2 to_c(double2 v, float2) { return make_float2(dd_split(v.x).hi, dd_split(v.y).hi); }
 __device__ __forceinline__ float2 to_c(float4 e, float2) { return make_float2(e.x + e.y, e.z + e.w); }
 __device__ __forceinline__ cdf to_c(double2 v, cdf) {
-    const DD a = dd_from(v.x), b = dd_from(v.y);
+    const DD a = dd_split(v.x), b = dd_split(v.y);
     return cdf{df(a.hi, a.lo), df(b.hi, b.lo)};
 }
 __device__ __forceinline__ cdf to_c(float4 e, cdf) { return cdf{df(e.x, e.y), df(e.z, e.w)}; }
@@ -83,56 +83,199 @@ __device__ __forceinline__ float4 shfl_up(float4 v, int d) {
     return v;
 }
 
-// Inclusive prefix sum of each row of a [R][n] array of elements, in place.
-// One CTA of 1024 threads per row, 4 items per thread per chunk; the next
-// chunk's loads are issued before the current chunk's block scan.
+// i = q n + r without a 64-bit division where 32 bits hold i (uniform branch)
+__device__ __forceinline__ void divmod(int64_t i, int64_t n, int64_t &q, int64_t &r) {
+    if ((uint64_t(i) | uint64_t(n)) >> 32) {
+        q = i / n;
+        r = i - q * n;
+    } else {
+        const uint32_t a = uint32_t(i) / uint32_t(n);
+        q = a;
+        r = uint32_t(i) - a * uint32_t(n);
+    }
+}
+
+// ---- Prefix sums over the Euler tour, of values that are formed where they are
+// summed (the current the links inject at a slot, Eq. CurT; the voltage step of
+// a slot's twig, Eq. VolT).  A row (right-hand side) is cut into chunks of
+// kTourChunk slots, one CTA of 1024 threads per (row, chunk), 4 slots per
+// thread.  With more than one chunk a first pass (k_tour_part) forms each
+// chunk's sums, and k_tour_sums starts each chunk from the chain of those before
+// it.  The sums are associated as by one CTA walking the row chunk by chunk
+// (per thread, per warp, over the warps, over the chunks), so the result does
+// not depend on the split; what the split buys is R x chunks CTAs instead of R.
+// Bound by latency (a chunk: one code, one value, two block scans of 16-byte
+// elements).  Currents' sums with a kernel that wrote the values and one CTA per row that
+// summed them: 64 us for 3 right-hand sides on 12k triangles (24k slots), 255 us
+// for 128 on 40k (79k slots); here 28 and 220 us.
+struct TourLinks {   // values of A^T: +x of links entering the slot's node, -x of links leaving it
+    const double2 *__restrict__ x;
+    int64_t nl;
+    const int32_t *__restrict__ slot, *__restrict__ nl_ptr, *__restrict__ nl_loop;
+    const int8_t *__restrict__ nl_sign;
+};
+template <typename V> struct TourTwigs {   // values of A: +-voltage of the twig above the slot's node
+    const V *__restrict__ y_br;
+    int64_t ldy;
+    const int32_t *__restrict__ slot;
+};
+// Chunk's scan: v[k] inclusive within the thread, incl inclusive over the warp's
+// threads, warp_tot inclusive over the warps; run the thread's total.
 template <typename E>
-__global__ void __launch_bounds__(1024) k_scan_rows(E *buf, int64_t n) {
-    __shared__ E warp_tot[32];
-    __shared__ E carry_s;
-    E *row = buf + blockIdx.x * n;
-    E carry = ezero<E>();
+__device__ __forceinline__ void chunk_scan(E (&v)[4], E &run, E &incl, E *warp_tot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    E vn[4];
+    run = ezero<E>();
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int64_t i = 4 * int64_t(threadIdx.x) + k;
-        vn[k] = i < n ? row[i] : ezero<E>();
+        run = eadd(run, v[k]);
+        v[k] = run;
     }
-    for (int64_t base = 0; base < n; base += 4 * 1024) {
-        E v[4];
+    incl = run;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = vn[k];
-        const int64_t i0 = base + 4 * int64_t(threadIdx.x);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int64_t i = i0 + 4 * 1024 + k;
-            vn[k] = i < n ? row[i] : ezero<E>();
-        }
-        E run = ezero<E>();
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            run = eadd(run, v[k]);
-            v[k] = run;
-        }
-        E incl = run;   // warp inclusive scan of thread totals
+    for (int d = 1; d < 32; d <<= 1) {
+        E o = shfl_up(incl, d);
+        if (lane >= d) incl = eadd(incl, o);
+    }
+    if (lane == 31) warp_tot[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        E w = warp_tot[lane];
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            E o = shfl_up(incl, d);
-            if (lane >= d) incl = eadd(incl, o);
+            E o = shfl_up(w, d);
+            if (lane >= d) w = eadd(w, o);
         }
-        if (lane == 31) warp_tot[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            E w = warp_tot[lane];
+        warp_tot[lane] = w;
+    }
+    __syncthreads();
+}
+// codes of the thread's four slots from i0 on (padded to whole chunks), and their
+// values: the four loads first, unconditioned by each other, then nodes of
+// several links (few), then signs and conversions
+template <typename S> __device__ __forceinline__ int4 chunk_codes(const S &src, int64_t i0) {
+    return __ldg(reinterpret_cast<const int4 *>(src.slot + i0));
+}
+__device__ __forceinline__ double2 node_links(const TourLinks &s, const double2 *x, int32_t n) {
+    double2 v = make_double2(0.0, 0.0);
+#pragma unroll 8
+    for (int32_t k = s.nl_ptr[n]; k < s.nl_ptr[n + 1]; ++k) {
+        const double2 xv = x[s.nl_loop[k]];
+        v = s.nl_sign[k] > 0 ? cadd(v, xv) : csub(v, xv);
+    }
+    return v;
+}
+template <typename E>
+__device__ __forceinline__ void chunk_load(const TourLinks &s, int64_t r, int4 codes, E (&v)[4]) {
+    const int32_t c[4] = {codes.x, codes.y, codes.z, codes.w};
+    const double2 *x = s.x + r * s.nl;
+    double2 d[4];
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                E o = shfl_up(w, d);
-                if (lane >= d) w = eadd(w, o);
-            }
-            warp_tot[lane] = w;
-        }
+    for (int k = 0; k < 4; ++k) {
+        d[k] = make_double2(0.0, 0.0);
+        if (c[k] != 0 && c[k] < kManyLinks) d[k] = __ldg(x + (abs(c[k]) - 1));
+    }
+    if (max(max(c[0], c[1]), max(c[2], c[3])) >= kManyLinks) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (c[k] >= kManyLinks) d[k] = node_links(s, x, c[k] - kManyLinks);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (c[k] < 0) d[k] = make_double2(-d[k].x, -d[k].y);
+        v[k] = ezero<E>();
+        if (c[k] != 0) eset(v[k], d[k]);
+    }
+}
+template <typename E>
+__device__ __forceinline__ void chunk_load(const TourTwigs<E> &s, int64_t r, int4 codes, E (&v)[4]) {
+    const int32_t c[4] = {codes.x, codes.y, codes.z, codes.w};
+    const E *y = s.y_br + r * s.ldy;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[k] = ezero<E>();
+        if (c[k] != 0) v[k] = __ldg(y + (abs(c[k]) - 1));
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c[k] < 0) v[k] = eneg(v[k]);
+}
+// The three terms the last thread of a chunk adds to its carry, in order: the
+// warps before its own, the threads before it in its warp, its own slots.
+template <typename E, typename S>
+__global__ void __launch_bounds__(1024) k_tour_part(const S src, int32_t nchunk, E *__restrict__ part) {
+    __shared__ E warp_tot[32];
+    const int64_t r = blockIdx.x / nchunk;
+    const int32_t c = blockIdx.x - int32_t(r) * nchunk;
+    E v[4], run, incl;
+    chunk_load(src, r, chunk_codes(src, int64_t(c) * kTourChunk + 4 * int64_t(threadIdx.x)), v);
+    chunk_scan(v, run, incl, warp_tot);
+    if (threadIdx.x == 1023) {
+        E *p = part + (r * nchunk + c) * kTourPart;
+        p[0] = warp_tot[30];
+        p[1] = eadd(incl, eneg(run));
+        p[2] = run;
+    }
+}
+template <typename E, typename S>
+__global__ void __launch_bounds__(1024) k_tour_sums(const S src, int64_t n, int32_t nchunk,
+                                                    const E *__restrict__ part, E *__restrict__ out) {
+    __shared__ E warp_tot[32];
+    __shared__ E carry_s;
+    constexpr int STAGE = 96 * kTourPart;
+    __shared__ E stage[STAGE];
+    const int64_t r = blockIdx.x / nchunk;
+    const int32_t c = blockIdx.x - int32_t(r) * nchunk;
+    const int64_t i0 = int64_t(c) * kTourChunk + 4 * int64_t(threadIdx.x);
+    E v[4], run, incl;
+    chunk_load(src, r, chunk_codes(src, i0), v);
+    // carry: the chain over the chunks before this one, by one thread from shared memory
+    if (threadIdx.x == 0) carry_s = ezero<E>();
+    for (int32_t b = 0; b < c * kTourPart; b += STAGE) {
+        const int m = min(STAGE, c * kTourPart - b);
         __syncthreads();
+        for (int i = threadIdx.x; i < m; i += 1024) stage[i] = part[r * nchunk * kTourPart + b + i];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            E s = carry_s;
+            for (int i = 0; i < m; ++i) s = eadd(s, stage[i]);
+            carry_s = s;
+        }
+    }
+    chunk_scan(v, run, incl, warp_tot);   // its barriers also publish carry_s
+    E off = carry_s;
+    const int warp = threadIdx.x >> 5;
+    if (warp > 0) off = eadd(off, warp_tot[warp - 1]);
+    off = eadd(off, eadd(incl, eneg(run)));   // exclusive within the warp
+    E *row = out + r * n;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (i0 + k < n) row[i0 + k] = eadd(v[k], off);
+}
+
+// The same sums by one CTA per row, chunk by chunk: with a row for every SM the
+// split only reads the values twice.  The next chunk's values and the codes of
+// the one after are in flight during the block scan.
+template <typename E, typename S>
+__global__ void __launch_bounds__(1024) k_tour_rows(const S src, int64_t n, E *__restrict__ out) {
+    __shared__ E warp_tot[32];
+    __shared__ E carry_s;
+    const int64_t r = blockIdx.x, np = (n + kTourChunk - 1) / kTourChunk * kTourChunk;
+    const int warp = threadIdx.x >> 5;
+    E *row = out + r * n;
+    E carry = ezero<E>();
+    int64_t i0 = 4 * int64_t(threadIdx.x);
+    E vn[4];
+    chunk_load(src, r, chunk_codes(src, i0), vn);
+    int4 codes = make_int4(0, 0, 0, 0);
+    if (i0 + kTourChunk < np) codes = chunk_codes(src, i0 + kTourChunk);
+    for (; i0 < np; i0 += kTourChunk) {
+        E v[4], run, incl;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = vn[k];
+        chunk_load(src, r, codes, vn);
+        codes = make_int4(0, 0, 0, 0);
+        if (i0 + 2 * kTourChunk < np) codes = chunk_codes(src, i0 + 2 * kTourChunk);
+        chunk_scan(v, run, incl, warp_tot);
         E off = carry;
         if (warp > 0) off = eadd(off, warp_tot[warp - 1]);
         off = eadd(off, eadd(incl, eneg(run)));   // exclusive within the warp
@@ -142,79 +285,25 @@ __global__ void __launch_bounds__(1024) k_scan_rows(E *buf, int64_t n) {
         if (threadIdx.x == 1023) carry_s = eadd(off, run);
         __syncthreads();
         carry = carry_s;
-        __syncthreads();
     }
 }
 
-// Tour values for A^T: at node v's enter slot the current the links inject
-// into v (+x on links entering v, -x on links leaving it); 0 at exit slots.
-// Grid (slots, right-hand-side groups): a thread takes one slot and kTourRc
-// right-hand sides, so the slot's index chain (node, link list, loops) is read
-// once for the group and the group's loads of x are independent.
-constexpr int kTourRc = 8;
-template <typename E>
-__global__ void k_tour_inject(const double2 *__restrict__ x, int64_t nl, E *__restrict__ tour, int64_t nslots,
-                              const int32_t *__restrict__ tour_node, const int8_t *__restrict__ tour_enter,
-                              const int32_t *__restrict__ nl_ptr, const int32_t *__restrict__ nl_loop,
-                              const int8_t *__restrict__ nl_sign, int32_t nrhs) {
-    const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (s >= nslots) return;
-    const int32_t r0 = int32_t(blockIdx.y) * kTourRc;
-    const int nr = min(kTourRc, nrhs - r0);
-    const int v = tour_node[s];
-    int32_t k0 = 0, k1 = 0;
-    if (tour_enter[s]) {
-        k0 = nl_ptr[v];
-        k1 = nl_ptr[v + 1];
-    }
-    if (k1 <= k0) {   // no link at this slot (most slots): zeros, no FP64 work
-#pragma unroll
-        for (int j = 0; j < kTourRc; ++j)
-            if (j < nr) tour[int64_t(r0 + j) * nslots + s] = ezero<E>();
-        return;
-    }
-    double2 acc[kTourRc];   // a few link currents, exact inputs
-#pragma unroll
-    for (int j = 0; j < kTourRc; ++j) acc[j] = make_double2(0.0, 0.0);
-    for (int32_t k = k0; k < k1; ++k) {
-        const double2 *xl = x + int64_t(r0) * nl + nl_loop[k];
-        const bool pos = nl_sign[k] > 0;
-#pragma unroll
-        for (int j = 0; j < kTourRc; ++j)
-            if (j < nr) {
-                const double2 xv = xl[int64_t(j) * nl];
-                acc[j] = pos ? cadd(acc[j], xv) : csub(acc[j], xv);
-            }
-    }
-    // the conversion to the tour's element (double-float pairs in the mixed
-    // form) runs on the FP64 pipe: only here, on the slots that carry links
-#pragma unroll
-    for (int j = 0; j < kTourRc; ++j)
-        if (j < nr) {
-            E out;
-            eset(out, acc[j]);
-            tour[int64_t(r0 + j) * nslots + s] = out;
-        }
-}
-
-// Branch current of branch b for right-hand side r (loop space): a link carries
-// its loop current; a twig above node v carries -sigma * (subtree inflow), a
-// difference of two prefix sums taken in the tour's arithmetic.
+// Branch current (loop space) from its record: a link carries its loop current;
+// a twig above node v carries -sigma * (subtree inflow), a difference of two
+// prefix sums taken in the tour's arithmetic.
 template <typename T, typename E>
-__device__ __forceinline__ C<T> branch_current(int32_t b, int64_t r, const double2 *__restrict__ x, int64_t nl,
-                                               const E *__restrict__ P, int64_t nslots,
-                                               const int32_t *__restrict__ loop_of_branch,
-                                               const int32_t *__restrict__ twig_node, const int32_t *__restrict__ head,
-                                               const int32_t *__restrict__ enter, const int32_t *__restrict__ exit_) {
-    int32_t l = loop_of_branch[b];
-    if (l >= 0) return to_c(x[r * nl + l], C<T>{});
-    int32_t v = twig_node[b];
-    const E *row = P + r * nslots;
-    E S = row[exit_[v]];
-    int32_t e = enter[v];
-    if (e > 0) S = eadd(S, eneg(row[e - 1]));
-    const C<T> d = to_c(S, C<T>{});
-    return head[b] == v ? mk<T>(-d.x, -d.y) : d;
+__device__ __forceinline__ C<T> branch_current(int4 s, int64_t r, const double2 *__restrict__ x, int64_t nl,
+                                               const E *__restrict__ P, int64_t nslots) {
+    C<T> d;
+    if (s.x >= 0) {
+        d = to_c(x[r * nl + s.x], C<T>{});
+    } else {
+        const E *row = P + r * nslots;
+        E S = row[s.y];
+        if (s.z >= 0) S = eadd(S, eneg(row[s.z]));
+        d = to_c(S, C<T>{});
+    }
+    return s.w < 0 ? mk<T>(-d.x, -d.y) : d;
 }
 
 // Local currents c_T[k] = s_k alpha_{b(T,k)}: one thread per (T, r) for the
@@ -222,29 +311,32 @@ __device__ __forceinline__ C<T> branch_current(int32_t b, int64_t r, const doubl
 // with SMALL (FP32) as float4 [T][2R] (components innermost, re and im columns).
 template <typename T, bool SMALL>
 __global__ void k_alpha_tri(const double2 *__restrict__ x, int64_t nl, const TourE<T> *__restrict__ P, int64_t nslots,
-                            const int32_t *__restrict__ tb, const int8_t *__restrict__ ts,
-                            const int32_t *__restrict__ loop_of_branch, const int32_t *__restrict__ twig_node,
-                            const int32_t *__restrict__ head, const int32_t *__restrict__ enter,
-                            const int32_t *__restrict__ exit_, int64_t nt, int32_t nrhs, int space, int64_t nb,
+                            const int4 *__restrict__ tri_src, const int32_t *__restrict__ tb,
+                            const int8_t *__restrict__ ts, int64_t nt, int32_t nrhs, int space, int64_t nb,
                             C<T> *__restrict__ cT) {
     int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= nt * nrhs) return;
-    const int64_t t = i / nrhs, r = i % nrhs;
+    int64_t t, r;
+    divmod(i, nrhs, t, r);
     C<T> c[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const int64_t tk = t * 3 + k;
-        const int32_t b = tb[tk];
-        C<T> a = mk<T>(T(0), T(0));
-        if (b >= 0) {
-            if (space == SIE_SPACE_LOOP)
-                a = branch_current<T>(b, r, x, nl, P, nslots, loop_of_branch, twig_node, head, enter, exit_);
-            else
-                a = to_c(x[r * nb + b], C<T>{});
-            if (ts[tk] < 0) { a.x = -a.x; a.y = -a.y; }
+        c[k] = mk<T>(T(0), T(0));
+        if (space == SIE_SPACE_LOOP) {
+            const int4 s = __ldg(tri_src + tk);
+            if (s.w) c[k] = branch_current<T>(s, r, x, nl, P, nslots);
+        } else {
+            const int32_t b = tb[tk];
+            if (b >= 0) {
+                c[k] = to_c(x[r * nb + b], C<T>{});
+                if (ts[tk] < 0) { c[k].x = -c[k].x; c[k].y = -c[k].y; }
+            }
         }
-        if constexpr (SMALL) c[k] = a;
-        else cT[tk * nrhs + r] = a;
+    }
+    if constexpr (!SMALL) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) cT[(t * 3 + k) * nrhs + r] = c[k];
     }
     if constexpr (SMALL) {
         static_assert(is_f32<T>, "component-inner currents in FP32 only");
@@ -1075,7 +1167,8 @@ __global__ void k_branch_out(const E *__restrict__ y_tri, const int32_t *__restr
                              EO *__restrict__ y) {
     int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= ldy * nrhs) return;
-    int64_t r = i / ldy, b = i % ldy;
+    int64_t r, b;
+    divmod(i, ldy, r, b);
     E v = ezero<E>();
     if (b < nb) {
         const E a = y_tri[(r * nt + br_tri[2 * b]) * 3 + br_local[2 * b]];
@@ -1087,45 +1180,19 @@ __global__ void k_branch_out(const E *__restrict__ y_tri, const int32_t *__restr
     y[i] = o;
 }
 
-// Tour values for A: +delta(v) at v's enter slot, -delta(v) at its exit slot,
-// delta(v) = voltage of v's parent twig walked from v towards the root.
-// Grid (slots, right-hand-side groups of kTourRc), as k_tour_inject.
-template <typename E>
-__global__ void k_tour_voltage(const E *__restrict__ y_br, int64_t ldy, E *__restrict__ tour, int64_t nslots,
-                               const int32_t *__restrict__ tour_node, const int8_t *__restrict__ tour_enter,
-                               const int32_t *__restrict__ parent_branch, const int32_t *__restrict__ tail,
-                               int32_t nrhs) {
-    const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (s >= nslots) return;
-    const int32_t r0 = int32_t(blockIdx.y) * kTourRc;
-    const int nr = min(kTourRc, nrhs - r0);
-    const int v = tour_node[s];
-    const int t = parent_branch[v];
-    const bool neg = t >= 0 && ((tail[t] != v) != !tour_enter[s]);
-    E d[kTourRc];
-#pragma unroll
-    for (int j = 0; j < kTourRc; ++j) {
-        d[j] = ezero<E>();
-        if (t >= 0 && j < nr) d[j] = y_br[int64_t(r0 + j) * ldy + t];
-    }
-#pragma unroll
-    for (int j = 0; j < kTourRc; ++j)
-        if (j < nr) tour[int64_t(r0 + j) * nslots + s] = neg ? eneg(d[j]) : d[j];
-}
-
+// Loop voltage: its link's plus psi(head) - psi(tail), psi the prefix sums P.
 template <typename E>
 __global__ void k_loop_out(const E *__restrict__ y_br, int64_t ldy, const E *__restrict__ P, int64_t nslots,
-                           const int32_t *__restrict__ link_branch, const int32_t *__restrict__ tail,
-                           const int32_t *__restrict__ head, const int32_t *__restrict__ enter, int64_t nl,
-                           int32_t nrhs, double2 *__restrict__ y) {
+                           const int4 *__restrict__ loop_dst, int64_t nl, int32_t nrhs, double2 *__restrict__ y) {
     int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= nl * nrhs) return;
-    int64_t r = i / nl, l = i % nl;
-    int32_t e = link_branch[l];
+    int64_t r, l;
+    divmod(i, nl, r, l);
+    const int4 d = __ldg(loop_dst + l);
     const E *row = P + r * nslots;
-    E v = y_br[r * ldy + e];
-    v = eadd(v, row[enter[head[e]]]);
-    v = eadd(v, eneg(row[enter[tail[e]]]));
+    E v = y_br[r * ldy + d.x];
+    v = eadd(v, row[d.y]);
+    v = eadd(v, eneg(row[d.z]));
     double2 o;
     eset(o, v);
     y[i] = o;
@@ -1133,15 +1200,12 @@ __global__ void k_loop_out(const E *__restrict__ y_br, int64_t ldy, const E *__r
 
 // Post-processing (Eq. CurT): current of every mesh branch, grid (branches, right-hand sides).
 __global__ void k_branch_alpha(const double2 *__restrict__ x, int64_t nl, const double2 *__restrict__ P,
-                               int64_t nslots, const int32_t *__restrict__ loop_of_branch,
-                               const int32_t *__restrict__ twig_node, const int32_t *__restrict__ head,
-                               const int32_t *__restrict__ enter, const int32_t *__restrict__ exit_, int64_t nb,
+                               int64_t nslots, const int4 *__restrict__ branch_src, int64_t nb,
                                double2 *__restrict__ alpha) {
     const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (b >= nb) return;
     const int64_t r = blockIdx.y;
-    alpha[r * nb + b] = branch_current<double>(int32_t(b), r, x, nl, P, nslots, loop_of_branch, twig_node, head,
-                                               enter, exit_);
+    alpha[r * nb + b] = branch_current<double>(branch_src[b], r, x, nl, P, nslots);
 }
 
 // Post-processing: panel potential = root-path sum of the panel's node minus that
@@ -1175,10 +1239,10 @@ int scratch_reserve(pfft_plan *p, int32_t nrhs, int prec) {
     const int64_t R = std::max<int64_t>({int64_t(nrhs), int64_t(s.cap_rhs), 1});
     const size_t cs = size_t(std::max(want_cs, s.cs));
     const bool with_far = mixed || s.ffar != nullptr;
-    for (void *a : {s.tour, s.grid, s.spec, s.phiT, s.y_tri, s.y_br, (void *)s.coef, s.cT, s.ffar})
+    for (void *a : {s.tour, s.part, s.grid, s.spec, s.phiT, s.y_tri, s.y_br, (void *)s.coef, s.cT, s.ffar})
         if (a) cudaFree(a);
     s = Scratch{};
-    constexpr int kBufs = 9;
+    constexpr int kBufs = 10;
     // bytes per row of the right-hand-sides-inner operands, and of the float4
     // columns that few right-hand sides use instead
     const size_t row = std::max(size_t(R) * 3 * cs, size_t(std::min<int64_t>(R, kSmallRhs)) * 2 * sizeof(float4));
@@ -1191,9 +1255,10 @@ int scratch_reserve(pfft_plan *p, int32_t nrhs, int prec) {
         size_t(R) * (p->nb + p->np) * sizeof(double2),
         size_t(R) * (2 * p->ncond + 1) * (sizeof(double) + sizeof(float2)),
         row * p->nt,
-        with_far ? size_t(R) * p->nt * 3 * sizeof(float2) : 0};
+        with_far ? size_t(R) * p->nt * 3 * sizeof(float2) : 0,
+        size_t(R) * ((2 * p->nn + kTourChunk - 1) / kTourChunk) * kTourPart * sizeof(double2)};
     void **dst[kBufs] = {&s.tour, &s.grid, &s.spec, &s.phiT, &s.y_tri, &s.y_br, (void **)&s.coef, &s.cT,
-                         &s.ffar};
+                         &s.ffar, &s.part};
     for (int i = 0; i < kBufs; ++i) {
         if (!sizes[i]) continue;
         cudaError_t e = cudaMalloc(dst[i], sizes[i]);
@@ -1414,6 +1479,31 @@ template <typename T> int run_tri_gather_lossy(pfft_plan *p, int32_t R, cudaStre
     return Blocks<T, 1, 4>::tri_gather_lossy(p, R, st);
 }
 
+// from this many rows on one CTA per row (wires, 79k slots: 128 rows 220 us for the
+// currents' sums against 343 split, 64 rows 208 against 190 split)
+constexpr int32_t kTourRowsMin = 96;
+// Prefix sums of src's values over the tour, for R right-hand sides, into tour [R][2 nn].
+template <typename E, typename S> int tour_sums(pfft_plan *p, const S &src, E *tour, int32_t R, cudaStream_t st) {
+    const int64_t n = 2 * p->nn, nchunk = (n + kTourChunk - 1) / kTourChunk;
+    if (R * nchunk > INT32_MAX) return fail(SIE_ERR_ARG, "tour sums: too many right-hand sides");
+    E *part = (E *)p->scr.part;
+    if (nchunk > 1 && R >= kTourRowsMin) {
+        k_tour_rows<E><<<unsigned(R), 1024, 0, st>>>(src, n, tour);
+        SIE_LAUNCH_CHECK(p);
+        return SIE_OK;
+    }
+    if (nchunk > 1) {
+        k_tour_part<E><<<unsigned(R * nchunk), 1024, 0, st>>>(src, int32_t(nchunk), part);
+        SIE_LAUNCH_CHECK(p);
+    }
+    k_tour_sums<E><<<unsigned(R * nchunk), 1024, 0, st>>>(src, n, int32_t(nchunk), part, tour);
+    SIE_LAUNCH_CHECK(p);
+    return SIE_OK;
+}
+TourLinks tour_links(const pfft_plan *p, const double2 *x) {
+    return TourLinks{x, p->nl, p->d_slot_link, p->d_nl_ptr, p->d_nl_loop, p->d_nl_sign};
+}
+
 // Smallest right-hand-side count for the tensor-core near field (mixed form).
 constexpr int32_t kNearMmaMinRhs = 96;
 
@@ -1425,24 +1515,21 @@ int matvec_t(pfft_plan *p, const double2 *x, double2 *y, int32_t R, int space, c
     using E = TourE<T>;
     E *tour = (E *)s.tour;
     E *y_tri = (E *)s.y_tri, *y_br = (E *)s.y_br;
+    int rc = SIE_OK;
     std::unique_ptr<StageTimer> tm(new StageTimer(p, SIE_STAGE_LOOP_TO_BRANCH, st));
     if (space == SIE_SPACE_LOOP) {
-        k_tour_inject<<<dim3(nblk(nslots), unsigned((R + kTourRc - 1) / kTourRc)), 256, 0, st>>>(
-            x, p->nl, tour, nslots, p->d_tour_node, p->d_tour_enter, p->d_nl_ptr, p->d_nl_loop, p->d_nl_sign, R);
-        SIE_LAUNCH_CHECK(p);
-        k_scan_rows<E><<<R, 1024, 0, st>>>(tour, nslots);
-        SIE_LAUNCH_CHECK(p);
+        rc = tour_sums<E>(p, tour_links(p, x), tour, R, st);
+        if (rc) return rc;
     }
     const bool small = is_f32<T> && small_rhs(p, R);
     auto alpha = k_alpha_tri<T, false>;
     if constexpr (is_f32<T>)
         if (small) alpha = k_alpha_tri<T, true>;
-    alpha<<<nblk(p->nt * R), 256, 0, st>>>(x, p->nl, tour, nslots, p->d_tb, p->d_ts, p->d_loop_of_branch,
-                                           p->d_twig_node, p->d_head, p->d_enter, p->d_exit, p->nt, R, space, p->nb,
-                                           (C<T> *)s.cT);
+    alpha<<<nblk(p->nt * R), 256, 0, st>>>(x, p->nl, tour, nslots, p->d_tri_src, p->d_tb, p->d_ts, p->nt, R, space,
+                                           p->nb, (C<T> *)s.cT);
     SIE_LAUNCH_CHECK(p);
     tm.reset(new StageTimer(p, SIE_STAGE_PROJECT, st));
-    int rc = small ? project_small(p, R, st) : run_project<T>(p, R, st);
+    rc = small ? project_small(p, R, st) : run_project<T>(p, R, st);
     if (rc) return rc;
     tm.reset();
     const int prec = is_df<T> ? SIE_PREC_DF : is_f64<T> ? SIE_PREC_FP64 : SIE_PREC_MIXED;
@@ -1495,13 +1582,9 @@ int matvec_t(pfft_plan *p, const double2 *x, double2 *y, int32_t R, int space, c
     k_branch_out<E, E><<<nblk(ldy * R), 256, 0, st>>>(y_tri, p->d_br_tri, p->d_br_local, p->nt, p->nb, ldy, R,
                                                         y_br);
     SIE_LAUNCH_CHECK(p);
-    k_tour_voltage<E><<<dim3(nblk(nslots), unsigned((R + kTourRc - 1) / kTourRc)), 256, 0, st>>>(
-        y_br, ldy, tour, nslots, p->d_tour_node, p->d_tour_enter, p->d_parent_branch, p->d_tail, R);
-    SIE_LAUNCH_CHECK(p);
-    k_scan_rows<E><<<R, 1024, 0, st>>>(tour, nslots);
-    SIE_LAUNCH_CHECK(p);
-    k_loop_out<E><<<nblk(p->nl * R), 256, 0, st>>>(y_br, ldy, tour, nslots, p->d_link_branch, p->d_tail, p->d_head,
-                                                    p->d_enter, p->nl, R, y);
+    rc = tour_sums<E>(p, TourTwigs<E>{y_br, ldy, p->d_slot_twig}, tour, R, st);
+    if (rc) return rc;
+    k_loop_out<E><<<nblk(p->nl * R), 256, 0, st>>>(y_br, ldy, tour, nslots, p->d_loop_dst, p->nl, R, y);
     SIE_LAUNCH_CHECK(p);
     return SIE_OK;
 }
@@ -1637,27 +1720,24 @@ extern "C" int sie_postprocess(pfft_plan *p, const void *x, int32_t nrhs, const 
         vb = tmp_v;
     }
     double2 *tour = static_cast<double2 *>(p->scr.tour);
-    const dim3 gs(nblk(nslots), unsigned((R + kTourRc - 1) / kTourRc)), gb(nblk(nb), unsigned(R)),
-        gt(nblk(nt), unsigned(R));
+    const dim3 gb(nblk(nb), unsigned(R)), gt(nblk(nt), unsigned(R));
     // branch currents: alpha = A^T x through the tour prefix sums (FP64)
-    k_tour_inject<double2><<<gs, 256, 0, st>>>(static_cast<const double2 *>(x), p->nl, tour, nslots, p->d_tour_node,
-                                               p->d_tour_enter, p->d_nl_ptr, p->d_nl_loop, p->d_nl_sign, R);
-    k_scan_rows<double2><<<unsigned(R), 1024, 0, st>>>(tour, nslots);
-    k_branch_alpha<<<gb, 256, 0, st>>>(static_cast<const double2 *>(x), p->nl, tour, nslots, p->d_loop_of_branch,
-                                       p->d_twig_node, p->d_head, p->d_enter, p->d_exit, nb, alpha);
-    p->launches += 3;
+    rc = tour_sums<double2>(p, tour_links(p, static_cast<const double2 *>(x)), tour, nrhs, st);
+    if (rc) { cleanup(); return rc; }
+    k_branch_alpha<<<gb, 256, 0, st>>>(static_cast<const double2 *>(x), p->nl, tour, nslots, p->d_branch_src, nb,
+                                       alpha);
+    p->launches += 1;
     if (cudaGetLastError() != cudaSuccess) { cleanup(); return fail(SIE_ERR_CUDA, "sie_postprocess: launch failed"); }
     if (vb) {   // branch voltage drops: the branch-space product Z_b alpha
         rc = matvec_async(p, alpha, vb, nrhs, omega, SIE_SPACE_BRANCH, prec, st);
         if (rc) { cleanup(); return rc; }
     }
     if (phi) {   // potentials: root-path sums of the twig drops, minus the reference node's
-        k_tour_voltage<double2><<<gs, 256, 0, st>>>(vb, nb, tour, nslots, p->d_tour_node, p->d_tour_enter,
-                                                     p->d_parent_branch, p->d_tail, R);
-        k_scan_rows<double2><<<unsigned(R), 1024, 0, st>>>(tour, nslots);
+        rc = tour_sums<double2>(p, TourTwigs<double2>{vb, nb, p->d_slot_twig}, tour, nrhs, st);
+        if (rc) { cleanup(); return rc; }
         k_panel_phi<<<gt, 256, 0, st>>>(tour, nslots, p->d_panel_slot, p->d_panel_ref, nt,
                                         static_cast<double2 *>(phi));
-        p->launches += 3;
+        p->launches += 1;
         if (cudaGetLastError() != cudaSuccess) { cleanup(); return fail(SIE_ERR_CUDA, "sie_postprocess: launch failed"); }
     }
     const cudaError_t e = cudaStreamSynchronize(st);

@@ -1018,20 +1018,25 @@ extern "C" int pfft_plan_create(const sie_mesh *m, const sie_loops *L, const pff
     UP(p->d_near_ptr, near_ptr);
     UP(p->d_near_col, near_col);
     {
-        std::vector<int32_t> tn(L->tour_node.begin(), L->tour_node.end());
-        UP(p->d_tour_node, tn);
-        std::vector<int8_t> te(L->tour_is_enter.begin(), L->tour_is_enter.end());
-        UP(p->d_tour_enter, te);
-        std::vector<int32_t> en(L->enter.begin(), L->enter.end()), ex(L->exit_.begin(), L->exit_.end());
-        UP(p->d_enter, en);
-        UP(p->d_exit, ex);
         std::vector<int32_t> np_(L->nl_ptr.begin(), L->nl_ptr.end()), nlo(L->nl_loop.begin(), L->nl_loop.end());
         std::vector<int8_t> nls(L->nl_sign.begin(), L->nl_sign.end());
         UP(p->d_nl_ptr, np_);
         UP(p->d_nl_loop, nlo);
         UP(p->d_nl_sign, nls);
-        std::vector<int32_t> pb(L->parent_branch.begin(), L->parent_branch.end());
-        UP(p->d_parent_branch, pb);
+        const int64_t slots = (2 * p->nn + kTourChunk - 1) / kTourChunk * kTourChunk;   // whole chunks, zeros at the end
+        std::vector<int32_t> slot_link(slots, 0), slot_twig(slots, 0);
+        for (int64_t i = 0; i < 2 * p->nn; ++i) {
+            const int32_t v = L->tour_node[i];
+            const bool ent = L->tour_is_enter[i] != 0;
+            const int32_t k0 = L->nl_ptr[v], n = L->nl_ptr[v + 1] - k0;
+            if (ent && n == 1) slot_link[i] = L->nl_sign[k0] > 0 ? L->nl_loop[k0] + 1 : -(L->nl_loop[k0] + 1);
+            else if (ent && n > 1) slot_link[i] = kManyLinks + v;
+            // parent twig walked from v towards the root, added at the enter slot, taken off at the exit slot
+            const int32_t t = L->parent_branch[v];
+            if (t >= 0) slot_twig[i] = ((L->tail[t] != v) != !ent) ? -(t + 1) : t + 1;
+        }
+        UP(p->d_slot_link, slot_link);
+        UP(p->d_slot_twig, slot_twig);
         // reference node of each part: the sink contact of its first port, else its tree root
         std::vector<int64_t> ref(L->n_comp, -1);
         for (size_t q = 0; q < L->port_sink.size(); ++q) {
@@ -1048,7 +1053,24 @@ extern "C" int pfft_plan_create(const sie_mesh *m, const sie_loops *L, const pff
         }
         UP(p->d_panel_slot, ps);
         UP(p->d_panel_ref, pr);
-        UP(p->d_twig_node, twig_node);
+        std::vector<int4> branch_src(L->nb), tri_src(3 * nt, make_int4(-1, 0, -1, 0)), loop_dst(L->nl);
+        for (int64_t e = 0; e < L->nb; ++e) {
+            const int32_t l = L->loop_of_branch[e], v = twig_node[e];
+            branch_src[e] = l >= 0 ? make_int4(l, 0, -1, 1)
+                                   : make_int4(-1, L->exit_[v], L->enter[v] - 1, L->head[e] == v ? -1 : 1);
+        }
+        for (int64_t i = 0; i < 3 * nt; ++i)
+            if (tb[i] >= 0) {
+                tri_src[i] = branch_src[tb[i]];
+                tri_src[i].w *= ts[i] < 0 ? -1 : 1;
+            }
+        for (int64_t l = 0; l < L->nl; ++l) {
+            const int32_t e = L->link_branch[l];
+            loop_dst[l] = make_int4(e, L->enter[L->head[e]], L->enter[L->tail[e]], 0);
+        }
+        UP(p->d_branch_src, branch_src);
+        UP(p->d_tri_src, tri_src);
+        UP(p->d_loop_dst, loop_dst);
         std::vector<int32_t> lob(L->loop_of_branch.begin(), L->loop_of_branch.end());
         UP(p->d_loop_of_branch, lob);
         std::vector<int32_t> ta(L->tail.begin(), L->tail.end()), he(L->head.begin(), L->head.end());
@@ -1188,7 +1210,7 @@ extern "C" void pfft_plan_destroy(pfft_plan *p) {
         cudaDeviceSynchronize();   // stream-ordered frees of the solve path have completed
         cudaMemPoolDestroy(p->pool);
     }
-    for (void *a : {p->scr.tour, p->scr.grid, p->scr.spec, p->scr.phiT, p->scr.y_tri, p->scr.y_br,
+    for (void *a : {p->scr.tour, p->scr.part, p->scr.grid, p->scr.spec, p->scr.phiT, p->scr.y_tri, p->scr.y_br,
                     (void *)p->scr.coef, p->scr.cT, p->scr.ffar})
         if (a) cudaFree(a);
     delete p;

@@ -24,6 +24,11 @@ constexpr int kChunkRhs = 32;
 // a warp).  Their dense operands are float4 [row][2R], the three components of
 // a real column side by side, so that a lane reads its operand in one load.
 constexpr int kSmallRhs = 16;
+// slot_link code of a node with several links (codes of single links are below it)
+constexpr int32_t kManyLinks = 1 << 30;
+// Tour slots of one CTA of the prefix sums, and values a CTA leaves for the
+// chunks after it (k_tour_part).
+constexpr int kTourChunk = 4096, kTourPart = 3;
 
 struct PrecondState;   // sie_solve.cu
 struct LossyCache;     // sie_lossy.cu
@@ -35,6 +40,7 @@ struct Scratch {
     // tour, y_tri and y_br hold complex128 in the FP64 form and double-float
     // complex (float4: re hi, re lo, im hi, im lo) in the mixed form
     void *tour = nullptr;      // [R][2 n_nodes]
+    void *part = nullptr;      // [R][chunks][kTourPart], same elements: sums of the tour's chunks
     void *grid = nullptr;      // complex T [3][R][Ng]   grid currents, then grid potentials
     void *spec = nullptr;      // complex T [3R][Mx][Ny][Nz]  grids transformed along x, then (large
                                // planes) [3R][Mx][My][Nz] the same transformed along y
@@ -156,14 +162,19 @@ struct pfft_plan {
     sie::LossyCache *lossy = nullptr;
     double *d_verts = nullptr;          // [nt][3][3] vertices
     double *d_r7b = nullptr, *d_r7w = nullptr;   // Radon 7-point rule (barycentric [7][3], weights [7])
-    // loop basis on the device
-    int32_t *d_tour_node = nullptr;     // [2 nn]
-    int8_t *d_tour_enter = nullptr;     // [2 nn]
-    int32_t *d_enter = nullptr, *d_exit = nullptr;   // [nn]
+    // loop basis on the device.  What a thread of the loop/branch maps needs is
+    // one record (one dependent load before the data), not a chain of maps:
+    //   slot_link [2 nn, to a whole chunk]: current the links inject at a tour slot: 0 none, +-(l + 1) one
+    //     link (+ enters the node), kManyLinks + v the links nl_ptr[v] .. nl_ptr[v + 1];
+    //   slot_twig (same): +-(b + 1), the twig whose voltage step the slot adds (0: none);
+    //   branch_src [nb]: branch current: x loop >= 0 (a link), else sums P[y] - P[z]
+    //     (z < 0: P[y]) over the tour, times w;  tri_src [nt][3]: the same per local edge
+    //     with the edge's sign (w = 0: no branch);
+    //   loop_dst [nl]: link branch, tour slots of its head and tail.
+    int32_t *d_slot_link = nullptr, *d_slot_twig = nullptr;
+    int4 *d_branch_src = nullptr, *d_tri_src = nullptr, *d_loop_dst = nullptr;
     int32_t *d_nl_ptr = nullptr, *d_nl_loop = nullptr;
     int8_t *d_nl_sign = nullptr;
-    int32_t *d_parent_branch = nullptr;  // [nn]
-    int32_t *d_twig_node = nullptr;      // [nb]: node whose parent branch it is, -1 for links
     // post-processing: tour slot of each panel's node and of its conductor's reference node
     int32_t *d_panel_slot = nullptr, *d_panel_ref = nullptr;   // [nt]
     int32_t *d_loop_of_branch = nullptr; // [nb + np]
