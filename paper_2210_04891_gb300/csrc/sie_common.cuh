@@ -89,13 +89,10 @@ template <typename V> __device__ __forceinline__ V mul_mi(V a, bool inv) {
 // One 3x3 real block of a block-sparse matrix with its column index, packed so
 // a warp reads it with a few uniform 16-byte loads: out[a] += sum_b b[3a+b] x[b].
 template <typename T> struct Rec;
-// FP32: three rows {b[3a], b[3a+1], b[3a+2], col}, so that a lane that owns one
-// output component reads its three coefficients and the column in one load.
 template <> struct alignas(16) Rec<float> {
-    struct {
-        float b[3];
-        int32_t col;
-    } row[3];
+    float b[9];
+    int32_t col;
+    float pad[2];
 };
 template <> struct alignas(16) Rec<double> {
     double b[9];
@@ -113,10 +110,10 @@ template <typename T> __device__ __forceinline__ int64_t load_rec(const Rec<T> *
 template <> __device__ __forceinline__ int64_t load_rec<float>(const Rec<float> *__restrict__ r, float (&b)[9]) {
     const float4 *v = reinterpret_cast<const float4 *>(r);
     const float4 u0 = __ldg(v), u1 = __ldg(v + 1), u2 = __ldg(v + 2);
-    b[0] = u0.x; b[1] = u0.y; b[2] = u0.z;
-    b[3] = u1.x; b[4] = u1.y; b[5] = u1.z;
-    b[6] = u2.x; b[7] = u2.y; b[8] = u2.z;
-    return __float_as_int(u0.w);
+    b[0] = u0.x; b[1] = u0.y; b[2] = u0.z; b[3] = u0.w;
+    b[4] = u1.x; b[5] = u1.y; b[6] = u1.z; b[7] = u1.w;
+    b[8] = u2.x;
+    return __float_as_int(u2.y);
 }
 template <> __device__ __forceinline__ int64_t load_rec<double>(const Rec<double> *__restrict__ r, double (&b)[9]) {
     const double2 *v = reinterpret_cast<const double2 *>(r);
@@ -145,9 +142,9 @@ template <> __device__ __forceinline__ int64_t load_rec<df>(const Rec<df> *__res
 }
 
 __host__ __device__ inline Rec<float> make_rec(const double (&b)[9], int32_t col) {
-    Rec<float> r;
-    for (int i = 0; i < 9; ++i) r.row[i / 3].b[i % 3] = float(b[i]);
-    for (int a = 0; a < 3; ++a) r.row[a].col = col;
+    Rec<float> r{};
+    for (int i = 0; i < 9; ++i) r.b[i] = float(b[i]);
+    r.col = col;
     return r;
 }
 

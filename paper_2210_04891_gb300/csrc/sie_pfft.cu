@@ -645,11 +645,11 @@ __global__ void __launch_bounds__(256) k_project_cols(const int64_t *__restrict_
 // every number of right-hand sides.
 // With little arithmetic per record these kernels are bound by their loads: by
 // latency on a small mesh (a row is a chain of record, then the operand it
-// names: U records are in flight and the next U are fetched a chunk ahead,
+// names: U records are in flight and the next U columns are fetched a chunk ahead,
 // which leaves one round trip per chunk), by L1 wavefronts on a larger one (a
 // warp's load takes one per row and 128 bytes, however few lanes it serves).
-// Hence the layouts: a lane's coefficients and column are one 16-byte load, its
-// operand (the three components of a column, float4 [row][C]) another.
+// Hence the operand's layout: the three components of a column are one 16-byte
+// load (float4 [row][C]).
 constexpr int kSmallWarps = 2;   // warps per block: a small mesh still reaches every SM
 
 template <int U>   // COMP: output component a of column c
@@ -658,23 +658,28 @@ __device__ __forceinline__ void gather_row(const Rec<float> *__restrict__ rec, i
                                            float (&acc)[1]) {
     const int n = int(e1 - e0);
     if (n <= 0) return;
-    const float4 *v = reinterpret_cast<const float4 *>(rec + e0) + a;
+    constexpr int W = sizeof(Rec<float>) / 4;   // words per record: b[9], column
+    const float *v = rec[e0].b;
     X += c;
-    float4 bn[U];
+    int32_t cn[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) bn[u] = __ldg(v + 3 * int64_t(min(u, n - 1)));
+    for (int u = 0; u < U; ++u) cn[u] = __float_as_int(__ldg(v + W * int64_t(min(u, n - 1)) + 9));
     for (int i = 0; i < n; i += U) {
-        float4 b[U], x[U];
+        float b0[U], b1[U], b2[U];
+        float4 x[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            b[u] = bn[u];
-            x[u] = __ldg(X + int64_t(__float_as_int(b[u].w)) * C);
+            x[u] = __ldg(X + int64_t(cn[u]) * C);
+            const float *r = v + W * int64_t(min(i + u, n - 1)) + 3 * a;
+            b0[u] = __ldg(r);
+            b1[u] = __ldg(r + 1);
+            b2[u] = __ldg(r + 2);
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u) bn[u] = __ldg(v + 3 * int64_t(min(i + U + u, n - 1)));
+        for (int u = 0; u < U; ++u) cn[u] = __float_as_int(__ldg(v + W * int64_t(min(i + U + u, n - 1)) + 9));
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (i + u < n) acc[0] += b[u].x * x[u].x + b[u].y * x[u].y + b[u].z * x[u].z;
+            if (i + u < n) acc[0] += b0[u] * x[u].x + b1[u] * x[u].y + b2[u] * x[u].z;
     }
 }
 template <int U>   // all three components of column c
@@ -684,28 +689,32 @@ __device__ __forceinline__ void gather_row(const Rec<float> *__restrict__ rec, i
     const int n = int(e1 - e0);
     if (n <= 0) return;
     const float4 *v = reinterpret_cast<const float4 *>(rec + e0);
+    auto tail = [&](int i) {   // b[8] and the column
+        return __ldg(reinterpret_cast<const float2 *>(v + 3 * int64_t(min(i, n - 1)) + 2));
+    };
     X += c;
-    float4 bn[U];   // the next chunk's first rows: coefficients and column
+    float2 bn[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) bn[u] = __ldg(v + 3 * int64_t(min(u, n - 1)));
+    for (int u = 0; u < U; ++u) bn[u] = tail(u);
     for (int i = 0; i < n; i += U) {
-        float4 b0[U], b1[U], b2[U], x[U];
+        float4 u0[U], u1[U], x[U];
+        float b8[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            b0[u] = bn[u];
-            x[u] = __ldg(X + int64_t(__float_as_int(b0[u].w)) * C);
+            b8[u] = bn[u].x;
+            x[u] = __ldg(X + int64_t(__float_as_int(bn[u].y)) * C);
             const float4 *r = v + 3 * int64_t(min(i + u, n - 1));
-            b1[u] = __ldg(r + 1);
-            b2[u] = __ldg(r + 2);
+            u0[u] = __ldg(r);
+            u1[u] = __ldg(r + 1);
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u) bn[u] = __ldg(v + 3 * int64_t(min(i + U + u, n - 1)));
+        for (int u = 0; u < U; ++u) bn[u] = tail(i + U + u);
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (i + u < n) {
-                acc[0] += b0[u].x * x[u].x + b0[u].y * x[u].y + b0[u].z * x[u].z;
-                acc[1] += b1[u].x * x[u].x + b1[u].y * x[u].y + b1[u].z * x[u].z;
-                acc[2] += b2[u].x * x[u].x + b2[u].y * x[u].y + b2[u].z * x[u].z;
+                acc[0] += u0[u].x * x[u].x + u0[u].y * x[u].y + u0[u].z * x[u].z;
+                acc[1] += u0[u].w * x[u].x + u1[u].x * x[u].y + u1[u].y * x[u].z;
+                acc[2] += u1[u].z * x[u].x + u1[u].w * x[u].y + b8[u] * x[u].z;
             }
     }
 }
@@ -756,7 +765,7 @@ __global__ void __launch_bounds__(32 * kSmallWarps)
                 const float4 *__restrict__ cT, const float4 *__restrict__ phiT, const double *__restrict__ gram,
                 const int32_t *__restrict__ cond, const float2 *__restrict__ coef_dd, int ncond, int64_t nt,
                 int32_t R, int rpw, float4 *__restrict__ y_tri) {
-    constexpr int NA = COMP ? 1 : 3, U = COMP ? 8 : 4;
+    constexpr int NA = COMP ? 1 : 3, U = COMP ? 8 : 6;
     const int64_t gw = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int32_t Cn = 2 * R;
