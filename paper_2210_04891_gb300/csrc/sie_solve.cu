@@ -562,9 +562,9 @@ __global__ void k_pc_solve(const double2 *__restrict__ kappa, const int32_t *__r
     }
 }
 
-// Band solve L d L^T u = rhs for bands wider than a warp (31 < W < 1024), one
-// CTA of Wt >= W threads per (right-hand side, block), after assembling
-// rhs_i = -sum over the incident branches of s * kappa_e.  The sweeps go 32 pivots at a time: the CTA
+// Band solve L d L^T u = rhs for bands wider than a warp (31 < W < 1024), in place
+// on the right-hand sides k_pc_rhs assembled; one CTA of Wt >= W threads per
+// (right-hand side, block).  The sweeps go 32 pivots at a time: the CTA
 // stages the chunk's 32 x 32 triangle of L in shared memory, warp 0 finishes the
 // chunk's rows in registers (a shuffle broadcasts each pivot, no CTA barrier),
 // then every thread subtracts the chunk's contribution from one of the W band
@@ -572,13 +572,12 @@ __global__ void k_pc_solve(const double2 *__restrict__ kappa, const int32_t *__r
 // in the forward sweep, the column-major copy in the backward sweep), and the
 // rows that enter the band take their right-hand sides.  Pending values live in
 // a circular shared-memory window of S >= W + 32 rows.  Three barriers per 32
-// pivots instead of one per pivot.
+// pivots.  Used where k_pc_sweep_pipe's buffers do not fit shared memory.
 template <typename T, int MAXT>
 __global__ void __launch_bounds__(MAXT) k_pc_sweep_blk(
-    const C<T> *__restrict__ kappa, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ row_br,
-    const int8_t *__restrict__ row_sg, const int64_t *__restrict__ blk_off, int32_t nblk, int32_t W, int32_t S,
-    int64_t nunk, int64_t nb, const C<T> *__restrict__ band, const C<T> *__restrict__ bandc,
-    const int32_t *__restrict__ slot, C<T> *__restrict__ u) {
+    const int64_t *__restrict__ blk_off, int32_t nblk, int32_t W, int32_t S, int64_t nunk,
+    const C<T> *__restrict__ band, const C<T> *__restrict__ bandc, const int32_t *__restrict__ slot,
+    C<T> *__restrict__ u) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C<T> *pend = reinterpret_cast<C<T> *>(smem_raw);   // [S] window of pending rows
     C<T> *tri = pend + S;                              // [32][33] chunk triangle
@@ -589,16 +588,8 @@ __global__ void __launch_bounds__(MAXT) k_pc_sweep_blk(
     const C<T> *B = band + (int64_t(slot[r]) * nunk + o) * Wp;
     const C<T> *Bc = bandc + (int64_t(slot[r]) * nunk + o) * Wp;
     C<T> *x = u + r * nunk + o;
-    const C<T> *kr = kappa + r * nb;
     const C<T> zero = mk<T>(T(0), T(0));
     const int64_t smask = S - 1;
-    for (int64_t i = tid; i < n; i += nt) {
-        C<T> acc = zero;
-        for (int32_t k = row_ptr[o + i]; k < row_ptr[o + i + 1]; ++k)
-            acc = row_sg[k] > 0 ? csub(acc, kr[row_br[k]]) : cadd(acc, kr[row_br[k]]);
-        x[i] = acc;
-    }
-    __syncthreads();
     // ---- forward: L z = rhs, rows in increasing order
     for (int64_t i = tid; i < n && i < W + 32; i += nt) pend[i & smask] = x[i];
     for (int64_t k0 = 0; k0 < n; k0 += 32) {
@@ -702,6 +693,134 @@ __global__ void __launch_bounds__(MAXT) k_pc_sweep_blk(
         for (int t = tid; t < 32; t += nt) {
             const int64_t k = k0 + 32 + W + t;
             if (k < n) pend[k & smask] = x[n - 1 - k];
+        }
+    }
+}
+
+// The same sweeps as a pipeline, for bands whose chunk panels fit shared memory
+// twice.  A chunk's solve is a chain (31 shuffles and multiply-adds) and needs
+// only the 32 rows below the previous chunk, so warp 0 runs from chunk to chunk:
+// it takes the previous chunk's contribution to its own 32 rows, then finishes
+// them.  Meanwhile the other warps apply the previous chunk to the W - 32 rows
+// further down, let rows enter the window, and copy the next triangle and panel
+// (W x 32 entries of L) into shared memory asynchronously, a warp per row, so
+// that the copies coalesce and a chunk starts with its data present.  One barrier
+// per 32 pivots.  Every row takes the same contributions in the same order as in
+// k_pc_sweep_blk.  FP32 is bound by the chain, about 31 x 45 cycles a chunk (plates,
+// two blocks of 12.8k unknowns, band 154, 4 right-hand sides: 2.4 ms against 10.2 ms,
+// whose panels were read a row per thread), FP64 by the FP64 pipe.
+// Row k of a sweep is row k (forward, row-major band B) or n - 1 - k (backward,
+// column-major copy Bc); its entry at pivot k - d is elem(k)[d].
+template <typename V> __device__ __forceinline__ void cp_async_value(V *dst, const V *src) {
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+    static_assert(sizeof(V) == 8 || sizeof(V) == 16, "complex values");
+    if constexpr (sizeof(V) == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+}
+// a + e v (s = 1) or a - e v (s = -1).  FP64 in four FMAs (the pipe is what an FP64
+// panel waits for); FP32 as product and sum, the order of k_pc_sweep_blk.
+template <int S, typename V> __device__ __forceinline__ V pipe_madd(V a, V e, V v) {
+    if constexpr (std::is_same<V, double2>::value) {
+        if (S < 0) { e.x = -e.x; e.y = -e.y; }
+        return make_double2(::fma(-e.y, v.y, ::fma(e.x, v.x, a.x)), ::fma(e.y, v.x, ::fma(e.x, v.y, a.y)));
+    } else {
+        return S > 0 ? cadd(a, cmul(e, v)) : csub(a, cmul(e, v));
+    }
+}
+constexpr int kPipeTri = 32 * 33;
+constexpr size_t kPipeMaxSmem = 227 * 1024;
+template <typename T> size_t pipe_smem(int W, int S) {
+    return (size_t(S) + 2 * 32 + 2 * kPipeTri + 2 * size_t(W) * 33) * sizeof(C<T>);
+}
+template <typename T>
+__global__ void __launch_bounds__(512) k_pc_sweep_pipe(
+    const int64_t *__restrict__ blk_off, int32_t nblk, int32_t W, int32_t S, int64_t nunk,
+    const C<T> *__restrict__ band, const C<T> *__restrict__ bandc, const int32_t *__restrict__ slot,
+    C<T> *__restrict__ u) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C<T> *pend = reinterpret_cast<C<T> *>(smem_raw);   // [S] window of pending rows
+    C<T> *xc = pend + S;                               // [2][32] finished chunks
+    C<T> *tri = xc + 64;                               // [2][32][33] chunk triangles
+    C<T> *pan = tri + 2 * kPipeTri;                    // [2][W][33] chunk panels
+    const int64_t r = blockIdx.x / nblk, b = blockIdx.x % nblk;
+    const int64_t o = blk_off[b], n = blk_off[b + 1] - o;
+    const int Wp = W + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x >> 5) - 1;
+    const C<T> *B = band + (int64_t(slot[r]) * nunk + o) * Wp;
+    const C<T> *Bc = bandc + (int64_t(slot[r]) * nunk + o) * Wp;
+    C<T> *x = u + r * nunk + o;
+    const C<T> zero = mk<T>(T(0), T(0));
+    const int64_t smask = S - 1, nch = (n + 31) / 32;
+    for (int dir = 0; dir < 2; ++dir) {
+        auto elem = [&](int64_t k) { return dir ? Bc + (n - 1 - k) * Wp : B + k * Wp; };
+        auto enter = [&](int64_t k) {   // right-hand side of row k; the backward sweep divides by the pivot
+            if (!dir) return x[k];
+            const int64_t i = n - 1 - k;
+            const C<T> dg = B[i * Wp];
+            const T den = dg.x * dg.x + dg.y * dg.y;
+            return cmul(x[i], mk<T>(dg.x / den, -dg.y / den));
+        };
+        auto copy_tri = [&](int64_t c) {   // tri[l][j] = L[k0 + l][k0 + j], j < l
+            C<T> *dst = tri + (c & 1) * kPipeTri;
+            for (int l = warp; l < 32; l += nw)   // worker warps 1 .. nw: rows 1 .. 31
+                if (lane < l && c * 32 + l < n) cp_async_value(dst + l * 33 + lane, elem(c * 32 + l) + (l - lane));
+        };
+        auto copy_panel = [&](int64_t c) {   // row t below the chunk, entries at its pivots j within the band
+            C<T> *dst = pan + (c & 1) * (int64_t(W) * 33);
+            for (int t = warp - 1; t < W; t += nw) {
+                const int64_t k = c * 32 + 32 + t;
+                if (k >= n) break;
+                const int d = 32 + t - lane;
+                if (d <= W) cp_async_value(dst + t * 33 + lane, elem(k) + d);
+            }
+        };
+        // contribution of the finished chunk (values v, panel row p) to the row t below it
+        auto apply = [&](const C<T> *p, const C<T> *v, int t) {
+            const int j0 = 32 + t - W > 0 ? 32 + t - W : 0;   // band edge
+            C<T> acc = zero;
+#pragma unroll 8
+            for (int j = 0; j < 32; ++j)
+                if (j >= j0) acc = pipe_madd<1>(acc, p[t * 33 + j], v[j]);
+            return acc;
+        };
+        for (int64_t k = threadIdx.x; k < n && k < W + 32; k += blockDim.x) pend[k & smask] = enter(k);
+        if (warp > 0) copy_tri(0);
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncthreads();
+        for (int64_t c = 0; c < nch; ++c) {
+            const int64_t k0 = c * 32;
+            const C<T> *pp = pan + ((c - 1) & 1) * (int64_t(W) * 33), *xp = xc + ((c - 1) & 1) * 32;
+            if (warp == 0) {
+                const bool in = k0 + lane < n;
+                C<T> v = in ? pend[(k0 + lane) & smask] : zero;
+                if (c > 0 && in) v = csub(v, apply(pp, xp, lane));
+                const C<T> *tl = tri + (c & 1) * kPipeTri + lane * 33;
+#pragma unroll
+                for (int j = 0; j < 31; ++j) {
+                    C<T> xj;
+                    xj.x = __shfl_sync(0xffffffffu, v.x, j);
+                    xj.y = __shfl_sync(0xffffffffu, v.y, j);
+                    if (lane > j) v = pipe_madd<-1>(v, tl[j], xj);
+                }
+                xc[(c & 1) * 32 + lane] = v;
+                if (in) x[dir ? n - 1 - k0 - lane : k0 + lane] = v;
+            } else {
+                if (c + 1 < nch) {
+                    copy_tri(c + 1);
+                    copy_panel(c);
+                }
+                if (c > 0) {
+                    if (warp == nw) {   // rows entering the window
+                        const int64_t k = k0 + W + lane;
+                        if (k < n) pend[k & smask] = enter(k);
+                    }
+                    for (int t = int(threadIdx.x); t < W; t += 32 * nw) {   // threads 32 ..: rows 32 ..
+                        const int64_t k = k0 + t;
+                        if (k < n) pend[k & smask] = csub(pend[k & smask], apply(pp, xp, t));
+                    }
+                }
+                asm volatile("cp.async.wait_all;\n" ::: "memory");
+            }
+            __syncthreads();
         }
     }
 }
@@ -1252,23 +1371,33 @@ int pc_apply_t(pfft_plan *p, const double2 *y, double2 *z, int32_t R, cudaStream
             k_pc_sweep<T><<<nblk_(int64_t(R) * nblk * 32, 128), 128, sm, st>>>(
                 s->d_blk_off, s->d_tile_off, nblk, s->nunk, s->nchunks, tiles, dinv, s->d_slot, R, u);
         } else if (s->W < kWideMax) {
-            const int wt = (s->W + 1 + 31) / 32 * 32;
             const C<T> *band, *bandc;
             if constexpr (f32) { band = s->d_band32; bandc = s->d_bandc32; } else { band = s->d_band; bandc = s->d_bandc; }
-            // blocked sweeps: Wt >= W threads, window of S >= W + 32 rows in shared memory
-            int S = 64;
+            k_pc_rhs<T><<<nblk_(int64_t(R) * s->nunk), 256, 0, st>>>(kappa, s->d_row_ptr, s->d_row_br, s->d_row_sg,
+                                                                       s->nunk, p->nb, R, u);
+            SIE_LAUNCH_CHECK(p);
+            int S = 64;   // window of S >= W + 32 rows in shared memory
             while (S < s->W + 32) S *= 2;
-            const size_t sm = size_t(S + 32 * 33 + 32) * sizeof(C<T>);
-            if (wt <= 256) {
-                if (int rc = set_smem((const void *)k_pc_sweep_blk<T, 256>, sm)) return rc;
-                k_pc_sweep_blk<T, 256><<<unsigned(int64_t(R) * nblk), wt, sm, st>>>(
-                    kappa, s->d_row_ptr, s->d_row_br, s->d_row_sg, s->d_blk_off, nblk, s->W, S, s->nunk, p->nb, band,
-                    bandc, s->d_slot, u);
+            const unsigned ctas = unsigned(int64_t(R) * nblk);
+            // the pipeline where two panels fit (band below about 400 in FP32, 180 in FP64)
+            const size_t pipe = pipe_smem<T>(s->W, S);
+            if (pipe <= kPipeMaxSmem) {
+                const int workers = std::min(15, std::max(7, (s->W + 31) / 32));
+                if (int rc = set_smem((const void *)k_pc_sweep_pipe<T>, pipe)) return rc;
+                k_pc_sweep_pipe<T><<<ctas, 32 * (workers + 1), pipe, st>>>(s->d_blk_off, nblk, s->W, S, s->nunk, band,
+                                                                           bandc, s->d_slot, u);
             } else {
-                if (int rc = set_smem((const void *)k_pc_sweep_blk<T, 1024>, sm)) return rc;
-                k_pc_sweep_blk<T, 1024><<<unsigned(int64_t(R) * nblk), wt, sm, st>>>(
-                    kappa, s->d_row_ptr, s->d_row_br, s->d_row_sg, s->d_blk_off, nblk, s->W, S, s->nunk, p->nb, band,
-                    bandc, s->d_slot, u);
+                const int wt = (s->W + 1 + 31) / 32 * 32;
+                const size_t sm = size_t(S + 32 * 33 + 32) * sizeof(C<T>);
+                if (wt <= 256) {
+                    if (int rc = set_smem((const void *)k_pc_sweep_blk<T, 256>, sm)) return rc;
+                    k_pc_sweep_blk<T, 256><<<ctas, wt, sm, st>>>(s->d_blk_off, nblk, s->W, S, s->nunk, band, bandc,
+                                                                 s->d_slot, u);
+                } else {
+                    if (int rc = set_smem((const void *)k_pc_sweep_blk<T, 1024>, sm)) return rc;
+                    k_pc_sweep_blk<T, 1024><<<ctas, wt, sm, st>>>(s->d_blk_off, nblk, s->W, S, s->nunk, band, bandc,
+                                                                  s->d_slot, u);
+                }
             }
         } else {
             if constexpr (f32) return fail(SIE_ERR_ARG, "preconditioner: FP32 sweeps need a band width below 1024");

@@ -1,0 +1,46 @@
+"""The pipelined band sweeps (bands 32 to about 180 in FP64, 400 in FP32) and the
+kernel of wider bands, against nested dissection of the same Laplacian (another
+factorisation, another order: 1e-10, the bar of those two routes) and FP32
+against FP64 (1e-4, the bar of the FP32 sweeps), on plates whose bands lie on
+both sides of the limits and whose unknowns are no multiple of the 32-pivot chunk."""
+import numpy as np
+import pytest
+
+import synth
+from synth.meshes import box_mesh
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2210_04891_gb300 import api, native as N, PREC_FP64, PREC_MIXED  # noqa: E402
+
+bands = {}
+
+
+@pytest.mark.parametrize("nx,ny", [(14, 12), (20, 17), (31, 30), (45, 43), (64, 62), (70, 69), (101, 97), (154, 152)])
+def test_band_sweeps_match_nested_dissection(nx, ny):
+    h = 40e-6
+    m = box_mesh(nx * h, ny * h, 35e-6, nx, ny, 1, jitter=0.1, seed=nx)
+    M = api.Mesh.from_synth(m)
+    L = api.Loops(M, m.ports)
+    P = api.Plan(M, L, dict(grid=(16, 16, 8), n_touch=4, near_factor=1.0, near_min_diam=1.0))
+    api.precond_set_method(P, N.PC_BAND)
+    bands[nx] = api.precond_info(P)["band_width"]
+    assert 31 < bands[nx] < 1024
+    R = 3
+    y = torch.from_numpy(synth.complex_gaussian(L.nl, R, seed=ny)).cuda()
+    om = 2 * np.pi * np.array([1e7, 1e9, 1e9])
+    z = api.pfft_precond_apply(P, y, om)
+    f = api.pfft_precond_apply(P, y, om, prec=PREC_MIXED)
+    api.precond_set_method(P, N.PC_ND)
+    ref = api.pfft_precond_apply(P, y, om)
+    nrm = torch.linalg.norm(ref, dim=1)
+    assert (torch.linalg.norm(z - ref, dim=1) / nrm).max().item() < 1e-10
+    assert (torch.linalg.norm(f - ref, dim=1) / nrm).max().item() < 1e-4
+
+
+def test_bands_cover_the_limits():
+    if len(bands) < 8:
+        pytest.skip("needs every size above")
+    w = sorted(bands.values())
+    assert w[0] < 64 and any(140 < v < 178 for v in w) and any(180 < v < 390 for v in w) and w[-1] > 400
