@@ -346,26 +346,6 @@ __global__ void k_alpha_tri(const double2 *__restrict__ x, int64_t nl, const Tou
     }
 }
 
-// acc += b x for double-float b and x into an unnormalised double-float sum:
-// the high part takes one FP32 add per term (the chain a gather runs along),
-// the two-product error of the high parts, the two-sum error of that add and
-// the cross products of high and low parts go to the low part, one add per
-// term.  A sum of n terms keeps about 48 bits plus log2(n); readers treat
-// (hi, lo) as the value hi + lo, whatever its normalisation.
-__device__ __forceinline__ void df_acc(df &acc, df b, df x) {
-    const float p = b.hi * x.hi;
-    const float e = fmaf(b.hi, x.hi, -p);
-    const float s = acc.hi + p, bb = s - acc.hi;
-    const float f = (acc.hi - (s - bb)) + (p - bb);
-    acc.hi = s;
-    acc.lo += fmaf(b.lo, x.hi, fmaf(b.hi, x.lo, e + f));
-}
-// the same value as a normalised pair (two-sum of its parts)
-__device__ __forceinline__ df df_norm(df a) {
-    const float s = a.hi + a.lo, bb = s - a.hi;
-    return df(s, (a.hi - (s - bb)) + (a.lo - bb));
-}
-
 // V complex values at p (16-byte aligned when V = 2).
 template <typename T, int V> __device__ __forceinline__ void ldv(const C<T> *p, C<T> (&v)[V]) {
     if constexpr (V == 2) {

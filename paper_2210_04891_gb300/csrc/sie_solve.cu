@@ -68,6 +68,10 @@ struct PrecondState {
     double2 *d_tile64 = nullptr, *d_dinv64 = nullptr;
     float2 *d_tile32 = nullptr, *d_dinv32 = nullptr;
     cdf *d_tiledf = nullptr, *d_dinvdf = nullptr;   // double-float sweeps (SIE_PREC_DF)
+    // chunk matrices of the matrix sweeps (k_pc_blocks), FP64 and double-float, built by
+    // pc_blocks_prepare for few chains
+    double2 *d_blk64 = nullptr;
+    cdf *d_blkdf = nullptr;
     float2 *d_u32 = nullptr;          // FP32 sweep buffer [R][nunk]
     // bands wider than a warp (31 < W < 1024): FP32 roundings of band and bandc (mixed form)
     float2 *d_band32 = nullptr, *d_bandc32 = nullptr;
@@ -129,7 +133,7 @@ void plan_free_precond(pfft_plan *p) {
     for (void *a : {(void *)p->pc->d_tile64, (void *)p->pc->d_dinv64, (void *)p->pc->d_tile32,
                     (void *)p->pc->d_dinv32, (void *)p->pc->d_u32, (void *)p->pc->d_a32,
                     (void *)p->pc->d_band32, (void *)p->pc->d_bandc32, (void *)p->pc->d_tiledf,
-                    (void *)p->pc->d_dinvdf, (void *)p->pc->d_adf})
+                    (void *)p->pc->d_dinvdf, (void *)p->pc->d_adf, (void *)p->pc->d_blk64, (void *)p->pc->d_blkdf})
         if (a) cudaFree(a);
     for (void *a : {(void *)p->pc->d_band, (void *)p->pc->d_bandc, (void *)p->pc->d_a, (void *)p->pc->d_kappa, (void *)p->pc->d_u,
                     (void *)p->pc->d_ibr, (void *)p->pc->d_slot, (void *)p->pc->d_ndL64, (void *)p->pc->d_ndL32,
@@ -707,8 +711,8 @@ __global__ void __launch_bounds__(MAXT) k_pc_sweep_blk(
 // that the copies coalesce and a chunk starts with its data present.  One barrier
 // per 32 pivots.  Every row takes the same contributions in the same order as in
 // k_pc_sweep_blk.  FP32 is bound by the chain, about 31 x 45 cycles a chunk (plates,
-// two blocks of 12.8k unknowns, band 154, 4 right-hand sides: 2.4 ms against 10.2 ms,
-// whose panels were read a row per thread), FP64 by the FP64 pipe.
+// two blocks of 12.8k unknowns, 4 right-hand sides: 2.4 ms against 10.2 ms,
+// whose panels were read a row per thread), FP64 by the FP64 pipe (9.9, 17.6 ms).
 // Row k of a sweep is row k (forward, row-major band B) or n - 1 - k (backward,
 // column-major copy Bc); its entry at pivot k - d is elem(k)[d].
 template <typename V> __device__ __forceinline__ void cp_async_value(V *dst, const V *src) {
@@ -1085,6 +1089,193 @@ __global__ void __launch_bounds__(128, 2) k_pc_sweep(
     asm volatile("cp.async.wait_group 0;\n" ::);
 }
 
+// ---- Matrix sweeps: the narrow band's solves for few chains (right-hand side x
+// block).  k_pc_sweep runs a chain on one warp, 32 dependent steps of about 70
+// (double-float) instructions a chunk; with a handful of chains the chip idles
+// beside them.  In a chunk of 32 pivots z_c = A_c^-1 (b_c - P_c z_c-1), A_c the
+// chunk's unit triangle and P_c its coupling to the last W rows of the chunk
+// before.  With G_c = A_c^-1 and M_c = G_c P_c formed once per factor,
+//   z_c = G_c b_c - M_c z_c-1:
+// the first term is independent of the other chunks (k_pc_chunks, a warp per chunk
+// over the whole chip), the second a 32 x W product, which kMatWarps warps of the
+// chain's CTA share by columns.  A_c is a diagonal block of the factor of a
+// diagonally dominant Laplacian, so its inverse is as well scaled as itself.
+// Bar (1.5k unknowns, one chain), both sweeps: double-float 424 us stepped, 100 us
+// as matrices; 3.6k unknowns, 3 chains, FP64: 1460 and 275 us for the whole
+// application.
+constexpr int kMatWarps = 4, kMatStages = 4;
+// Chains up to which the matrix sweeps serve (their matrices cost 32 (W + 32)
+// values per chunk and direction, and a product more per chunk than the steps).
+constexpr int64_t kMatChains = 64;
+
+// blocks[slot][dir][chunk][W + 32][32]: W columns of M_c (rows 32 - W .. 31 of the
+// chunk before), then the 32 columns of G_c; lanes over the chunk's rows.  One
+// CTA per (slot, dir, chunk); chunk rows as in k_pc_sweep_pipe.
+template <typename T>
+__global__ void __launch_bounds__(256) k_pc_blocks(
+    const double2 *__restrict__ band, const double2 *__restrict__ bandc, const int64_t *__restrict__ blk_off,
+    const int64_t *__restrict__ tile_off, int32_t nblk, int32_t W, int64_t nunk, int64_t nchunks,
+    C<T> *__restrict__ blocks) {
+    extern __shared__ __align__(16) unsigned char pc_smem[];
+    double2 *A = reinterpret_cast<double2 *>(pc_smem), *G = A + 32 * 33, *P = G + 32 * 33;   // pitch 33
+    const int64_t gc = blockIdx.x % nchunks, sd = blockIdx.x / nchunks;
+    const int dir = int(sd & 1);
+    const int64_t s = sd >> 1;
+    int lo = 0, hi = nblk - 1;   // block holding chunk gc
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) / 2;
+        if (tile_off[mid] <= gc) lo = mid; else hi = mid - 1;
+    }
+    const int64_t c = gc - tile_off[lo], o = blk_off[lo], n = blk_off[lo + 1] - o;
+    auto elem = [&](int64_t k, int d) {
+        if (d < 1 || d > W || k >= n || k - d < 0) return make_double2(0.0, 0.0);
+        return dir ? bandc[(s * nunk + o + n - 1 - k) * (W + 1) + d] : band[(s * nunk + o + k) * (W + 1) + d];
+    };
+    for (int i = threadIdx.x; i < 32 * 32; i += blockDim.x) {
+        const int l = i >> 5, j = i & 31;
+        A[l * 33 + j] = elem(c * 32 + l, l - j);
+        P[l * 33 + j] = elem(c * 32 + l, 32 + l - j);   // column j: row j of the chunk before
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {   // G: one column per lane by forward substitution
+        const int j = threadIdx.x;
+        for (int l = 0; l < 32; ++l) {
+            double2 a = make_double2(l == j ? 1.0 : 0.0, 0.0);
+            for (int i = 0; i < l; ++i) {
+                const double2 e = A[l * 33 + i], g = i >= j ? G[i * 33 + j] : make_double2(0.0, 0.0);
+                a.x = ::fma(-e.x, g.x, ::fma(e.y, g.y, a.x));
+                a.y = ::fma(-e.x, g.y, ::fma(-e.y, g.x, a.y));
+            }
+            G[l * 33 + j] = a;
+        }
+    }
+    __syncthreads();
+    C<T> *out = blocks + blockIdx.x * int64_t(W + 32) * 32;
+    for (int i = threadIdx.x; i < (W + 32) * 32; i += blockDim.x) {
+        const int l = i & 31, q = i >> 5;
+        double2 v = make_double2(0.0, 0.0);
+        if (q >= W) {
+            v = G[l * 33 + (q - W)];
+        } else {
+            for (int j = 0; j <= l; ++j) {
+                const double2 g = G[l * 33 + j], e = P[j * 33 + 32 - W + q];
+                v.x = ::fma(g.x, e.x, ::fma(-g.y, e.y, v.x));
+                v.y = ::fma(g.x, e.y, ::fma(g.y, e.x, v.y));
+            }
+        }
+        out[i] = mk<T>(T(v.x), T(v.y));
+    }
+}
+
+// acc += m z
+__device__ __forceinline__ void mat_acc(double2 &acc, double2 m, double2 z) {
+    acc.x = ::fma(m.x, z.x, ::fma(-m.y, z.y, acc.x));
+    acc.y = ::fma(m.x, z.y, ::fma(m.y, z.x, acc.y));
+}
+__device__ __forceinline__ void mat_acc(cdf &acc, cdf m, cdf z) {
+    df_acc(acc.x, m.x, z.x);
+    df_acc(acc.x, -m.y, z.y);
+    df_acc(acc.y, m.x, z.y);
+    df_acc(acc.y, m.y, z.x);
+}
+__device__ __forceinline__ double2 mat_norm(double2 a) { return a; }
+__device__ __forceinline__ cdf mat_norm(cdf a) { return cdf{df_norm(a.x), df_norm(a.y)}; }
+
+// b_c <- G_c b_c of every chunk of R right-hand sides, in place, a warp per chunk;
+// the backward sweep's right-hand sides are divided by the pivots first.
+template <typename T>
+__global__ void __launch_bounds__(64) k_pc_chunks(
+    const int64_t *__restrict__ blk_off, const int64_t *__restrict__ tile_off, int32_t nblk, int32_t W, int64_t nunk,
+    int64_t nchunks, const C<T> *__restrict__ blocks, const C<T> *__restrict__ dinv, const int32_t *__restrict__ slot,
+    int32_t R, int dir, C<T> *__restrict__ xs) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    if (i >= R * nchunks) return;
+    const int64_t r = i / nchunks, gc = i - r * nchunks;
+    int lo = 0, hi = nblk - 1;   // block holding chunk gc
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) / 2;
+        if (tile_off[mid] <= gc) lo = mid; else hi = mid - 1;
+    }
+    const int64_t o = blk_off[lo], n = blk_off[lo + 1] - o, k = (gc - tile_off[lo]) * 32 + lane;
+    const int64_t row = o + (dir ? n - 1 - k : k), sl = slot[r];
+    C<T> v = mk<T>(T(0.0), T(0.0)), acc = v;
+    if (k < n) v = xs[r * nunk + row];
+    if (dir && k < n) v = mat_norm(cmul(v, dinv[sl * nunk + row]));
+    const C<T> *g = blocks + ((sl * 2 + dir) * nchunks + gc) * (int64_t(W + 32) * 32) + int64_t(W) * 32 + lane;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) mat_acc(acc, g[j * 32], shfl_c(v, j));
+    if (k < n) xs[r * nunk + row] = mat_norm(acc);
+}
+
+// z_c = (G_c b_c) - M_c z_c-1 along a chain, in place.
+template <typename T>
+__global__ void __launch_bounds__(32 * kMatWarps) k_pc_sweep_mat(
+    const int64_t *__restrict__ blk_off, const int64_t *__restrict__ tile_off, int32_t nblk, int32_t W, int64_t nunk,
+    int64_t nchunks, const C<T> *__restrict__ blocks, const int32_t *__restrict__ slot, int dir,
+    C<T> *__restrict__ xs) {
+    extern __shared__ __align__(16) unsigned char pc_smem[];
+    C<T> *part = reinterpret_cast<C<T> *>(pc_smem);   // [kMatWarps][32] column shares of M z
+    C<T> *zp = part + kMatWarps * 32;                 // [32] the chunk before
+    C<T> *gs = zp + 32;                               // [kMatStages][32] G_c b_c
+    C<T> *ring = gs + kMatStages * 32;                // [kMatStages][W][32] columns of M
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t r = blockIdx.x / nblk, b = blockIdx.x % nblk;
+    const int64_t o = blk_off[b], n = blk_off[b + 1] - o;
+    const int nch = int((n + 31) / 32);
+    const int64_t per = int64_t(W + 32) * 32;
+    C<T> *x = xs + r * nunk + o;
+    const C<T> *blk = blocks + ((int64_t(slot[r]) * 2 + dir) * nchunks + tile_off[b]) * per;
+    auto row = [&](int64_t k) { return dir ? n - 1 - k : k; };
+    // a warp's columns of M_c (and warp 0's G_c b_c), copied kMatStages - 1 chunks
+    // ahead: a register fetched ahead would be waited for when it is renamed
+    auto copy = [&](int c) {
+        if (c < nch) {
+            const int st = c & (kMatStages - 1);
+            for (int q = warp; q < W; q += kMatWarps)
+                cp_async_value(ring + (st * W + q) * 32 + lane, blk + c * per + q * 32 + lane);
+            if (warp == 0 && int64_t(c) * 32 + lane < n)
+                cp_async_value(gs + st * 32 + lane, const_cast<const C<T> *>(x) + row(int64_t(c) * 32 + lane));
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    static_assert((kMatStages & (kMatStages - 1)) == 0, "stages: a power of two");
+#pragma unroll
+    for (int k = 0; k < kMatStages - 1; ++k) copy(k);
+    for (int c = 0; c < nch; ++c) {
+        const int st = c & (kMatStages - 1);
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(kMatStages - 2) : "memory");   // own columns of chunk c
+        __syncwarp();
+        if (c > 0) {
+            C<T> acc = mk<T>(T(0.0), T(0.0));
+            const C<T> *m = ring + st * W * 32 + lane;
+#pragma unroll 4
+            for (int q = warp; q < W; q += kMatWarps) mat_acc(acc, m[q * 32], zp[32 - W + q]);
+            part[warp * 32 + lane] = acc;   // warps without columns leave zeros
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const int64_t k = int64_t(c) * 32 + lane;
+            C<T> z = k < n ? gs[st * 32 + lane] : mk<T>(T(0.0), T(0.0));
+            if (c > 0) {
+                C<T> p[kMatWarps];
+#pragma unroll
+                for (int w = 0; w < kMatWarps; ++w) p[w] = part[w * 32 + lane];
+#pragma unroll
+                for (int h = kMatWarps / 2; h > 0; h /= 2)
+#pragma unroll
+                    for (int w = 0; w < h; ++w) p[w] = cadd(p[w], p[w + h]);
+                z = mat_norm(csub(z, p[0]));
+            }
+            zp[lane] = z;
+            if (k < n) x[row(k)] = z;
+        }
+        copy(c + kMatStages - 1);   // the stage of chunk c - 1: every warp has read its own columns
+        __syncthreads();
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+
 // Branch currents i_e = a_e (phi_tail - phi_head + emf_e) = a_e (u_t - u_h) + kappa_e.
 template <typename T>
 __global__ void k_pc_currents(const C<T> *__restrict__ u, int64_t nunk, const C<T> *__restrict__ kappa,
@@ -1186,12 +1377,14 @@ int pc_prepare(pfft_plan *p, const double *omega, int32_t R, std::vector<int32_t
     if (s->d_band) cudaFreeAsync(s->d_band, st);
     if (s->d_bandc) cudaFreeAsync(s->d_bandc, st);
     for (void *q : {(void *)s->d_tile64, (void *)s->d_dinv64, (void *)s->d_tile32, (void *)s->d_dinv32,
-                    (void *)s->d_tiledf, (void *)s->d_dinvdf, (void *)s->d_adf})
+                    (void *)s->d_tiledf, (void *)s->d_dinvdf, (void *)s->d_adf, (void *)s->d_blk64, (void *)s->d_blkdf})
         if (q) cudaFreeAsync(q, st);
     s->d_tile64 = s->d_dinv64 = nullptr;
     s->d_tile32 = s->d_dinv32 = nullptr;
     s->d_tiledf = s->d_dinvdf = nullptr;
     s->d_adf = nullptr;
+    s->d_blk64 = nullptr;
+    s->d_blkdf = nullptr;
     if (s->d_a) cudaFreeAsync(s->d_a, st);
     if (s->d_a32) cudaFreeAsync(s->d_a32, st);
     if (s->d_band32) cudaFreeAsync(s->d_band32, st);
@@ -1318,6 +1511,36 @@ int pc_prepare(pfft_plan *p, const double *omega, int32_t R, std::vector<int32_t
     return SIE_OK;
 }
 
+template <typename T>
+int sweep_mat(pfft_plan *p, int32_t nblk, const C<T> *blocks, const C<T> *dinv, int32_t R, C<T> *u, cudaStream_t st) {
+    PrecondState *s = p->pc;
+    const size_t sm = (size_t(kMatWarps + 1 + kMatStages) * 32 + size_t(kMatStages) * s->W * 32) * sizeof(C<T>);
+    if (int rc = set_smem((const void *)k_pc_sweep_mat<T>, sm)) return rc;
+    for (int dir = 0; dir < 2; ++dir) {
+        k_pc_chunks<T><<<nblk_(int64_t(R) * s->nchunks * 32, 64), 64, 0, st>>>(
+            s->d_blk_off, s->d_tile_off, nblk, s->W, s->nunk, s->nchunks, blocks, dinv, s->d_slot, R, dir, u);
+        SIE_LAUNCH_CHECK(p);
+        k_pc_sweep_mat<T><<<unsigned(R * nblk), 32 * kMatWarps, sm, st>>>(
+            s->d_blk_off, s->d_tile_off, nblk, s->W, s->nunk, s->nchunks, blocks, s->d_slot, dir, u);
+        SIE_LAUNCH_CHECK(p);
+    }
+    return SIE_OK;
+}
+
+// branch currents and loop currents from the node potentials u
+template <typename T>
+int pc_finish(pfft_plan *p, const C<T> *kappa, const C<T> *a, C<T> *ibr, const C<T> *u, double2 *z, int32_t R,
+              cudaStream_t st) {
+    PrecondState *s = p->pc;
+    k_pc_currents<T><<<nblk_(p->nb * R), 256, 0, st>>>(u, s->nunk, kappa, a, s->d_slot, s->d_unk_of_node,
+                                                       p->d_tail, p->d_head, p->nb, R, ibr);
+    SIE_LAUNCH_CHECK(p);
+    k_pc_out<T><<<nblk_(p->nl * R), 256, 0, st>>>(ibr, p->d_link_branch, s->d_src_ptr, s->d_src_br, s->d_src_sg,
+                                                  p->nb, p->nl, R, z);
+    SIE_LAUNCH_CHECK(p);
+    return SIE_OK;
+}
+
 // z = P^-1 y.  T = float: FP32 band factors and FP32 bookkeeping (mixed form,
 // band width <= 31); T = double: everything in FP64.
 template <typename T>
@@ -1344,11 +1567,15 @@ int pc_apply_t(pfft_plan *p, const double2 *y, double2 *z, int32_t R, cudaStream
             k_pc_rhs<T><<<nblk_(int64_t(R) * s->nunk), 256, 0, st>>>(kappa, s->d_row_ptr, s->d_row_br, s->d_row_sg,
                                                                        s->nunk, p->nb, R, u);
             SIE_LAUNCH_CHECK(p);
-            const size_t sm = size_t(4) * pc_nbuf<T>() * PC_TILE * sizeof(C<T>);
-            if (int rc = set_smem((const void *)k_pc_sweep<T>, sm)) return rc;
-            k_pc_sweep<T><<<nblk_(int64_t(R) * nblk * 32, 128), 128, sm, st>>>(
-                s->d_blk_off, s->d_tile_off, nblk, s->nunk, s->nchunks, s->d_tiledf, s->d_dinvdf, s->d_slot, R, u);
-            SIE_LAUNCH_CHECK(p);
+            if (s->d_blkdf && R * int64_t(nblk) <= kMatChains) {
+                if (int rc = sweep_mat<T>(p, nblk, s->d_blkdf, s->d_dinvdf, R, u, st)) return rc;
+            } else {
+                const size_t sm = size_t(4) * pc_nbuf<T>() * PC_TILE * sizeof(C<T>);
+                if (int rc = set_smem((const void *)k_pc_sweep<T>, sm)) return rc;
+                k_pc_sweep<T><<<nblk_(int64_t(R) * nblk * 32, 128), 128, sm, st>>>(
+                    s->d_blk_off, s->d_tile_off, nblk, s->nunk, s->nchunks, s->d_tiledf, s->d_dinvdf, s->d_slot, R, u);
+                SIE_LAUNCH_CHECK(p);
+            }
         }
     } else if (s->nd && s->nunk > 0) {
         k_pc_rhs<T><<<nblk_(int64_t(R) * s->nunk), 256, 0, st>>>(kappa, s->d_row_ptr, s->d_row_br, s->d_row_sg,
@@ -1363,6 +1590,12 @@ int pc_apply_t(pfft_plan *p, const double2 *y, double2 *z, int32_t R, cudaStream
             k_pc_rhs<T><<<nblk_(int64_t(R) * s->nunk), 256, 0, st>>>(kappa, s->d_row_ptr, s->d_row_br, s->d_row_sg,
                                                                        s->nunk, p->nb, R, u);
             SIE_LAUNCH_CHECK(p);
+            if constexpr (!f32) {
+                if (s->d_blk64 && R * int64_t(nblk) <= kMatChains) {
+                    if (int rc = sweep_mat<T>(p, nblk, s->d_blk64, s->d_dinv64, R, u, st)) return rc;
+                    return pc_finish<T>(p, kappa, a, ibr, u, z, R, st);
+                }
+            }
             // four warps per CTA, pc_nbuf tiles of shared memory per warp
             const size_t sm = size_t(4) * pc_nbuf<T>() * PC_TILE * sizeof(C<T>);
             if (int rc = set_smem((const void *)k_pc_sweep<T>, sm)) return rc;
@@ -1408,11 +1641,30 @@ int pc_apply_t(pfft_plan *p, const double2 *y, double2 *z, int32_t R, cudaStream
         }
         SIE_LAUNCH_CHECK(p);
     }
-    k_pc_currents<T><<<nblk_(p->nb * R), 256, 0, st>>>(u, s->nunk, kappa, a, s->d_slot, s->d_unk_of_node,
-                                                       p->d_tail, p->d_head, p->nb, R, ibr);
-    SIE_LAUNCH_CHECK(p);
-    k_pc_out<T><<<nblk_(p->nl * R), 256, 0, st>>>(ibr, p->d_link_branch, s->d_src_ptr, s->d_src_br, s->d_src_sg,
-                                                  p->nb, p->nl, R, z);
+    return pc_finish<T>(p, kappa, a, ibr, u, z, R, st);
+}
+
+// Chunk matrices for R right-hand sides' sweeps in FP64 or double-float, if the
+// matrix sweeps will serve them; before a capture, on the factors of pc_prepare.
+int pc_blocks_prepare(pfft_plan *p, int32_t R, bool dfl, cudaStream_t st) {
+    PrecondState *s = p->pc;
+    const int32_t nblk = int32_t(s->blk_off.size()) - 1;
+    if (s->nd || s->W > 31 || s->W < 1 || s->nunk == 0 || R * int64_t(nblk) > kMatChains) return SIE_OK;
+    if (dfl ? s->d_blkdf != nullptr : s->d_blk64 != nullptr) return SIE_OK;
+    const int64_t ctas = int64_t(s->nslots) * 2 * s->nchunks;
+    if (ctas > INT32_MAX) return SIE_OK;
+    const size_t bytes = size_t(ctas) * (s->W + 32) * 32 * sizeof(double2), sm = size_t(3) * 32 * 33 * sizeof(double2);
+    if (dfl) {
+        SIE_CUDA(pool_alloc(p, &s->d_blkdf, bytes, st));
+        if (int rc = set_smem((const void *)k_pc_blocks<df>, sm)) return rc;
+        k_pc_blocks<df><<<unsigned(ctas), 256, sm, st>>>(s->d_band, s->d_bandc, s->d_blk_off, s->d_tile_off, nblk,
+                                                         s->W, s->nunk, s->nchunks, s->d_blkdf);
+    } else {
+        SIE_CUDA(pool_alloc(p, &s->d_blk64, bytes, st));
+        if (int rc = set_smem((const void *)k_pc_blocks<double>, sm)) return rc;
+        k_pc_blocks<double><<<unsigned(ctas), 256, sm, st>>>(s->d_band, s->d_bandc, s->d_blk_off, s->d_tile_off, nblk,
+                                                             s->W, s->nunk, s->nchunks, s->d_blk64);
+    }
     SIE_LAUNCH_CHECK(p);
     return SIE_OK;
 }
@@ -1631,6 +1883,8 @@ extern "C" int pfft_precond_apply(pfft_plan *p, const void *y, void *z, int32_t 
     std::vector<int32_t> slot;
     int rc = pc_prepare(p, omega, nrhs, slot, st);
     if (rc) return rc;
+    if (prec != SIE_PREC_MIXED && (rc = pc_blocks_prepare(p, nrhs, prec == SIE_PREC_DF && pc_df_route(p), st)))
+        return rc;
     rc = pc_apply_async(p, (const double2 *)y, (double2 *)z, nrhs, prec, st);
     if (rc) return rc;
     SIE_CUDA(cudaStreamSynchronize(st));
@@ -1773,6 +2027,9 @@ int gmres_create(pfft_plan *p, const double *freqs, int32_t nf, const int32_t *p
     // the tests' P^-1 (b - Z x): FP64, or with refine = 2 on the narrow band route the
     // double-float sweeps (within 1e-11 of FP64, a third of its time)
     g->outer_pc_prec = g->pc_prec == SIE_PREC_DF ? SIE_PREC_DF : g->outer_prec;
+    for (int prec : {g->pc_prec, g->outer_pc_prec})
+        if (g->use_pc && prec != SIE_PREC_MIXED && (rc = pc_blocks_prepare(p, R, prec == SIE_PREC_DF, st)))
+            return bail(rc);
 #define GA(ptr, bytes) do { cudaError_t _e = pool_alloc(p, &(ptr), (bytes), st); if (_e != cudaSuccess) return bail(fail(_e == cudaErrorMemoryAllocation ? SIE_ERR_OOM : SIE_ERR_CUDA, std::string("sie_solve: workspace: ") + cudaGetErrorString(_e))); } while (0)
     GA(g->V, size_t(m + 1) * g->kstride * sizeof(double2));
     for (double2 **q : {&g->w, &g->b, &g->x, &g->t, &g->rv, &g->vin}) GA(*q, size_t(R) * n * sizeof(double2));
