@@ -55,15 +55,18 @@ template <typename V> __host__ __device__ __forceinline__ V cmulc(V a, V b) {
 }
 // Double-float a c + b d, a fused product sum: both high products exact (FMA
 // two-product), one two-sum of them, every error and cross product in the low
-// part, unnormalised as the sums above.  16 FP32 operations against 27 for two
-// normalised products and a normalised sum.
+// part, then one normalisation (without it the product's error against FP64 can
+// exceed that of separately rounded products: 1.1e-14 against 9e-15 on the bar).
+// 19 FP32 operations against 27 for two normalised products and a normalised sum.
 __host__ __device__ __forceinline__ df df_dot2(df a, df c, df b, df d) {
     const float p = a.hi * c.hi, q = b.hi * d.hi;
     const float s = p + q, bb = s - p;
     float l = fmaf(a.hi, c.hi, -p) + fmaf(b.hi, d.hi, -q);
     l += (p - (s - bb)) + (q - bb);
     l = fmaf(a.hi, c.lo, fmaf(a.lo, c.hi, l));
-    return df(s, fmaf(b.hi, d.lo, fmaf(b.lo, d.hi, l)));
+    l = fmaf(b.hi, d.lo, fmaf(b.lo, d.hi, l));
+    const float h = s + l;
+    return df(h, l - (h - s));
 }
 template <> __host__ __device__ __forceinline__ cdf cmul<cdf>(cdf a, cdf b) {
     return cdf{df_dot2(a.x, b.x, a.y, -b.y), df_dot2(a.x, b.y, a.y, b.x)};
