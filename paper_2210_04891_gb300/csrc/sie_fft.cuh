@@ -601,19 +601,20 @@ template <int N1, int N2> struct Pencil {
 
 // ---- x pencils.  Buffers [batch][rows][ncols], row x at x * ncols; one CTA
 // per (batch, KT consecutive columns), KT * max(N1, N2) threads, a shared
-// line per column (pitch M + 1).  The same kernels run the y pencils of
-// grids whose (y, z) plane does not fit one CTA (batch = grid and
-// x-frequency, rows = y, columns = z).
+// line per column (pitch M + 1).  list: the column tiles to transform (of
+// `tiles`), NULL for all.  The same kernels run the y pencils of grids whose
+// (y, z) plane does not fit one CTA (batch = grid and x-frequency, rows = y,
+// columns = z).
 
 // Forward: in [batch][M/2][ncols] (zero-padded to M) -> out [batch][M][ncols].
 template <typename T, int N1, int N2>
 __global__ void __launch_bounds__(256) k_fft_xf(const C<T> *__restrict__ in, C<T> *__restrict__ out, int ncols,
-                                                const C<T> *__restrict__ tf) {
+                                                const C<T> *__restrict__ tf, const int32_t *__restrict__ list,
+                                                int tiles) {
     constexpr int KT = Pencil<N1, N2>::KT, M = N1 * N2, pitch = M + 1, H1 = N1 / 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C<T> *S = reinterpret_cast<C<T> *>(smem_raw);
-    const int tiles = ncols / KT;
-    const int b = blockIdx.x / tiles, c0 = (blockIdx.x % tiles) * KT;
+    const int b = blockIdx.x / tiles, tile = blockIdx.x - b * tiles, c0 = (list ? list[tile] : tile) * KT;
     const int line = threadIdx.x & (KT - 1), q = threadIdx.x >> Pencil<N1, N2>::LGKT;
     C<T> *Sl = S + line * pitch;
     const int64_t stride = int64_t(N2) * ncols;
@@ -642,12 +643,12 @@ __global__ void __launch_bounds__(256) k_fft_xf(const C<T> *__restrict__ in, C<T
 // Inverse: in [batch][M][ncols] -> out [batch][M/2][ncols] (rows x < M/2 kept).
 template <typename T, int N1, int N2>
 __global__ void __launch_bounds__(256) k_fft_xi(const C<T> *__restrict__ in, C<T> *__restrict__ out, int ncols,
-                                                const C<T> *__restrict__ ti) {
+                                                const C<T> *__restrict__ ti, const int32_t *__restrict__ list,
+                                                int tiles) {
     constexpr int KT = Pencil<N1, N2>::KT, M = N1 * N2, pitch = M + 1, H1 = N1 / 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C<T> *S = reinterpret_cast<C<T> *>(smem_raw);
-    const int tiles = ncols / KT;
-    const int b = blockIdx.x / tiles, c0 = (blockIdx.x % tiles) * KT;
+    const int b = blockIdx.x / tiles, tile = blockIdx.x - b * tiles, c0 = (list ? list[tile] : tile) * KT;
     const int line = threadIdx.x & (KT - 1), q = threadIdx.x >> Pencil<N1, N2>::LGKT;
     C<T> *Sl = S + line * pitch;
     C<T> v[Pencil<N1, N2>::NM];
@@ -772,14 +773,20 @@ __global__ void __launch_bounds__(256) k_fft_rows(C<T> *__restrict__ buf, int M,
 }
 
 // ---- (y, z) plane passes with compile-time split (see k_fft_yzc).  The
-// input extent is half of each padded length (Ny = My/2, Nz = Mz/2).
+// input extent is half of each padded length (Ny = My/2, Nz = Mz/2).  The z
+// passes run over the rows that hold data (Rows); F1 clears the others in Q for F3.
+struct Rows {
+    const uint8_t *list;   // shared memory, ascending
+    int n;
+    __device__ __forceinline__ int row(int i) const { return list[i]; }
+};
 template <typename T, int N1, int N2>   // F1: z pass 1, rows y < Ny, global -> P row slots
-__device__ __forceinline__ void yz_f1(const C<T> *in, C<T> *P, int pitch, int Ny, const C<T> *tfz) {
+__device__ __forceinline__ void yz_f1(const C<T> *in, C<T> *P, int pitch, const Rows rw, const C<T> *tfz) {
     constexpr int Mz = N1 * N2, Nz = Mz / 2, H1 = N1 / 2;
     constexpr int LG2 = N2 == 2 ? 1 : N2 == 4 ? 2 : N2 == 8 ? 3 : 4;
     C<T> v[FFT_NMAX];
-    for (int it = threadIdx.x; it < Ny * N2; it += blockDim.x) {
-        const int y = it >> LG2, j2 = it & (N2 - 1);
+    for (int it = threadIdx.x; it < rw.n * N2; it += blockDim.x) {
+        const int y = rw.row(it >> LG2), j2 = it & (N2 - 1);
         const C<T> *src = in + y * Nz + j2;
 #pragma unroll
         for (int j1 = 0; j1 < H1; ++j1) v[j1] = src[N2 * j1];
@@ -790,11 +797,10 @@ __device__ __forceinline__ void yz_f1(const C<T> *in, C<T> *P, int pitch, int Ny
     }
 }
 template <typename T, int N1, int N2>   // F2: z pass 2, P row slots -> Q natural rows
-__device__ __forceinline__ void yz_f2(const C<T> *P, C<T> *Q, int pitch, int lgNy, const C<T> *tfz) {
+__device__ __forceinline__ void yz_f2(const C<T> *P, C<T> *Q, int pitch, const Rows rw, const C<T> *tfz) {
     C<T> v[FFT_NMAX];
-    const int Ny = 1 << lgNy;
-    for (int it = threadIdx.x; it < Ny * N1; it += blockDim.x) {
-        const int y = it & (Ny - 1), k1 = it >> lgNy;
+    for (int it = threadIdx.x; it < rw.n * N1; it += blockDim.x) {
+        const int k1 = it / rw.n, y = rw.row(it - k1 * rw.n);
         const C<T> *row = P + y * pitch + k1 * N2;
 #pragma unroll
         for (int j2 = 0; j2 < N2; ++j2) v[j2] = row[j2];
@@ -840,11 +846,10 @@ __device__ __forceinline__ void yz_i2(const C<T> *P, C<T> *Q, int pitch, int lgM
 // run over p2 with k1 fixed per load, read consecutive slots: both passes hit
 // distinct shared-memory banks.
 template <typename T, int N1, int N2>   // I3: z inverse pass A, Q rows -> P row slots
-__device__ __forceinline__ void yz_i3(const C<T> *Q, C<T> *P, int pitch, int lgNy, const C<T> *tiz) {
+__device__ __forceinline__ void yz_i3(const C<T> *Q, C<T> *P, int pitch, const Rows rw, const C<T> *tiz) {
     C<T> v[FFT_NMAX];
-    const int Ny = 1 << lgNy;
-    for (int it = threadIdx.x; it < Ny * N1; it += blockDim.x) {
-        const int y = it & (Ny - 1), k1 = it >> lgNy;
+    for (int it = threadIdx.x; it < rw.n * N1; it += blockDim.x) {
+        const int k1 = it / rw.n, y = rw.row(it - k1 * rw.n);
         const C<T> *src = Q + y * pitch + k1;
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) v[k2] = src[N1 * k2];
@@ -855,12 +860,12 @@ __device__ __forceinline__ void yz_i3(const C<T> *Q, C<T> *P, int pitch, int lgN
     }
 }
 template <typename T, int N1, int N2>   // I4: z inverse pass B, P row slots -> global, z < Nz
-__device__ __forceinline__ void yz_i4(const C<T> *P, C<T> *out, int pitch, int Ny, const C<T> *tiz) {
+__device__ __forceinline__ void yz_i4(const C<T> *P, C<T> *out, int pitch, const Rows rw, const C<T> *tiz) {
     constexpr int Mz = N1 * N2, Nz = Mz / 2, H1 = N1 / 2;
     constexpr int LG2 = N2 == 2 ? 1 : N2 == 4 ? 2 : N2 == 8 ? 3 : 4;
     C<T> v[FFT_NMAX];
-    for (int it = threadIdx.x; it < Ny * N2; it += blockDim.x) {
-        const int y = it >> LG2, p2 = it & (N2 - 1);
+    for (int it = threadIdx.x; it < rw.n * N2; it += blockDim.x) {
+        const int y = rw.row(it >> LG2), p2 = it & (N2 - 1);
         const C<T> *src = P + y * pitch + p2;
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) v[k1] = src[k1 * N2];
@@ -928,15 +933,24 @@ __device__ __forceinline__ void yz_mid(C<T> *P, int pitch, int lgMz, const HT *_
 // Hp: kernel spectrum [fold(kx)][fold(ky)][fold(kz)], scaled by 1/(Mx My Mz):
 // real (HT = T, the static kernel) or complex (HT = C<T>, the lossy kernel).
 // Htab / gslot: as in k_fft_zconv (grid g = blockIdx.x / Mx uses Htab[gslot[g]]).
+// rows: bit mask of the rows y < Ny that hold data and are wanted (the others are
+// not written).
 template <typename T, int NT, typename HT>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_fft_yzc(C<T> *__restrict__ buf, int lgMx, int My, int Mz,
                                                  const HT *__restrict__ Hp, const C<T> *__restrict__ tfy,
                                                  const C<T> *__restrict__ tiy, const C<T> *__restrict__ tfz,
                                                  const C<T> *__restrict__ tiz, const HT *const *__restrict__ Htab,
-                                                 const int32_t *__restrict__ gslot) {
+                                                 const int32_t *__restrict__ gslot, ulonglong2 rows) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint8_t s_rows[128];
     const int pitch = Mz + 1, Ny = My / 2, Nz = Mz / 2;
-    const int lgNy = ilog2(Ny), lgMz = ilog2(Mz);
+    const int lgMz = ilog2(Mz);
+    const Rows rw{s_rows, __popcll(rows.x) + __popcll(rows.y)};
+    for (int y = threadIdx.x; y < Ny; y += NT) {
+        const uint64_t below = y < 64 ? rows.x : rows.y, bit = 1ull << (y & 63);
+        if (below & bit) s_rows[(y < 64 ? 0 : __popcll(rows.x)) + __popcll(below & (bit - 1))] = uint8_t(y);
+    }
+    __syncthreads();
     const int Mx = 1 << lgMx;
     const int kx = blockIdx.x & (Mx - 1);
     C<T> *P = reinterpret_cast<C<T> *>(smem_raw);
@@ -944,18 +958,23 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_fft_yzc(C<T> *__
     C<T> *plane = buf + int64_t(blockIdx.x) * Ny * Nz;
     const HT *Hg = Htab ? Htab[gslot[blockIdx.x >> lgMx]] : Hp;
     const HT *Hk = Hg + int64_t(fold_index(kx, Mx)) * (My / 2 + 1) * (Mz / 2 + 1);
-    SIE_SPLIT_DISPATCH(Mz, (yz_f1<T, N1, N2>(plane, P, pitch, Ny, tfz)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_f1<T, N1, N2>(plane, P, pitch, rw, tfz)));
+    if (rw.n < Ny)
+        for (int i = threadIdx.x; i < Ny * Mz; i += NT) {
+            const int y = i >> lgMz;
+            if (!(((y < 64 ? rows.x : rows.y) >> (y & 63)) & 1)) Qb[y * pitch + (i & (Mz - 1))] = mk<T>(T(0.0), T(0.0));
+        }
     __syncthreads();
-    SIE_SPLIT_DISPATCH(Mz, (yz_f2<T, N1, N2>(P, Qb, pitch, lgNy, tfz)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_f2<T, N1, N2>(P, Qb, pitch, rw, tfz)));
     __syncthreads();
     SIE_SPLIT_DISPATCH(My, (yz_f3<T, N1, N2>(Qb, P, pitch, lgMz, tfy)));
     __syncthreads();
     SIE_SPLIT_DISPATCH(My, (yz_mid<T, N1, N2, HT>(P, pitch, lgMz, Hk, tfy, tiy)));
     SIE_SPLIT_DISPATCH(My, (yz_i2<T, N1, N2>(P, Qb, pitch, lgMz, tiy)));
     __syncthreads();
-    SIE_SPLIT_DISPATCH(Mz, (yz_i3<T, N1, N2>(Qb, P, pitch, lgNy, tiz)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_i3<T, N1, N2>(Qb, P, pitch, rw, tiz)));
     __syncthreads();
-    SIE_SPLIT_DISPATCH(Mz, (yz_i4<T, N1, N2>(P, plane, pitch, Ny, tiz)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_i4<T, N1, N2>(P, plane, pitch, rw, tiz)));
 }
 
 }  // namespace sie

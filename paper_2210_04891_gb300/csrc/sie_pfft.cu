@@ -1523,7 +1523,7 @@ int matvec_t(pfft_plan *p, const double2 *x, double2 *y, int32_t R, int space, c
     tm.reset();
     const int prec = is_df<T> ? SIE_PREC_DF : is_f64<T> ? SIE_PREC_FP64 : SIE_PREC_MIXED;
     const bool lossy = !is_df<T> && p->params.kernel == SIE_KERNEL_LOSSY;
-    rc = fft_conv(p, s.grid, s.spec, R, prec, st, lossy ? lossy_sel(p, prec) : nullptr);
+    rc = fft_conv(p, s.grid, s.spec, R, prec, st, lossy ? lossy_sel(p, prec) : nullptr, true);
     if (rc) return rc;
     tm.reset(new StageTimer(p, SIE_STAGE_INTERP, st));
     if (small) {

@@ -502,27 +502,29 @@ template <> struct Tables<df> {   // the double-float product: static kernel onl
 // plane route, ncols = N_z per (grid, x-frequency)) for `nbatch` batches.
 template <typename T, int N1, int N2>
 int launch_pencils(pfft_plan *p, const C<T> *in, C<T> *out, int64_t nbatch, int ncols, int axis, bool inverse,
-                   cudaStream_t s) {
+                   cudaStream_t s, bool active = false) {
     using Tb = Tables<T>;
     using Pc = Pencil<N1, N2>;
     const size_t pb = size_t(Pc::KT) * (N1 * N2 + 1) * sizeof(C<T>);
-    const int64_t ctas = nbatch * (ncols / Pc::KT);
+    const int32_t *list = active ? p->d_xtiles : nullptr;
+    const int tiles = list ? p->n_xtiles : ncols / Pc::KT;
+    const int64_t ctas = nbatch * tiles;
     if (ncols % Pc::KT || ctas > INT32_MAX) return fail(SIE_ERR_ARG, "pencil FFT: unsupported shape");
     if (!inverse) {
         int rc = set_smem((const void *)k_fft_xf<T, N1, N2>, pb);
         if (rc) return rc;
-        k_fft_xf<T, N1, N2><<<unsigned(ctas), Pc::threads, pb, s>>>(in, out, ncols, Tb::tf(p, axis));
+        k_fft_xf<T, N1, N2><<<unsigned(ctas), Pc::threads, pb, s>>>(in, out, ncols, Tb::tf(p, axis), list, tiles);
     } else {
         int rc = set_smem((const void *)k_fft_xi<T, N1, N2>, pb);
         if (rc) return rc;
-        k_fft_xi<T, N1, N2><<<unsigned(ctas), Pc::threads, pb, s>>>(in, out, ncols, Tb::ti(p, axis));
+        k_fft_xi<T, N1, N2><<<unsigned(ctas), Pc::threads, pb, s>>>(in, out, ncols, Tb::ti(p, axis), list, tiles);
     }
     return SIE_OK;
 }
 
 template <typename T, int N1, int N2>
-int launch_x(pfft_plan *p, const C<T> *in, C<T> *out, int ngrids, bool inverse, cudaStream_t s) {
-    return launch_pencils<T, N1, N2>(p, in, out, ngrids, p->Ny * p->Nz, 0, inverse, s);
+int launch_x(pfft_plan *p, const C<T> *in, C<T> *out, int ngrids, bool inverse, cudaStream_t s, bool active) {
+    return launch_pencils<T, N1, N2>(p, in, out, ngrids, p->Ny * p->Nz, 0, inverse, s, active);
 }
 
 // z rows of the large plane route: forward, kernel product, inverse, in place.
@@ -565,13 +567,13 @@ int launch_yz_large(pfft_plan *p, C<T> *spec, int32_t ngrids, const HT *Hp, cons
 }
 
 template <typename T, typename HT>
-int launch_yzc(pfft_plan *p, C<T> *spec, int32_t ngrids, const HT *Hp, cudaStream_t s,
+int launch_yzc(pfft_plan *p, C<T> *spec, int32_t ngrids, const HT *Hp, bool active, cudaStream_t s,
                const HT *const *Htab = nullptr, const int32_t *gslot = nullptr) {
     using Tb = Tables<T>;
     if (p->large_plane) return launch_yz_large<T, HT>(p, spec, ngrids, Hp, Htab, gslot, s);
     if constexpr (sizeof(T) == 4 && sizeof(HT) == sizeof(T)) {   // static kernel in FP32: paired form
         bool done = false;
-        const int rc = plane_conv_f32(p, spec, ngrids, s, done);
+        const int rc = plane_conv_f32(p, spec, ngrids, active, s, done);
         if (rc || done) return rc;
     }
     const size_t plane_bytes = size_t(p->My + p->Ny) * (p->Mz + 1) * sizeof(C<T>);
@@ -579,11 +581,15 @@ int launch_yzc(pfft_plan *p, C<T> *spec, int32_t ngrids, const HT *Hp, cudaStrea
     while ((1 << lgMx) < p->Mx) ++lgMx;
     split4(p->My, n1y, n2y);
     split4(p->Mz, n1z, n2z);
+    ulonglong2 rows = make_ulonglong2(~0ull, ~0ull);   // every row of N_y <= 128
+    if (p->Ny < 64) rows.x = (1ull << p->Ny) - 1;
+    if (p->Ny < 128) rows.y = p->Ny > 64 ? (1ull << (p->Ny - 64)) - 1 : 0;
+    if (active) rows = make_ulonglong2(p->act_rows[0], p->act_rows[1]);
     auto launch = [&](auto nt) -> int {
         constexpr int NT = decltype(nt)::value;
         if (int rc = set_smem((const void *)k_fft_yzc<T, NT, HT>, plane_bytes)) return rc;
         k_fft_yzc<T, NT, HT><<<unsigned(ngrids * p->Mx), NT, plane_bytes, s>>>(
-            spec, lgMx, p->My, p->Mz, Hp, Tb::tf(p, 1), Tb::ti(p, 1), Tb::tf(p, 2), Tb::ti(p, 2), Htab, gslot);
+            spec, lgMx, p->My, p->Mz, Hp, Tb::tf(p, 1), Tb::ti(p, 1), Tb::tf(p, 2), Tb::ti(p, 2), Htab, gslot, rows);
         SIE_LAUNCH_CHECK(p);
         return SIE_OK;
     };
@@ -602,45 +608,49 @@ int launch_yzc(pfft_plan *p, C<T> *spec, int32_t ngrids, const HT *Hp, cudaStrea
 
 template <typename T>
 int fft_conv_t(pfft_plan *p, C<T> *grid, C<T> *spec, int32_t ngrids, cudaStream_t s, bool lossy,
-               const SpecSel *sel) {
+               const SpecSel *sel, bool active) {
     using Tb = Tables<T>;
+    active = active && p->d_xtiles;
     int rc;
     {
         StageTimer tm(p, SIE_STAGE_FFT_X_FWD, s);
-        SIE_SPLIT_DISPATCH_P(p->Mx, (rc = launch_x<T, N1, N2>(p, grid, spec, ngrids, false, s)));
+        SIE_SPLIT_DISPATCH_P(p->Mx, (rc = launch_x<T, N1, N2>(p, grid, spec, ngrids, false, s, active)));
         if (rc) return rc;
         SIE_LAUNCH_CHECK(p);
     }
     {
         StageTimer tm(p, SIE_STAGE_FFT_YZ, s);
         if constexpr (std::is_same<T, df>::value)
-            rc = launch_yzc<T>(p, spec, ngrids, Tb::Hp(p), s);
+            rc = launch_yzc<T>(p, spec, ngrids, Tb::Hp(p), active, s);
         else if (sel && sel->tab)   // one lossy spectrum per grid
-            rc = launch_yzc<T, C<T>>(p, spec, ngrids, nullptr, s, reinterpret_cast<const C<T> *const *>(sel->tab),
+            rc = launch_yzc<T, C<T>>(p, spec, ngrids, nullptr, active, s, reinterpret_cast<const C<T> *const *>(sel->tab),
                                      sel->gslot);
         else
-            rc = lossy ? launch_yzc<T>(p, spec, ngrids, Tb::Hl(p), s) : launch_yzc<T>(p, spec, ngrids, Tb::Hp(p), s);
+            rc = lossy ? launch_yzc<T>(p, spec, ngrids, Tb::Hl(p), active, s)
+                   : launch_yzc<T>(p, spec, ngrids, Tb::Hp(p), active, s);
         if (rc) return rc;
     }
     StageTimer tm(p, SIE_STAGE_FFT_X_INV, s);
-    SIE_SPLIT_DISPATCH_P(p->Mx, (rc = launch_x<T, N1, N2>(p, spec, grid, ngrids, true, s)));
+    SIE_SPLIT_DISPATCH_P(p->Mx, (rc = launch_x<T, N1, N2>(p, spec, grid, ngrids, true, s, active)));
     if (rc) return rc;
     SIE_LAUNCH_CHECK(p);
     return SIE_OK;
 }
 
 int fft_conv_n(pfft_plan *p, void *grid, void *spec, int32_t ngrids, int prec, cudaStream_t s, bool lossy,
-               const SpecSel *sel) {
-    if (prec == SIE_PREC_FP64) return fft_conv_t<double>(p, (double2 *)grid, (double2 *)spec, ngrids, s, lossy, sel);
+               const SpecSel *sel, bool active) {
+    if (prec == SIE_PREC_FP64)
+        return fft_conv_t<double>(p, (double2 *)grid, (double2 *)spec, ngrids, s, lossy, sel, active);
     if (prec == SIE_PREC_DF) {
         if (lossy || !p->df_ready) return fail(SIE_ERR_ARG, "double-float convolution: static kernel, tables built");
-        return fft_conv_t<df>(p, (cdf *)grid, (cdf *)spec, ngrids, s, false, nullptr);
+        return fft_conv_t<df>(p, (cdf *)grid, (cdf *)spec, ngrids, s, false, nullptr, active);
     }
-    return fft_conv_t<float>(p, (float2 *)grid, (float2 *)spec, ngrids, s, lossy, sel);
+    return fft_conv_t<float>(p, (float2 *)grid, (float2 *)spec, ngrids, s, lossy, sel, active);
 }
 
-int fft_conv(pfft_plan *p, void *grid, void *spec, int32_t nrhs, int prec, cudaStream_t s, const SpecSel *sel) {
-    return fft_conv_n(p, grid, spec, 3 * nrhs, prec, s, sel != nullptr, sel);
+int fft_conv(pfft_plan *p, void *grid, void *spec, int32_t nrhs, int prec, cudaStream_t s, const SpecSel *sel,
+             bool active) {
+    return fft_conv_n(p, grid, spec, 3 * nrhs, prec, s, sel != nullptr, sel, active);
 }
 
 // Reads and clears the plan's device error flags (call after the work that
@@ -1008,6 +1018,26 @@ extern "C" int pfft_plan_create(const sie_mesh *m, const sie_loops *L, const pff
     UP(p->d_pt_rec64, pt_rec64);
     UP(p->d_pt_rec32, pt_rec32);
     UP(p->d_tiles, tiles);
+    if (!p->large_plane && p->Ny >= kActiveMinRows && p->Ny <= 128) {
+        for (int64_t n = 0; n < p->Ng; ++n)
+            if (pn_ptr[n + 1] > pn_ptr[n]) {
+                const int y = int(n / p->Nz % p->Ny) & ~1;
+                p->act_rows[y >> 6] |= 3ull << (y & 63);
+            }
+        int rows = 0;
+        for (int y = 0; y < p->Ny; ++y) rows += p->row_active(y);
+        if (8 * rows <= 7 * p->Ny) {
+            const int KT = p->Mx > 256 ? 8 : 16;   // Pencil<N1, N2>::KT of the x axis
+            std::vector<int32_t> xt;
+            for (int t = 0; t < p->Ny * p->Nz / KT; ++t) {
+                bool any = false;
+                for (int c = t * KT; c < (t + 1) * KT && !any; ++c) any = p->row_active(c / p->Nz);
+                if (any) xt.push_back(t);
+            }
+            p->n_xtiles = int32_t(xt.size());
+            UP(p->d_xtiles, xt);
+        }
+    }
     if (p->n_pchunk > 0) {
         UP(p->d_pch_node_ptr, pch_node_ptr);
         UP(p->d_pch_nodes, pch_nodes);

@@ -24,6 +24,10 @@ constexpr int kChunkRhs = 32;
 // a warp).  Their dense operands are float4 [row][2R], the three components of
 // a real column side by side, so that a lane reads its operand in one load.
 constexpr int kSmallRhs = 16;
+// The matvec's convolution skips grid rows without stencil nodes when the plane has
+// at least this many rows (and fits one CTA) and an eighth of its row pairs is empty:
+// below, a pass is a single round of a few warps either way.
+constexpr int kActiveMinRows = 32;
 // slot_link code of a node with several links (codes of single links are below it)
 constexpr int32_t kManyLinks = 1 << 30;
 // Tour slots of one CTA of the prefix sums, and values a CTA leaves for the
@@ -117,6 +121,13 @@ struct pfft_plan {
     int32_t *d_pch_tri_ptr = nullptr;   // [n_pchunk + 1] into d_pch_tri
     int32_t *d_pch_tri = nullptr;       // triangles of each chunk
     uint16_t *d_pn_lcol = nullptr;      // [n_pair] per node record: index of its triangle in the chunk
+    // y rows (over all x) that hold a stencil node, in pairs (2m, 2m + 1), where skipping
+    // the others pays (kActiveMinRows), and the x-pencil tiles of Pencil<Mx>::KT columns
+    // over them; d_xtiles NULL: every row is transformed
+    uint64_t act_rows[2] = {0, 0};
+    bool row_active(int y) const { return (act_rows[y >> 6] >> (y & 63)) & 1; }
+    int32_t n_xtiles = 0;
+    int32_t *d_xtiles = nullptr;
     int64_t n_tiles = 0;                // 32-node tiles that hold at least one stencil node
     int32_t *d_tiles = nullptr;         // [n_tiles] tile index n / 32, ascending
     // near field CSR over triangles (row T: near T', ascending), 3x3 blocks
@@ -255,17 +266,19 @@ struct SpecSel {
     const void *const *tab = nullptr;
     const int32_t *gslot = nullptr;
 };
+// active: the grids are zero, and their results are not wanted, outside the plan's
+// active rows (the matvec's); the other rows of the results are then not written.
 int fft_conv(pfft_plan *p, void *grid, void *spec, int32_t nrhs, int prec, cudaStream_t s,
-             const SpecSel *sel = nullptr);
+             const SpecSel *sel = nullptr, bool active = false);
 int fft_conv_n(pfft_plan *p, void *grid, void *spec, int32_t ngrids, int prec, cudaStream_t s,
-               bool lossy = false, const SpecSel *sel = nullptr);
+               bool lossy = false, const SpecSel *sel = nullptr, bool active = false);
 int near_mma_prepare(pfft_plan *p, const std::vector<int64_t> &near_ptr, const std::vector<int32_t> &near_col,
                      cudaStream_t s);
 int near_mma_launch(pfft_plan *p, int32_t R, cudaStream_t st);
 // paired FP32 (y, z) plane convolution of ngrids x-transformed grids (static
 // kernel); done = false when the plane size is not one it is built for
 bool plane_conv_supported(const pfft_plan *p);
-int plane_conv_f32(pfft_plan *p, float2 *spec, int32_t ngrids, cudaStream_t s, bool &done);
+int plane_conv_f32(pfft_plan *p, float2 *spec, int32_t ngrids, bool active, cudaStream_t s, bool &done);
 int check_device_errors(pfft_plan *p);
 // Lossy kernel in pfft_matvec (sie_lossy.cu).  lossy_prepare: builds the per-frequency
 // data missing for omega[R] (on stream st, synchronising it when something is built)

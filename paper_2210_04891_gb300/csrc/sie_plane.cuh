@@ -230,6 +230,17 @@ template <int MY, int MZ> struct Geo {
 __device__ __forceinline__ float2 &at2(float *base, int i) { return *reinterpret_cast<float2 *>(base + i); }
 __device__ __forceinline__ float2 ld2(const float *base, int i) { return *reinterpret_cast<const float2 *>(base + i); }
 
+// Row pairs of a plane that hold data (SP): grids projected from a mesh carry
+// currents, and are interpolated from, only in the y rows that its stencils
+// touch.  F1, F2, I3 and I4 skip the other pairs, F3 takes them as zero and I2
+// does not store them.  The lane maps stay (a compact list of pairs loses their
+// distinct banks: 2.42 ms on the bond-wire step, with 40 of 64 rows, against 2.33
+// for all rows).
+struct Pairs {
+    unsigned long long mask;
+    __device__ __forceinline__ bool has(int m) const { return (mask >> m) & 1; }
+};
+
 // Row-pair index of z-pass item u with G = 16 / A2 row pairs per half-warp:
 // the G row pairs of a half-warp are spaced A2 apart so that, at row-pair pitch
 // PZZ = 2 (mod 8), their 64-bit accesses cover distinct banks.
@@ -267,15 +278,15 @@ template <int MY, int MZ> struct F1In {
     static constexpr int kItems = (Geo<MY, MZ>::NYP * Geo<MY, MZ>::A2 + kThreads - 1) / kThreads;
     float2 a[kItems][Geo<MY, MZ>::A1 / 2], b[kItems][Geo<MY, MZ>::A1 / 2];   // rows 2m, 2m + 1
 };
-template <int MY, int MZ>
-__device__ __forceinline__ void f1_load(const float2 *__restrict__ src, F1In<MY, MZ> &in) {
+template <int MY, int MZ, bool SP>
+__device__ __forceinline__ void f1_load(const float2 *__restrict__ src, F1In<MY, MZ> &in, const Pairs &pr) {
     using G = Geo<MY, MZ>;
     constexpr int A2 = G::A2, H1 = G::A1 / 2;
 #pragma unroll
     for (int q = 0; q < F1In<MY, MZ>::kItems; ++q) {
         const int it = threadIdx.x + q * kThreads;
-        if (it < G::NYP * A2) {
-            const int j2 = it % A2, m = zrow<G::NYP, A2>(it / A2);
+        const int j2 = it % A2, m = zrow<G::NYP, A2>(it / A2);
+        if (it < G::NYP * A2 && (!SP || pr.has(m))) {
             const float2 *r0 = src + (2 * m) * G::Nz + j2, *r1 = r0 + G::Nz;
 #pragma unroll
             for (int j1 = 0; j1 < H1; ++j1) {
@@ -285,8 +296,8 @@ __device__ __forceinline__ void f1_load(const float2 *__restrict__ src, F1In<MY,
         }
     }
 }
-template <int MY, int MZ>
-__device__ __forceinline__ void f1(const F1In<MY, MZ> &in, float *Pre, float *Pim, const float2 *tw) {
+template <int MY, int MZ, bool SP>
+__device__ __forceinline__ void f1(const F1In<MY, MZ> &in, float *Pre, float *Pim, const float2 *tw, const Pairs &pr) {
     using G = Geo<MY, MZ>;
     constexpr int A1 = G::A1, A2 = G::A2, H1 = A1 / 2;
 #pragma unroll
@@ -294,6 +305,7 @@ __device__ __forceinline__ void f1(const F1In<MY, MZ> &in, float *Pre, float *Pi
         const int it = threadIdx.x + q * kThreads;
         if (it >= G::NYP * A2) break;
         const int j2 = it % A2, m = zrow<G::NYP, A2>(it / A2);
+        if (SP && !pr.has(m)) continue;
         CP v[16];
 #pragma unroll
         for (int j1 = 0; j1 < H1; ++j1) {
@@ -316,12 +328,13 @@ __device__ __forceinline__ void f1(const F1In<MY, MZ> &in, float *Pre, float *Pi
 }
 
 // F2: z pass 2, P (Lz) -> Q (Lq), natural kz = k1 + A1 k2.
-template <int MY, int MZ>
-__device__ __forceinline__ void f2(const float *Pre, const float *Pim, float *Qre, float *Qim) {
+template <int MY, int MZ, bool SP>
+__device__ __forceinline__ void f2(const float *Pre, const float *Pim, float *Qre, float *Qim, const Pairs &pr) {
     using G = Geo<MY, MZ>;
     constexpr int A1 = G::A1, A2 = G::A2;
     for (int it = threadIdx.x; it < G::NYP * A1; it += kThreads) {
         const int m = it % G::NYP, k1 = it / G::NYP;
+        if (SP && !pr.has(m)) continue;
         CP v[16];
 #pragma unroll
         for (int j2 = 0; j2 < A2; ++j2) {
@@ -340,8 +353,9 @@ __device__ __forceinline__ void f2(const float *Pre, const float *Pim, float *Qr
 }
 
 // F3: y pass 1 of column pairs (2c, 2c + 1), Q (Lq, rows y < Ny) -> P (Ly), row k1 B2 + j2.
-template <int MY, int MZ>
-__device__ __forceinline__ void f3(const float *Qre, const float *Qim, float *Pre, float *Pim, const float2 *tw) {
+template <int MY, int MZ, bool SP>
+__device__ __forceinline__ void f3(const float *Qre, const float *Qim, float *Pre, float *Pim, const float2 *tw,
+                                   const Pairs &pr) {
     using G = Geo<MY, MZ>;
     constexpr int B1 = G::B1, B2 = G::B2, H1 = B1 / 2, NC = MZ / 2;
     for (int it = threadIdx.x; it < NC * B2; it += kThreads) {
@@ -352,7 +366,8 @@ __device__ __forceinline__ void f3(const float *Qre, const float *Qim, float *Pr
         for (int j1 = 0; j1 < H1; ++j1) {
             const int y = j2 + B2 * j1;
             const int i0 = (y >> 1) * G::PZZ + 2 * c + (y & 1), i1 = i0 + MZ;   // kz = 2c, 2c + 1
-            v[j1] = CP{make_float2(Qre[i0], Qre[i1]), make_float2(Qim[i0], Qim[i1])};
+            if (SP && !pr.has(y >> 1)) v[j1] = CP{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            else v[j1] = CP{make_float2(Qre[i0], Qre[i1]), make_float2(Qim[i0], Qim[i1])};
         }
         pdft_zpad<B1>(v);   // rows y >= N_y are the zero padding
 #pragma unroll
@@ -425,8 +440,8 @@ __device__ __forceinline__ void ymid(float *Pre, float *Pim, const float *Hs, co
 
 // I2: inverse y pass B of column pairs, P (Ly, rows p2 B1 + k1) -> Q (Lq, rows
 // y = p2 + B2 p1 < Ny).
-template <int MY, int MZ>
-__device__ __forceinline__ void i2(const float *Pre, const float *Pim, float *Qre, float *Qim) {
+template <int MY, int MZ, bool SP>
+__device__ __forceinline__ void i2(const float *Pre, const float *Pim, float *Qre, float *Qim, const Pairs &pr) {
     using G = Geo<MY, MZ>;
     constexpr int B1 = G::B1, B2 = G::B2, H1 = B1 / 2, NC = MZ / 2;
     for (int it = threadIdx.x; it < NC * B2; it += kThreads) {
@@ -442,6 +457,7 @@ __device__ __forceinline__ void i2(const float *Pre, const float *Pim, float *Qr
 #pragma unroll
         for (int p1 = 0; p1 < H1; ++p1) {
             const int y = p2 + B2 * p1;
+            if (SP && !pr.has(y >> 1)) continue;
             const int i0 = (y >> 1) * G::PZZ + 2 * c + (y & 1), i1 = i0 + MZ;   // kz = 2c, 2c + 1
             Qre[i0] = v[p1].re.x;
             Qre[i1] = v[p1].re.y;
@@ -452,12 +468,14 @@ __device__ __forceinline__ void i2(const float *Pre, const float *Pim, float *Qr
 }
 
 // I3: inverse z pass A of rows y < Ny, Q (Lq, kz = k1 + A1 k2) -> P (Lz), slot p2 + A2 k1.
-template <int MY, int MZ>
-__device__ __forceinline__ void i3(const float *Qre, const float *Qim, float *Pre, float *Pim, const float2 *twi) {
+template <int MY, int MZ, bool SP>
+__device__ __forceinline__ void i3(const float *Qre, const float *Qim, float *Pre, float *Pim, const float2 *twi,
+                                   const Pairs &pr) {
     using G = Geo<MY, MZ>;
     constexpr int A1 = G::A1, A2 = G::A2;
     for (int it = threadIdx.x; it < G::NYP * A1; it += kThreads) {
         const int m = it % G::NYP, k1 = it / G::NYP;
+        if (SP && !pr.has(m)) continue;
         CP v[16];
 #pragma unroll
         for (int k2 = 0; k2 < A2; ++k2) {
@@ -481,12 +499,13 @@ __device__ __forceinline__ void i3(const float *Qre, const float *Qim, float *Pr
 }
 
 // I4: inverse z pass B, P (Lz) -> global rows y < Ny, z = p2 + A2 p1 < Nz.
-template <int MY, int MZ>
-__device__ __forceinline__ void i4(const float *Pre, const float *Pim, float2 *__restrict__ dst) {
+template <int MY, int MZ, bool SP>
+__device__ __forceinline__ void i4(const float *Pre, const float *Pim, float2 *__restrict__ dst, const Pairs &pr) {
     using G = Geo<MY, MZ>;
     constexpr int A1 = G::A1, A2 = G::A2, H1 = A1 / 2;
     for (int it = threadIdx.x; it < G::NYP * A2; it += kThreads) {
         const int p2 = it % A2, m = zrow<G::NYP, A2>(it / A2);
+        if (SP && !pr.has(m)) continue;
         CP v[16];
 #pragma unroll
         for (int k1 = 0; k1 < A1; ++k1) {
@@ -509,13 +528,15 @@ __device__ __forceinline__ void i4(const float *Pre, const float *Pim, float2 *_
 // in shared memory once and serve every plane of the run.
 // Hp: spectrum [fold(kx)][fold(ky)][fold(kz)], scaled by 1/(Mx My Mz);
 // tf[j2 N1 + k1] = W^(j2 k1), ti[k1 N2 + p2] = W^(k1 p2) (applied conjugated)
-// for axis y (tfy, tiy) and z (tfz, tiz).
-template <int MY, int MZ>
+// for axis y (tfy, tiy) and z (tfz, tiz).  SP: only the row pairs of pairs hold
+// data or are wanted (the others are not written).
+template <int MY, int MZ, bool SP>
 __global__ void __launch_bounds__(kThreads, 2)
     k_plane_conv(float2 *__restrict__ buf, int ngrids, int gpc, int lgMx, const float *__restrict__ Hp,
                  const float2 *__restrict__ tfy, const float2 *__restrict__ tiy, const float2 *__restrict__ tfz,
-                 const float2 *__restrict__ tiz) {
+                 const float2 *__restrict__ tiz, unsigned long long pairs) {
     using G = Geo<MY, MZ>;
+    const Pairs pr{pairs};
     extern __shared__ __align__(16) float psm[];
     float *Pre = psm, *Pim = psm + G::NP, *Qre = psm + 2 * G::NP, *Qim = Qre + G::NQ;
     float *Hs = Qim + G::NQ;
@@ -544,23 +565,23 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     const int64_t pstride = int64_t(Mx) * G::Ny * G::Nz;
     F1In<MY, MZ> in;
-    if (b0 < b1) f1_load<MY, MZ>(buf + int64_t(b0) * pstride + int64_t(kx) * G::Ny * G::Nz, in);
+    if (b0 < b1) f1_load<MY, MZ, SP>(buf + int64_t(b0) * pstride + int64_t(kx) * G::Ny * G::Nz, in, pr);
     __syncthreads();
     for (int b = b0; b < b1; ++b) {
         float2 *plane = buf + int64_t(b) * pstride + int64_t(kx) * G::Ny * G::Nz;
-        f1<MY, MZ>(in, Pre, Pim, s_tfz);
+        f1<MY, MZ, SP>(in, Pre, Pim, s_tfz, pr);
         __syncthreads();
-        f2<MY, MZ>(Pre, Pim, Qre, Qim);
+        f2<MY, MZ, SP>(Pre, Pim, Qre, Qim, pr);
         __syncthreads();
-        f3<MY, MZ>(Qre, Qim, Pre, Pim, s_tfy);
+        f3<MY, MZ, SP>(Qre, Qim, Pre, Pim, s_tfy, pr);
         __syncthreads();
         ymid<MY, MZ>(Pre, Pim, Hs, s_tiy);
-        i2<MY, MZ>(Pre, Pim, Qre, Qim);
+        i2<MY, MZ, SP>(Pre, Pim, Qre, Qim, pr);
         __syncthreads();
-        if (b + 1 < b1) f1_load<MY, MZ>(plane + pstride, in);   // next plane, in flight during I3 and I4
-        i3<MY, MZ>(Qre, Qim, Pre, Pim, s_tiz);
+        if (b + 1 < b1) f1_load<MY, MZ, SP>(plane + pstride, in, pr);   // next plane, in flight during I3 and I4
+        i3<MY, MZ, SP>(Qre, Qim, Pre, Pim, s_tiz, pr);
         __syncthreads();
-        i4<MY, MZ>(Pre, Pim, plane);
+        i4<MY, MZ, SP>(Pre, Pim, plane, pr);
         __syncthreads();
     }
 }

@@ -59,3 +59,25 @@ def test_mixed_columns_match_oracle_and_single_right_hand_side(system, R):
 def check(y, ref, tol):
     err = np.linalg.norm(y.cpu().numpy() - ref, axis=1) / np.linalg.norm(ref, axis=1)
     assert err.max() < tol
+
+
+def test_empty_grid_rows_are_skipped_without_a_trace():
+    """Wires far apart leave most y rows of the grid without stencil nodes; the
+    products skip them (32 rows and more) and must not see what another product, here
+    of NaN currents, left in the buffers.  Against the oracle at the parity bars."""
+    m = synth.wire_array_mesh(2, 10e-6, 60e-6, 900e-6, n_sides=6, n_seg=4, jitter=0.1, seed=9)
+    O = build_loops(m)
+    prm = dict(grid=(8, 64, 4), order=2, near_factor=1.0, near_min_diam=2.0, n_touch=8)
+    S = PfftSystem(m, O, PfftParams(**prm))
+    P = api.Plan(api.Mesh.from_synth(m), api.Loops(api.Mesh.from_synth(m), m.ports), dict(prm, h0=0.0))
+    om = 2 * np.pi * np.logspace(8, 9, 20)
+    x = synth.complex_gaussian(O.nl, 20, seed=4)
+    ref = np.stack([S.matvec(x[r], om[r]) for r in range(20)])
+    xt = torch.from_numpy(x).cuda()
+    for prec, tol in ((PREC_FP64, 1e-10), (PREC_DF, 1e-10), (PREC_MIXED, 1e-5)):
+        for R in (1, 20):
+            g = torch.full((3 * R, 8, 64, 4), float("nan"), device="cuda",
+                           dtype=torch.complex64 if prec == PREC_MIXED else torch.complex128)
+            api.pfft_convolve(P, g, PREC_MIXED if prec == PREC_MIXED else PREC_FP64)
+            api.pfft_matvec(P, torch.full_like(xt[:R], float("nan")), om[:R], SPACE_LOOP, prec)
+            check(api.pfft_matvec(P, xt[:R].contiguous(), om[:R], SPACE_LOOP, prec), ref[:R], tol)
