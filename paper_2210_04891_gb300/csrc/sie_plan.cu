@@ -570,7 +570,14 @@ template <typename T, typename HT>
 int launch_yzc(pfft_plan *p, C<T> *spec, int32_t ngrids, const HT *Hp, bool active, cudaStream_t s,
                const HT *const *Htab = nullptr, const int32_t *gslot = nullptr) {
     using Tb = Tables<T>;
-    if (p->large_plane) return launch_yz_large<T, HT>(p, spec, ngrids, Hp, Htab, gslot, s);
+    if (p->large_plane) {
+        if constexpr (sizeof(T) == 4 && sizeof(HT) == sizeof(T)) {
+            bool done = false;
+            const int rc = plane_large_f32(p, spec, ngrids, s, done);
+            if (rc || done) return rc;
+        }
+        return launch_yz_large<T, HT>(p, spec, ngrids, Hp, Htab, gslot, s);
+    }
     if constexpr (sizeof(T) == 4 && sizeof(HT) == sizeof(T)) {   // static kernel in FP32: paired form
         bool done = false;
         const int rc = plane_conv_f32(p, spec, ngrids, active, s, done);

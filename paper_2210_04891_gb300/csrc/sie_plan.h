@@ -279,6 +279,8 @@ int near_mma_launch(pfft_plan *p, int32_t R, cudaStream_t st);
 // kernel); done = false when the plane size is not one it is built for
 bool plane_conv_supported(const pfft_plan *p);
 int plane_conv_f32(pfft_plan *p, float2 *spec, int32_t ngrids, bool active, cudaStream_t s, bool &done);
+// the same for planes larger than one CTA's shared memory (sie_plane_large.cu)
+int plane_large_f32(pfft_plan *p, float2 *spec, int32_t ngrids, cudaStream_t s, bool &done);
 int check_device_errors(pfft_plan *p);
 // Lossy kernel in pfft_matvec (sie_lossy.cu).  lossy_prepare: builds the per-frequency
 // data missing for omega[R] (on stream st, synchronising it when something is built)
