@@ -32,6 +32,21 @@ namespace plane {
 
 constexpr int kThreads = 256;
 
+// A plane is worked on by TP threads (a power of two, 32 .. 256), kThreads / TP
+// planes of one x-frequency side by side in a CTA: Grp is a thread's place in its
+// plane's group and the group's barrier.  (With a CTA per plane a 16 x 16 plane kept
+// 32 of its 256 threads busy: 96 grids of 256 x 8 x 8 took 177 us, 54 in groups.)
+template <int TP> struct Grp {
+    int t, g;   // thread of the group, group
+    __device__ __forceinline__ Grp()
+        : t(TP == kThreads ? threadIdx.x : threadIdx.x % TP), g(TP == kThreads ? 0 : threadIdx.x / TP) {}
+    __device__ __forceinline__ void sync() const {
+        if constexpr (TP == kThreads) __syncthreads();
+        else if constexpr (TP == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;\n" ::"r"(g + 1), "n"(TP) : "memory");
+    }
+};
+
 struct CP {
     float2 re, im;
 };
@@ -222,7 +237,12 @@ template <int MY, int MZ> struct Geo {
     static constexpr int HSP = MZ / 2 + 2;                          // staged spectrum row pitch
     static constexpr int NH = ((MY / 2 + 1) * HSP + 1) / 2 * 2;     // staged spectrum (floats, even)
     static constexpr int NTW = 2 * (MY + MZ);                       // staged twiddles (float2)
-    static constexpr size_t kSmem = size_t(2 * NP + 2 * NQ + NH) * sizeof(float) + size_t(NTW) * sizeof(float2);
+    // threads per plane: its widest pass, a power of two from 32 to 256
+    static constexpr int kWide = cmax(cmax(NYP * A1, NYP * A2), cmax(MZ / 2 * B1, MZ / 2 * B2));
+    static constexpr int TP = kWide <= 32 ? 32 : kWide <= 64 ? 64 : kWide <= 128 ? 128 : kThreads;
+    static constexpr int NG = kThreads / TP;                        // planes side by side in a CTA
+    static constexpr size_t kSmem =
+        size_t(NG * (2 * NP + 2 * NQ) + NH) * sizeof(float) + size_t(NTW) * sizeof(float2);
     static_assert(NYP >= 1 && A1 >= 2 && A2 >= 2 && B1 >= 2 && B2 >= 2 && A2 <= 16 && B2 <= 16, "plane size");
 };
 
@@ -275,16 +295,17 @@ __device__ __forceinline__ void ycol(int it, int &c, int &j) {
 // tw = W_Mz^(j2 k1) stored [k1][j2].  The global loads are split off (f1_load)
 // so that a CTA issues the next plane's loads while it finishes the current one.
 template <int MY, int MZ> struct F1In {
-    static constexpr int kItems = (Geo<MY, MZ>::NYP * Geo<MY, MZ>::A2 + kThreads - 1) / kThreads;
+    static constexpr int kItems = (Geo<MY, MZ>::NYP * Geo<MY, MZ>::A2 + Geo<MY, MZ>::TP - 1) / Geo<MY, MZ>::TP;
     float2 a[kItems][Geo<MY, MZ>::A1 / 2], b[kItems][Geo<MY, MZ>::A1 / 2];   // rows 2m, 2m + 1
 };
 template <int MY, int MZ, bool SP>
-__device__ __forceinline__ void f1_load(const float2 *__restrict__ src, F1In<MY, MZ> &in, const Pairs &pr) {
+__device__ __forceinline__ void f1_load(const float2 *__restrict__ src, F1In<MY, MZ> &in, const Pairs &pr,
+                                        const Grp<Geo<MY, MZ>::TP> gr) {
     using G = Geo<MY, MZ>;
     constexpr int A2 = G::A2, H1 = G::A1 / 2;
 #pragma unroll
     for (int q = 0; q < F1In<MY, MZ>::kItems; ++q) {
-        const int it = threadIdx.x + q * kThreads;
+        const int it = gr.t + q * G::TP;
         const int j2 = it % A2, m = zrow<G::NYP, A2>(it / A2);
         if (it < G::NYP * A2 && (!SP || pr.has(m))) {
             const float2 *r0 = src + (2 * m) * G::Nz + j2, *r1 = r0 + G::Nz;
@@ -297,12 +318,13 @@ __device__ __forceinline__ void f1_load(const float2 *__restrict__ src, F1In<MY,
     }
 }
 template <int MY, int MZ, bool SP>
-__device__ __forceinline__ void f1(const F1In<MY, MZ> &in, float *Pre, float *Pim, const float2 *tw, const Pairs &pr) {
+__device__ __forceinline__ void f1(const F1In<MY, MZ> &in, float *Pre, float *Pim, const float2 *tw, const Pairs &pr,
+                                   const Grp<Geo<MY, MZ>::TP> gr) {
     using G = Geo<MY, MZ>;
     constexpr int A1 = G::A1, A2 = G::A2, H1 = A1 / 2;
 #pragma unroll
     for (int q = 0; q < F1In<MY, MZ>::kItems; ++q) {
-        const int it = threadIdx.x + q * kThreads;
+        const int it = gr.t + q * G::TP;
         if (it >= G::NYP * A2) break;
         const int j2 = it % A2, m = zrow<G::NYP, A2>(it / A2);
         if (SP && !pr.has(m)) continue;
@@ -329,10 +351,11 @@ __device__ __forceinline__ void f1(const F1In<MY, MZ> &in, float *Pre, float *Pi
 
 // F2: z pass 2, P (Lz) -> Q (Lq), natural kz = k1 + A1 k2.
 template <int MY, int MZ, bool SP>
-__device__ __forceinline__ void f2(const float *Pre, const float *Pim, float *Qre, float *Qim, const Pairs &pr) {
+__device__ __forceinline__ void f2(const float *Pre, const float *Pim, float *Qre, float *Qim, const Pairs &pr,
+                                   const Grp<Geo<MY, MZ>::TP> gr) {
     using G = Geo<MY, MZ>;
     constexpr int A1 = G::A1, A2 = G::A2;
-    for (int it = threadIdx.x; it < G::NYP * A1; it += kThreads) {
+    for (int it = gr.t; it < G::NYP * A1; it += G::TP) {
         const int m = it % G::NYP, k1 = it / G::NYP;
         if (SP && !pr.has(m)) continue;
         CP v[16];
@@ -355,10 +378,10 @@ __device__ __forceinline__ void f2(const float *Pre, const float *Pim, float *Qr
 // F3: y pass 1 of column pairs (2c, 2c + 1), Q (Lq, rows y < Ny) -> P (Ly), row k1 B2 + j2.
 template <int MY, int MZ, bool SP>
 __device__ __forceinline__ void f3(const float *Qre, const float *Qim, float *Pre, float *Pim, const float2 *tw,
-                                   const Pairs &pr) {
+                                   const Pairs &pr, const Grp<Geo<MY, MZ>::TP> gr) {
     using G = Geo<MY, MZ>;
     constexpr int B1 = G::B1, B2 = G::B2, H1 = B1 / 2, NC = MZ / 2;
-    for (int it = threadIdx.x; it < NC * B2; it += kThreads) {
+    for (int it = gr.t; it < NC * B2; it += G::TP) {
         int c, j2;
         ycol<NC>(it, c, j2);
         CP v[16];
@@ -396,10 +419,11 @@ __device__ __forceinline__ int hz_slot(int kz) {
     return f + (f == MZ / 2 ? 1 : 0);
 }
 template <int MY, int MZ>
-__device__ __forceinline__ void ymid(float *Pre, float *Pim, const float *Hs, const float2 *twi) {
+__device__ __forceinline__ void ymid(float *Pre, float *Pim, const float *Hs, const float2 *twi,
+                                     const Grp<Geo<MY, MZ>::TP> gr) {
     using G = Geo<MY, MZ>;
-    constexpr int B1 = G::B1, B2 = G::B2, NC = MZ / 2, CW = kThreads / B1;
-    const int k1 = threadIdx.x / CW, cl = threadIdx.x % CW;
+    constexpr int B1 = G::B1, B2 = G::B2, NC = MZ / 2, CW = G::TP / B1;
+    const int k1 = gr.t / CW, cl = gr.t % CW;
     for (int c0 = 0; c0 < NC; c0 += CW) {
         const int c = c0 + cl;
         const bool act = k1 < B1 && c < NC;
@@ -425,7 +449,7 @@ __device__ __forceinline__ void ymid(float *Pre, float *Pim, const float *Hs, co
                 v[p2] = pmulc(v[p2], dup2(w.x), dup2(w.y));
             }
         }
-        __syncthreads();
+        gr.sync();
         if (act) {
 #pragma unroll
             for (int p2 = 0; p2 < B2; ++p2) {
@@ -434,17 +458,18 @@ __device__ __forceinline__ void ymid(float *Pre, float *Pim, const float *Hs, co
                 at2(Pim, i) = v[p2].im;
             }
         }
-        __syncthreads();
+        gr.sync();
     }
 }
 
 // I2: inverse y pass B of column pairs, P (Ly, rows p2 B1 + k1) -> Q (Lq, rows
 // y = p2 + B2 p1 < Ny).
 template <int MY, int MZ, bool SP>
-__device__ __forceinline__ void i2(const float *Pre, const float *Pim, float *Qre, float *Qim, const Pairs &pr) {
+__device__ __forceinline__ void i2(const float *Pre, const float *Pim, float *Qre, float *Qim, const Pairs &pr,
+                                   const Grp<Geo<MY, MZ>::TP> gr) {
     using G = Geo<MY, MZ>;
     constexpr int B1 = G::B1, B2 = G::B2, H1 = B1 / 2, NC = MZ / 2;
-    for (int it = threadIdx.x; it < NC * B2; it += kThreads) {
+    for (int it = gr.t; it < NC * B2; it += G::TP) {
         int c, p2;
         ycol<NC>(it, c, p2);
         CP v[16];
@@ -470,10 +495,10 @@ __device__ __forceinline__ void i2(const float *Pre, const float *Pim, float *Qr
 // I3: inverse z pass A of rows y < Ny, Q (Lq, kz = k1 + A1 k2) -> P (Lz), slot p2 + A2 k1.
 template <int MY, int MZ, bool SP>
 __device__ __forceinline__ void i3(const float *Qre, const float *Qim, float *Pre, float *Pim, const float2 *twi,
-                                   const Pairs &pr) {
+                                   const Pairs &pr, const Grp<Geo<MY, MZ>::TP> gr) {
     using G = Geo<MY, MZ>;
     constexpr int A1 = G::A1, A2 = G::A2;
-    for (int it = threadIdx.x; it < G::NYP * A1; it += kThreads) {
+    for (int it = gr.t; it < G::NYP * A1; it += G::TP) {
         const int m = it % G::NYP, k1 = it / G::NYP;
         if (SP && !pr.has(m)) continue;
         CP v[16];
@@ -500,10 +525,11 @@ __device__ __forceinline__ void i3(const float *Qre, const float *Qim, float *Pr
 
 // I4: inverse z pass B, P (Lz) -> global rows y < Ny, z = p2 + A2 p1 < Nz.
 template <int MY, int MZ, bool SP>
-__device__ __forceinline__ void i4(const float *Pre, const float *Pim, float2 *__restrict__ dst, const Pairs &pr) {
+__device__ __forceinline__ void i4(const float *Pre, const float *Pim, float2 *__restrict__ dst, const Pairs &pr,
+                                   const Grp<Geo<MY, MZ>::TP> gr) {
     using G = Geo<MY, MZ>;
     constexpr int A1 = G::A1, A2 = G::A2, H1 = A1 / 2;
-    for (int it = threadIdx.x; it < G::NYP * A2; it += kThreads) {
+    for (int it = gr.t; it < G::NYP * A2; it += G::TP) {
         const int p2 = it % A2, m = zrow<G::NYP, A2>(it / A2);
         if (SP && !pr.has(m)) continue;
         CP v[16];
@@ -523,23 +549,24 @@ __device__ __forceinline__ void i4(const float *Pre, const float *Pim, float2 *_
 }
 
 // The (y, z) part of the 3-D convolution, in place on planes [Ny][Nz] of the
-// buffer [ngrids][Mx][Ny][Nz] (complex64).  One CTA per (kx, run of up to G
-// grids): the kx slice of the spectrum and the four-step twiddles are staged
-// in shared memory once and serve every plane of the run.
+// buffer [ngrids][Mx][Ny][Nz] (complex64).  One CTA per (kx, run of grids): the
+// kx slice of the spectrum and the four-step twiddles are staged in shared memory
+// once and serve every plane of the run, which the CTA's groups take in turn.
 // Hp: spectrum [fold(kx)][fold(ky)][fold(kz)], scaled by 1/(Mx My Mz);
 // tf[j2 N1 + k1] = W^(j2 k1), ti[k1 N2 + p2] = W^(k1 p2) (applied conjugated)
 // for axis y (tfy, tiy) and z (tfz, tiz).  SP: only the row pairs of pairs hold
 // data or are wanted (the others are not written).
 template <int MY, int MZ, bool SP>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, Geo<MY, MZ>::TP <= 64 ? 4 : 2)
     k_plane_conv(float2 *__restrict__ buf, int ngrids, int gpc, int lgMx, const float *__restrict__ Hp,
                  const float2 *__restrict__ tfy, const float2 *__restrict__ tiy, const float2 *__restrict__ tfz,
                  const float2 *__restrict__ tiz, unsigned long long pairs) {
     using G = Geo<MY, MZ>;
     const Pairs pr{pairs};
     extern __shared__ __align__(16) float psm[];
-    float *Pre = psm, *Pim = psm + G::NP, *Qre = psm + 2 * G::NP, *Qim = Qre + G::NQ;
-    float *Hs = Qim + G::NQ;
+    const Grp<G::TP> gr;
+    float *Pre = psm + gr.g * (2 * G::NP + 2 * G::NQ), *Pim = Pre + G::NP, *Qre = Pim + G::NP, *Qim = Qre + G::NQ;
+    float *Hs = psm + G::NG * (2 * G::NP + 2 * G::NQ);
     float2 *s_tfy = reinterpret_cast<float2 *>(Hs + G::NH), *s_tiy = s_tfy + MY, *s_tfz = s_tiy + MY,
            *s_tiz = s_tfz + MZ;
     const int Mx = 1 << lgMx;
@@ -565,24 +592,26 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     const int64_t pstride = int64_t(Mx) * G::Ny * G::Nz;
     F1In<MY, MZ> in;
-    if (b0 < b1) f1_load<MY, MZ, SP>(buf + int64_t(b0) * pstride + int64_t(kx) * G::Ny * G::Nz, in, pr);
+    if (b0 + gr.g < b1)
+        f1_load<MY, MZ, SP>(buf + int64_t(b0 + gr.g) * pstride + int64_t(kx) * G::Ny * G::Nz, in, pr, gr);
     __syncthreads();
-    for (int b = b0; b < b1; ++b) {
+    for (int b = b0 + gr.g; b < b1; b += G::NG) {   // groups do not wait for one another here
         float2 *plane = buf + int64_t(b) * pstride + int64_t(kx) * G::Ny * G::Nz;
-        f1<MY, MZ, SP>(in, Pre, Pim, s_tfz, pr);
-        __syncthreads();
-        f2<MY, MZ, SP>(Pre, Pim, Qre, Qim, pr);
-        __syncthreads();
-        f3<MY, MZ, SP>(Qre, Qim, Pre, Pim, s_tfy, pr);
-        __syncthreads();
-        ymid<MY, MZ>(Pre, Pim, Hs, s_tiy);
-        i2<MY, MZ, SP>(Pre, Pim, Qre, Qim, pr);
-        __syncthreads();
-        if (b + 1 < b1) f1_load<MY, MZ, SP>(plane + pstride, in, pr);   // next plane, in flight during I3 and I4
-        i3<MY, MZ, SP>(Qre, Qim, Pre, Pim, s_tiz, pr);
-        __syncthreads();
-        i4<MY, MZ, SP>(Pre, Pim, plane, pr);
-        __syncthreads();
+        f1<MY, MZ, SP>(in, Pre, Pim, s_tfz, pr, gr);
+        gr.sync();
+        f2<MY, MZ, SP>(Pre, Pim, Qre, Qim, pr, gr);
+        gr.sync();
+        f3<MY, MZ, SP>(Qre, Qim, Pre, Pim, s_tfy, pr, gr);
+        gr.sync();
+        ymid<MY, MZ>(Pre, Pim, Hs, s_tiy, gr);
+        i2<MY, MZ, SP>(Pre, Pim, Qre, Qim, pr, gr);
+        gr.sync();
+        if (b + G::NG < b1)   // next plane, in flight during I3 and I4
+            f1_load<MY, MZ, SP>(plane + G::NG * pstride, in, pr, gr);
+        i3<MY, MZ, SP>(Qre, Qim, Pre, Pim, s_tiz, pr, gr);
+        gr.sync();
+        i4<MY, MZ, SP>(Pre, Pim, plane, pr, gr);
+        gr.sync();
     }
 }
 
