@@ -1654,13 +1654,20 @@ int pc_blocks_prepare(pfft_plan *p, int32_t R, bool dfl, cudaStream_t st) {
     const int64_t ctas = int64_t(s->nslots) * 2 * s->nchunks;
     if (ctas > INT32_MAX) return SIE_OK;
     const size_t bytes = size_t(ctas) * (s->W + 32) * 32 * sizeof(double2), sm = size_t(3) * 32 * 33 * sizeof(double2);
+    // no memory for them: the stepped sweeps serve
+    const cudaError_t e = dfl ? pool_alloc(p, &s->d_blkdf, bytes, st) : pool_alloc(p, &s->d_blk64, bytes, st);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        s->d_blkdf = dfl ? nullptr : s->d_blkdf;
+        s->d_blk64 = dfl ? s->d_blk64 : nullptr;
+        if (e == cudaErrorMemoryAllocation) return SIE_OK;
+        return fail(SIE_ERR_CUDA, std::string("preconditioner: ") + cudaGetErrorString(e));
+    }
     if (dfl) {
-        SIE_CUDA(pool_alloc(p, &s->d_blkdf, bytes, st));
         if (int rc = set_smem((const void *)k_pc_blocks<df>, sm)) return rc;
         k_pc_blocks<df><<<unsigned(ctas), 256, sm, st>>>(s->d_band, s->d_bandc, s->d_blk_off, s->d_tile_off, nblk,
                                                          s->W, s->nunk, s->nchunks, s->d_blkdf);
     } else {
-        SIE_CUDA(pool_alloc(p, &s->d_blk64, bytes, st));
         if (int rc = set_smem((const void *)k_pc_blocks<double>, sm)) return rc;
         k_pc_blocks<double><<<unsigned(ctas), 256, sm, st>>>(s->d_band, s->d_bandc, s->d_blk_off, s->d_tile_off, nblk,
                                                              s->W, s->nunk, s->nchunks, s->d_blk64);
