@@ -237,10 +237,14 @@ template <int MY, int MZ> struct Geo {
     static constexpr int HSP = MZ / 2 + 2;                          // staged spectrum row pitch
     static constexpr int NH = ((MY / 2 + 1) * HSP + 1) / 2 * 2;     // staged spectrum (floats, even)
     static constexpr int NTW = 2 * (MY + MZ);                       // staged twiddles (float2)
-    // threads per plane: its widest pass, a power of two from 32 to 256
-    static constexpr int kWide = cmax(cmax(NYP * A1, NYP * A2), cmax(MZ / 2 * B1, MZ / 2 * B2));
+    // threads per plane: its widest y pass, or half its widest z pass, to a power of
+    // two from 32 to 256 (256 x 16: 128 threads, two planes side by side, 374 us for 96
+    // grids of 128 x 128 x 8 against 475 with 256, which the y passes half fill)
+    static constexpr int kWide = cmax(NYP * cmax(A1, A2) / 2, MZ / 2 * cmax(B1, B2));
     static constexpr int TP = kWide <= 32 ? 32 : kWide <= 64 ? 64 : kWide <= 128 ? 128 : kThreads;
     static constexpr int NG = kThreads / TP;                        // planes side by side in a CTA
+    // CTAs per SM by registers: four where the short transforms are at most 8 long
+    static constexpr int kCtas = TP <= 64 && cmax(A2, B2) <= 8 ? 4 : 2;
     static constexpr size_t kSmem =
         size_t(NG * (2 * NP + 2 * NQ) + NH) * sizeof(float) + size_t(NTW) * sizeof(float2);
     static_assert(NYP >= 1 && A1 >= 2 && A2 >= 2 && B1 >= 2 && B2 >= 2 && A2 <= 16 && B2 <= 16, "plane size");
@@ -557,7 +561,7 @@ __device__ __forceinline__ void i4(const float *Pre, const float *Pim, float2 *_
 // for axis y (tfy, tiy) and z (tfz, tiz).  SP: only the row pairs of pairs hold
 // data or are wanted (the others are not written).
 template <int MY, int MZ, bool SP>
-__global__ void __launch_bounds__(kThreads, Geo<MY, MZ>::TP <= 64 ? 4 : 2)
+__global__ void __launch_bounds__(kThreads, Geo<MY, MZ>::kCtas)
     k_plane_conv(float2 *__restrict__ buf, int ngrids, int gpc, int lgMx, const float *__restrict__ Hp,
                  const float2 *__restrict__ tfy, const float2 *__restrict__ tiy, const float2 *__restrict__ tfz,
                  const float2 *__restrict__ tiz, unsigned long long pairs) {
