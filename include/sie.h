@@ -243,9 +243,10 @@ int pfft_precond_apply(pfft_plan *p, const void *y, void *z, int32_t nrhs, const
 /* Structure of the preconditioner (built on first use, or by this call): band
  * width W of its banded LDL^T after the reverse Cuthill-McKee ordering (max
  * over blocks), unknowns, and blocks (one per connected group of unknowns).
- * The sweeps take warp-register tiles for W <= 31, one CTA per (right-hand
- * side, block) for 31 < W < 1024 (FP32 in the mixed form), and a one-warp FP64
- * sweep beyond.  Any pointer may be NULL. */
+ * The sweeps take warp-register tiles for W <= 31 (per-chunk matrices for FP64
+ * and double-float with few right-hand sides), one CTA per (right-hand side,
+ * block) for 31 < W < 1024 (FP32 in the mixed form), and a one-warp FP64 sweep
+ * beyond.  Any pointer may be NULL. */
 int pfft_precond_info(pfft_plan *p, int32_t *band_width, int64_t *unknowns, int64_t *blocks);
 
 /* Factorisation route of the preconditioner (Eq. Precond asks for a direct
