@@ -255,6 +255,15 @@ extern "C" int sie_batch_stats(const sie_batch *b, int64_t *captures, int64_t *r
     return SIE_OK;
 }
 
+namespace {
+// Takes back the memory of what only speeds the plans' preconditioners up; false if there is none.
+bool release_spare(sie_batch *b) {
+    bool any = false;
+    for (pfft_plan *p : b->plans) any |= precond_release_spare(p);
+    return any;
+}
+}  // namespace
+
 extern "C" int sie_batch_solve(sie_batch *b, const double *const *freqs, const int32_t *nf,
                                const int32_t *const *ports, const int32_t *np, const sie_solve_opts *opts,
                                sie_c64 *const *Z_out, sie_solve_stats *st_out) {
@@ -280,6 +289,13 @@ extern "C" int sie_batch_solve(sie_batch *b, const double *const *freqs, const i
         });
     }
     for (auto &t : workers) t.join();
+    // out of memory: once more, one plan at a time, without what only speeds the plans up
+    for (size_t i = 0; i < n; ++i)
+        if (rcs[i] == SIE_ERR_OOM && release_spare(b)) {
+            rcs[i] = sie_solve(b->plans[i], freqs[i], nf[i], ports[i], np[i], opts, Z_out[i],
+                               st_out ? &st_out[i] : nullptr);
+            msgs[i] = rcs[i] ? sie_last_error() : "";
+        }
     for (size_t i = 0; i < n; ++i)
         if (rcs[i]) return fail(rcs[i], "sie_batch_solve: plan " + std::to_string(i) + ": " + msgs[i]);
     return SIE_OK;
@@ -383,6 +399,12 @@ extern "C" int sie_batch_solve_graph(sie_batch *b, const double *const *freqs, c
         rcs[i] = gmres_create(b->plans[i], freqs[i], nf[i], ports[i], np[i], opts, b->streams[i], &runs[i]);
         if (rcs[i]) msgs[i] = sie_last_error();
     });
+    // out of memory: once more without what only speeds the plans up
+    for (size_t i = 0; i < n; ++i)
+        if (rcs[i] == SIE_ERR_OOM && release_spare(b)) {
+            rcs[i] = gmres_create(b->plans[i], freqs[i], nf[i], ports[i], np[i], opts, b->streams[i], &runs[i]);
+            msgs[i] = rcs[i] ? sie_last_error() : "";
+        }
     if (int rc = first_error("set-up")) { cleanup(); return rc; }
     std::vector<size_t> live(all);           // runs not finished
     std::vector<int64_t> launches(n, 0);

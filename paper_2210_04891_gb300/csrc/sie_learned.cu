@@ -720,7 +720,7 @@ extern "C" int pfft_branch_probe_target(pfft_plan *p, const void *alpha, int32_t
     }
     double2 *zb = nullptr;
     double *d_zs = nullptr;
-    SIE_CUDA(cudaMalloc(&zb, size_t(k) * p->nb * sizeof(double2)));
+    SIE_CUDA(plan_malloc(p, (void **)&zb, size_t(k) * p->nb * sizeof(double2)));
     if (cudaMalloc(&d_zs, zs.size() * sizeof(double)) != cudaSuccess) {
         cudaFree(zb);
         return fail(SIE_ERR_OOM, "pfft_branch_probe_target: out of device memory");

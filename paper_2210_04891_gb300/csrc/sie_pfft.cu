@@ -1250,7 +1250,7 @@ int scratch_reserve(pfft_plan *p, int32_t nrhs, int prec) {
                          &s.ffar, &s.part};
     for (int i = 0; i < kBufs; ++i) {
         if (!sizes[i]) continue;
-        cudaError_t e = cudaMalloc(dst[i], sizes[i]);
+        cudaError_t e = plan_malloc(p, dst[i], sizes[i]);
         if (e != cudaSuccess) {
             for (int j = 0; j < i; ++j) if (*dst[j]) { cudaFree(*dst[j]); *dst[j] = nullptr; }
             set_error(std::string("scratch allocation failed: ") + cudaGetErrorString(e));
@@ -1697,12 +1697,12 @@ extern "C" int sie_postprocess(pfft_plan *p, const void *x, int32_t nrhs, const 
         if (tmp_v) cudaFree(tmp_v);
     };
     if (!alpha) {
-        if (cudaMalloc((void **)&tmp_a, size_t(R) * nb * sizeof(double2)) != cudaSuccess)
+        if (plan_malloc(p, (void **)&tmp_a, size_t(R) * nb * sizeof(double2)) != cudaSuccess)
             return fail(SIE_ERR_OOM, "sie_postprocess: out of device memory");
         alpha = tmp_a;
     }
     if (phi && !vb) {
-        if (cudaMalloc((void **)&tmp_v, size_t(R) * nb * sizeof(double2)) != cudaSuccess) {
+        if (plan_malloc(p, (void **)&tmp_v, size_t(R) * nb * sizeof(double2)) != cudaSuccess) {
             cleanup();
             return fail(SIE_ERR_OOM, "sie_postprocess: out of device memory");
         }

@@ -29,7 +29,7 @@ namespace sie {
 int plan_alloc(pfft_plan *p, void **ptr, size_t bytes) {
     *ptr = nullptr;
     if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMalloc(ptr, bytes);
+    cudaError_t e = plan_malloc(p, ptr, bytes);
     if (e != cudaSuccess) {
         set_error(std::string("cudaMalloc(") + std::to_string(bytes) + ") failed: " + cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? SIE_ERR_OOM : SIE_ERR_CUDA;

@@ -235,6 +235,12 @@ int plan_alloc(pfft_plan *p, void **ptr, size_t bytes);
 int set_smem(const void *fn, size_t bytes);
 void plan_free(pfft_plan *p, void *ptr);
 void plan_free_precond(pfft_plan *p);
+// Frees the device memory of what only speeds the plan's preconditioner up (the chunk
+// matrices of the narrow band's sweeps); false if it holds none.  Not while a call of
+// the plan is being captured.
+bool precond_release_spare(pfft_plan *p);
+// cudaMalloc for the plan; on failure once more without that memory
+cudaError_t plan_malloc(pfft_plan *p, void **ptr, size_t bytes);
 int scratch_reserve(pfft_plan *p, int32_t nrhs, int prec);
 // Builds the double-float tables of the SIE_PREC_DF product from the FP64 ones
 // on stream st (once per plan; no-op afterwards).

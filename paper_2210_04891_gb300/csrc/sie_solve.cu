@@ -116,7 +116,28 @@ cudaError_t pool_alloc(pfft_plan *p, Ptr **ptr, size_t bytes, cudaStream_t st) {
     cudaMemPool_t pool;
     cudaError_t e = plan_pool(p, &pool);
     if (e != cudaSuccess) return e;
-    return cudaMallocFromPoolAsync((void **)ptr, bytes, pool, st);
+    e = cudaMallocFromPoolAsync((void **)ptr, bytes, pool, st);
+    if (e == cudaErrorMemoryAllocation && precond_release_spare(p)) e = cudaMallocFromPoolAsync((void **)ptr, bytes, pool, st);
+    return e;
+}
+
+bool precond_release_spare(pfft_plan *p) {
+    PrecondState *s = p->pc;
+    if (!s || (!s->d_blk64 && !s->d_blkdf)) return false;
+    (void)cudaGetLastError();
+    cudaDeviceSynchronize();   // no sweep still reads them
+    if (s->d_blk64) cudaFree(s->d_blk64);
+    if (s->d_blkdf) cudaFree(s->d_blkdf);
+    s->d_blk64 = nullptr;
+    s->d_blkdf = nullptr;
+    if (p->pool) cudaMemPoolTrimTo(p->pool, 0);
+    return true;
+}
+
+cudaError_t plan_malloc(pfft_plan *p, void **ptr, size_t bytes) {
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e == cudaErrorMemoryAllocation && precond_release_spare(p)) e = cudaMalloc(ptr, bytes);
+    return e;
 }
 
 // DC (omega = 0) has a solution only when every conductor has a slab surface
@@ -1646,6 +1667,9 @@ int pc_apply_t(pfft_plan *p, const double2 *y, double2 *z, int32_t R, cudaStream
 
 // Chunk matrices for R right-hand sides' sweeps in FP64 or double-float, if the
 // matrix sweeps will serve them; before a capture, on the factors of pc_prepare.
+// They only speed the sweeps up: callers allocate what they cannot do without
+// first, and an allocation that fails later takes their memory back
+// (precond_release_spare), after which the stepped sweeps serve.
 int pc_blocks_prepare(pfft_plan *p, int32_t R, bool dfl, cudaStream_t st) {
     PrecondState *s = p->pc;
     const int32_t nblk = int32_t(s->blk_off.size()) - 1;
@@ -1655,7 +1679,10 @@ int pc_blocks_prepare(pfft_plan *p, int32_t R, bool dfl, cudaStream_t st) {
     if (ctas > INT32_MAX) return SIE_OK;
     const size_t bytes = size_t(ctas) * (s->W + 32) * 32 * sizeof(double2), sm = size_t(3) * 32 * 33 * sizeof(double2);
     // no memory for them: the stepped sweeps serve
-    const cudaError_t e = dfl ? pool_alloc(p, &s->d_blkdf, bytes, st) : pool_alloc(p, &s->d_blk64, bytes, st);
+    cudaMemPool_t pool;
+    cudaError_t e = plan_pool(p, &pool);
+    if (e == cudaSuccess)
+        e = cudaMallocFromPoolAsync(dfl ? (void **)&s->d_blkdf : (void **)&s->d_blk64, bytes, pool, st);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         s->d_blkdf = dfl ? nullptr : s->d_blkdf;
@@ -2034,9 +2061,6 @@ int gmres_create(pfft_plan *p, const double *freqs, int32_t nf, const int32_t *p
     // the tests' P^-1 (b - Z x): FP64, or with refine = 2 on the narrow band route the
     // double-float sweeps (within 1e-11 of FP64, a third of its time)
     g->outer_pc_prec = g->pc_prec == SIE_PREC_DF ? SIE_PREC_DF : g->outer_prec;
-    for (int prec : {g->pc_prec, g->outer_pc_prec})
-        if (g->use_pc && prec != SIE_PREC_MIXED && (rc = pc_blocks_prepare(p, R, prec == SIE_PREC_DF, st)))
-            return bail(rc);
 #define GA(ptr, bytes) do { cudaError_t _e = pool_alloc(p, &(ptr), (bytes), st); if (_e != cudaSuccess) return bail(fail(_e == cudaErrorMemoryAllocation ? SIE_ERR_OOM : SIE_ERR_CUDA, std::string("sie_solve: workspace: ") + cudaGetErrorString(_e))); } while (0)
     GA(g->V, size_t(m + 1) * g->kstride * sizeof(double2));
     for (double2 **q : {&g->w, &g->b, &g->x, &g->t, &g->rv, &g->vin}) GA(*q, size_t(R) * n * sizeof(double2));
@@ -2079,6 +2103,14 @@ int gmres_create(pfft_plan *p, const double *freqs, int32_t nf, const int32_t *p
     g->iters.assign(R, 0);
     g->resid.assign(R, 1.0);
     GC(cudaMemcpyAsync(g->act, g->active.data(), R * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    // the product's coefficients stay in the plan's scratch for the whole solve
+    if ((rc = scratch_reserve(p, R, g->o.prec))) return bail(rc);
+    if ((rc = scratch_reserve(p, R, g->outer_prec))) return bail(rc);
+    if (g->resid_prec == SIE_PREC_DF && (rc = df_prepare(p, st))) return bail(rc);
+    // the chunk matrices last, when everything the solve cannot do without is there
+    for (int prec : {g->pc_prec, g->outer_pc_prec})
+        if (g->use_pc && prec != SIE_PREC_MIXED && (rc = pc_blocks_prepare(p, R, prec == SIE_PREC_DF, st)))
+            return bail(rc);
     // ||P^-1 b|| (the outer precision's preconditioner); r = b - Z x with x = 0
     if (g->use_pc) {
         if ((rc = pc_apply_async(p, g->b, g->w, R, g->outer_pc_prec, st))) return bail(rc);
@@ -2090,10 +2122,6 @@ int gmres_create(pfft_plan *p, const double *freqs, int32_t nf, const int32_t *p
     GC(cudaMemcpyAsync(g->gd.bnorm, g->dnorm, size_t(R) * sizeof(double), cudaMemcpyDeviceToDevice, st));
     GC(cudaMemcpyAsync(g->rv, g->b, size_t(R) * n * sizeof(double2), cudaMemcpyDeviceToDevice, st));
 #undef GC
-    // the product's coefficients stay in the plan's scratch for the whole solve
-    if ((rc = scratch_reserve(p, R, g->o.prec))) return bail(rc);
-    if ((rc = scratch_reserve(p, R, g->outer_prec))) return bail(rc);
-    if (g->resid_prec == SIE_PREC_DF && (rc = df_prepare(p, st))) return bail(rc);
     *out = g;
     return SIE_OK;
 }
