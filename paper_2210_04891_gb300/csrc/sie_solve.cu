@@ -1678,28 +1678,34 @@ int pc_blocks_prepare(pfft_plan *p, int32_t R, bool dfl, cudaStream_t st) {
     const int64_t ctas = int64_t(s->nslots) * 2 * s->nchunks;
     if (ctas > INT32_MAX) return SIE_OK;
     const size_t bytes = size_t(ctas) * (s->W + 32) * 32 * sizeof(double2), sm = size_t(3) * 32 * 33 * sizeof(double2);
-    // no memory for them: the stepped sweeps serve
+    void *blocks = nullptr;
     cudaMemPool_t pool;
     cudaError_t e = plan_pool(p, &pool);
-    if (e == cudaSuccess)
-        e = cudaMallocFromPoolAsync(dfl ? (void **)&s->d_blkdf : (void **)&s->d_blk64, bytes, pool, st);
-    if (e != cudaSuccess) {
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(&blocks, bytes, pool, st);
+    if (e == cudaErrorMemoryAllocation) {   // no memory for them: the stepped sweeps serve
         (void)cudaGetLastError();
-        s->d_blkdf = dfl ? nullptr : s->d_blkdf;
-        s->d_blk64 = dfl ? s->d_blk64 : nullptr;
-        if (e == cudaErrorMemoryAllocation) return SIE_OK;
-        return fail(SIE_ERR_CUDA, std::string("preconditioner: ") + cudaGetErrorString(e));
+        return SIE_OK;
     }
-    if (dfl) {
-        if (int rc = set_smem((const void *)k_pc_blocks<df>, sm)) return rc;
-        k_pc_blocks<df><<<unsigned(ctas), 256, sm, st>>>(s->d_band, s->d_bandc, s->d_blk_off, s->d_tile_off, nblk,
-                                                         s->W, s->nunk, s->nchunks, s->d_blkdf);
-    } else {
-        if (int rc = set_smem((const void *)k_pc_blocks<double>, sm)) return rc;
-        k_pc_blocks<double><<<unsigned(ctas), 256, sm, st>>>(s->d_band, s->d_bandc, s->d_blk_off, s->d_tile_off, nblk,
-                                                             s->W, s->nunk, s->nchunks, s->d_blk64);
+    if (e != cudaSuccess) return fail(SIE_ERR_CUDA, std::string("preconditioner: ") + cudaGetErrorString(e));
+    auto build = [&]() -> int {
+        if (dfl) {
+            if (int rc = set_smem((const void *)k_pc_blocks<df>, sm)) return rc;
+            k_pc_blocks<df><<<unsigned(ctas), 256, sm, st>>>(s->d_band, s->d_bandc, s->d_blk_off, s->d_tile_off, nblk,
+                                                             s->W, s->nunk, s->nchunks, (cdf *)blocks);
+        } else {
+            if (int rc = set_smem((const void *)k_pc_blocks<double>, sm)) return rc;
+            k_pc_blocks<double><<<unsigned(ctas), 256, sm, st>>>(s->d_band, s->d_bandc, s->d_blk_off, s->d_tile_off,
+                                                                 nblk, s->W, s->nunk, s->nchunks, (double2 *)blocks);
+        }
+        SIE_LAUNCH_CHECK(p);
+        return SIE_OK;
+    };
+    if (int rc = build()) {   // not built: no later call may find them
+        cudaFreeAsync(blocks, st);
+        return rc;
     }
-    SIE_LAUNCH_CHECK(p);
+    if (dfl) s->d_blkdf = (cdf *)blocks;
+    else s->d_blk64 = (double2 *)blocks;
     return SIE_OK;
 }
 
