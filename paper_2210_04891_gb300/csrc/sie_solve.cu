@@ -1354,20 +1354,20 @@ int pc_prepare(pfft_plan *p, const double *omega, int32_t R, std::vector<int32_t
     slot.resize(R);
     for (int32_t r = 0; r < R; ++r) slot[r] = int32_t(std::lower_bound(uniq.begin(), uniq.end(), omega[r]) - uniq.begin());
     if (R > s->cap_rhs) {
-        for (void *a : {(void *)s->d_kappa, (void *)s->d_u, (void *)s->d_ibr, (void *)s->d_slot})
+        for (void *a : {(void *)s->d_kappa, (void *)s->d_u, (void *)s->d_ibr, (void *)s->d_slot, (void *)s->d_u32,
+                        (void *)s->d_uv})
             if (a) cudaFreeAsync(a, st);
-        s->d_kappa = s->d_u = s->d_ibr = nullptr;
+        s->d_kappa = s->d_u = s->d_ibr = s->d_uv = nullptr;
+        s->d_u32 = nullptr;
         s->d_slot = nullptr;
+        s->cap_rhs = 0;   // until every buffer below has the new size
         SIE_CUDA(pool_alloc(p, &s->d_kappa, size_t(R) * p->nb * sizeof(double2), st));
         SIE_CUDA(pool_alloc(p, &s->d_ibr, size_t(R) * p->nb * sizeof(double2), st));
         SIE_CUDA(pool_alloc(p, &s->d_u, size_t(R) * std::max<int64_t>(s->nunk, 1) * sizeof(double2), st));
-        if (s->d_u32) cudaFreeAsync(s->d_u32, st);
         SIE_CUDA(pool_alloc(p, &s->d_u32, size_t(R) * std::max<int64_t>(s->nunk, 1) * sizeof(float2), st));
         SIE_CUDA(pool_alloc(p, &s->d_slot, size_t(R) * sizeof(int32_t), st));
-        if (s->nd) {
-            if (s->d_uv) cudaFreeAsync(s->d_uv, st);
+        if (s->nd)
             SIE_CUDA(pool_alloc(p, &s->d_uv, size_t(R) * std::max<int64_t>(nd_update_size(s->nd), 1) * sizeof(double2), st));
-        }
         s->cap_rhs = R;
     }
     SIE_CUDA(cudaMemcpyAsync(s->d_slot, slot.data(), R * sizeof(int32_t), cudaMemcpyHostToDevice, st));

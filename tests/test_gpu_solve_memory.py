@@ -7,12 +7,13 @@ import contextlib
 import numpy as np
 import pytest
 
+import synth
 from synth.meshes import box_mesh
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from paper_2210_04891_gb300 import api, PREC_FP64  # noqa: E402
+from paper_2210_04891_gb300 import api, native, PREC_FP64  # noqa: E402
 
 NF = 64
 FREQS = np.logspace(8.5, 9.5, NF)
@@ -81,6 +82,19 @@ def test_matrices_give_way_to_a_larger_workspace():
     with only(larger - mats // 2):
         Z2, st = solve(P, restart)
     assert st["converged"] and np.abs(Z2 - Z).max() < 1e-5 * np.abs(Z).max()
+
+
+def test_preconditioner_after_a_growth_that_failed():
+    M, L = bar()
+    P = plan(M, L)
+    om = 2 * np.pi * 1e9
+    y = torch.from_numpy(synth.complex_gaussian(L.nl, 2, seed=5)).cuda()
+    z = api.pfft_precond_apply(P, y, om)
+    many = torch.zeros(8000, L.nl, dtype=torch.complex128, device="cuda")
+    out = torch.empty_like(many)
+    with only(200 << 20), pytest.raises(native.SieError):
+        api.pfft_precond_apply(P, many, om, out=out)
+    assert torch.equal(api.pfft_precond_apply(P, y, om), z)
 
 
 def test_batch_solve_gives_the_matrices_back():
