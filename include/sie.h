@@ -232,7 +232,11 @@ int pfft_matvec(pfft_plan *p, const void *x, void *y, int32_t nrhs, const double
  * see pfft_precond_info; wider bands fall back to FP64); SIE_PREC_DF runs them
  * in double-float (factor rounded to FP32 pairs) where the band width is at most
  * 31 and in FP64 otherwise (an FP32 LDL^T solve of the nodal Laplacian, whose
- * condition grows with the mesh, keeps few correct digits).  The factor buffers and
+ * condition grows with the mesh, keeps few correct digits).  In FP64 and
+ * double-float several orders of the same sweeps serve, chosen by the number of
+ * right-hand sides, by how often a set of factors has been applied and by the
+ * memory left: their results agree to rounding (1e-11 of the norm), not bit for
+ * bit.  A solve keeps to one order.  The factor buffers and
  * the sweeps' scratch are stream-ordered allocations on cuda_stream from a
  * plan-owned memory pool.  omega[r] > 0, or 0 when every conductor has
  * a slab surface model (SIE_ERR_ARG otherwise).  Errors: SIE_ERR_BREAKDOWN for

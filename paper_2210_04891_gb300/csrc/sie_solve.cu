@@ -72,6 +72,7 @@ struct PrecondState {
     // pc_blocks_prepare for few chains
     double2 *d_blk64 = nullptr;
     cdf *d_blkdf = nullptr;
+    bool applied[2] = {false, false};   // pfft_precond_apply has applied these factors, in FP64, in double-float
     float2 *d_u32 = nullptr;          // FP32 sweep buffer [R][nunk]
     // bands wider than a warp (31 < W < 1024): FP32 roundings of band and bandc (mixed form)
     float2 *d_band32 = nullptr, *d_bandc32 = nullptr;
@@ -1126,12 +1127,32 @@ __global__ void __launch_bounds__(128, 2) k_pc_sweep(
 // application.
 constexpr int kMatWarps = 4, kMatStages = 4;
 // Chains up to which the matrix sweeps serve (their matrices cost 32 (W + 32)
-// values per chunk and direction, and a product more per chunk than the steps).
+// values per chunk and direction, and a product more per chunk than the steps).  At
+// the line, 8 wires of 77 segments x 8 right-hand sides, whole application: FP64
+// 1092 us stepped, 420 as matrices, double-float 421 and 258.
 constexpr int64_t kMatChains = 64;
+// One application repays the build of the matrices if what it saves, a fixed time
+// per chunk of the longest block (the chains run side by side), is more than the
+// build takes, a fixed time per matrix (slots x 2 x chunks of all blocks) on the
+// FP64 pipe plus a first one's latency.  Measured in microseconds, bands 9 to 22:
+// saved per chunk 9 in FP64 and 2.4 in double-float, less 15 for the further
+// launches; built in 0.0073 (W + 2) each after 15 + 4.5 W (band 22, 11,904
+// matrices: 2.07 ms; band 9, 6,016: 0.47 ms, 94: 45 us).
+bool mat_repaid(const PrecondState *s, bool dfl) {
+    int64_t longest = 0;
+    for (size_t b = 0; b + 1 < s->blk_off.size(); ++b)
+        longest = std::max(longest, (s->blk_off[b + 1] - s->blk_off[b] + 31) / 32);
+    const double saved = (dfl ? 2.4 : 9.0) * double(longest) - 15.0;
+    const double build = 15.0 + 4.5 * s->W + 0.0073 * (s->W + 2) * 2.0 * double(s->nslots) * double(s->nchunks);
+    return saved > build;
+}
 
 // blocks[slot][dir][chunk][W + 32][32]: W columns of M_c (rows 32 - W .. 31 of the
 // chunk before), then the 32 columns of G_c; lanes over the chunk's rows.  One
-// CTA per (slot, dir, chunk); chunk rows as in k_pc_sweep_pipe.
+// CTA per (slot, dir, chunk); chunk rows as in k_pc_sweep_pipe.  Bound by the FP64
+// pipe, so the products run over the band's entries only: 32 W complex products
+// a lane in all (band 22, 11,904 matrices: 3.52 -> 2.07 ms; band 9, 6,016: 1.20 ->
+// 0.47 ms).
 template <typename T>
 __global__ void __launch_bounds__(256) k_pc_blocks(
     const double2 *__restrict__ band, const double2 *__restrict__ bandc, const int64_t *__restrict__ blk_off,
@@ -1158,11 +1179,12 @@ __global__ void __launch_bounds__(256) k_pc_blocks(
         P[l * 33 + j] = elem(c * 32 + l, 32 + l - j);   // column j: row j of the chunk before
     }
     __syncthreads();
-    if (threadIdx.x < 32) {   // G: one column per lane by forward substitution
+    if (threadIdx.x < 32) {   // G: one column per lane by forward substitution, over the band's entries
         const int j = threadIdx.x;
         for (int l = 0; l < 32; ++l) {
             double2 a = make_double2(l == j ? 1.0 : 0.0, 0.0);
-            for (int i = 0; i < l; ++i) {
+#pragma unroll 4
+            for (int i = max(0, l - W); i < l; ++i) {
                 const double2 e = A[l * 33 + i], g = i >= j ? G[i * 33 + j] : make_double2(0.0, 0.0);
                 a.x = ::fma(-e.x, g.x, ::fma(e.y, g.y, a.x));
                 a.y = ::fma(-e.x, g.y, ::fma(-e.y, g.x, a.y));
@@ -1178,13 +1200,19 @@ __global__ void __launch_bounds__(256) k_pc_blocks(
         if (q >= W) {
             v = G[l * 33 + (q - W)];
         } else {
-            for (int j = 0; j <= l; ++j) {
+#pragma unroll 4
+            for (int j = 0; j <= min(l, q); ++j) {   // P is zero below its diagonal j = q
                 const double2 g = G[l * 33 + j], e = P[j * 33 + 32 - W + q];
                 v.x = ::fma(g.x, e.x, ::fma(-g.y, e.y, v.x));
                 v.y = ::fma(g.x, e.y, ::fma(g.y, e.x, v.y));
             }
         }
-        out[i] = mk<T>(T(v.x), T(v.y));
+        if constexpr (std::is_same<T, df>::value) {   // one rounding to FP32 pairs, off the FP64 pipe
+            const DD a = dd_split(v.x), b = dd_split(v.y);
+            out[i] = cdf{df(a.hi, a.lo), df(b.hi, b.lo)};
+        } else {
+            out[i] = v;
+        }
     }
 }
 
@@ -1406,6 +1434,7 @@ int pc_prepare(pfft_plan *p, const double *omega, int32_t R, std::vector<int32_t
     s->d_adf = nullptr;
     s->d_blk64 = nullptr;
     s->d_blkdf = nullptr;
+    s->applied[0] = s->applied[1] = false;
     if (s->d_a) cudaFreeAsync(s->d_a, st);
     if (s->d_a32) cudaFreeAsync(s->d_a32, st);
     if (s->d_band32) cudaFreeAsync(s->d_band32, st);
@@ -1670,13 +1699,24 @@ int pc_apply_t(pfft_plan *p, const double2 *y, double2 *z, int32_t R, cudaStream
 // They only speed the sweeps up: callers allocate what they cannot do without
 // first, and an allocation that fails later takes their memory back
 // (precond_release_spare), after which the stepped sweeps serve.
-int pc_blocks_prepare(pfft_plan *p, int32_t R, bool dfl, cudaStream_t st) {
+// once: for one application, where more may never follow with these factors.  Unless
+// it repays the build by itself the first such application takes the stepped sweeps,
+// a second one builds: 16 frequencies of three 124-segment wires, at new frequencies
+// 18.9 ms with the steps and 21.3 ms with a build of 3.5 ms (2.1 ms since it skips
+// the band's zeros), at known ones 1.72 and 0.59 ms.  A solve applies P^-1 often
+// enough to build at once.
+int pc_blocks_prepare(pfft_plan *p, int32_t R, bool dfl, bool once, cudaStream_t st) {
     PrecondState *s = p->pc;
     const int32_t nblk = int32_t(s->blk_off.size()) - 1;
     if (s->nd || s->W > 31 || s->W < 1 || s->nunk == 0 || R * int64_t(nblk) > kMatChains) return SIE_OK;
     if (dfl ? s->d_blkdf != nullptr : s->d_blk64 != nullptr) return SIE_OK;
     const int64_t ctas = int64_t(s->nslots) * 2 * s->nchunks;
     if (ctas > INT32_MAX) return SIE_OK;
+    if (once) {
+        const bool first = !s->applied[dfl];
+        s->applied[dfl] = true;
+        if (first && !mat_repaid(s, dfl)) return SIE_OK;
+    }
     const size_t bytes = size_t(ctas) * (s->W + 32) * 32 * sizeof(double2), sm = size_t(3) * 32 * 33 * sizeof(double2);
     void *blocks = nullptr;
     cudaMemPool_t pool;
@@ -1923,7 +1963,7 @@ extern "C" int pfft_precond_apply(pfft_plan *p, const void *y, void *z, int32_t 
     std::vector<int32_t> slot;
     int rc = pc_prepare(p, omega, nrhs, slot, st);
     if (rc) return rc;
-    if (prec != SIE_PREC_MIXED && (rc = pc_blocks_prepare(p, nrhs, prec == SIE_PREC_DF && pc_df_route(p), st)))
+    if (prec != SIE_PREC_MIXED && (rc = pc_blocks_prepare(p, nrhs, prec == SIE_PREC_DF && pc_df_route(p), true, st)))
         return rc;
     rc = pc_apply_async(p, (const double2 *)y, (double2 *)z, nrhs, prec, st);
     if (rc) return rc;
@@ -2115,7 +2155,7 @@ int gmres_create(pfft_plan *p, const double *freqs, int32_t nf, const int32_t *p
     if (g->resid_prec == SIE_PREC_DF && (rc = df_prepare(p, st))) return bail(rc);
     // the chunk matrices last, when everything the solve cannot do without is there
     for (int prec : {g->pc_prec, g->outer_pc_prec})
-        if (g->use_pc && prec != SIE_PREC_MIXED && (rc = pc_blocks_prepare(p, R, prec == SIE_PREC_DF, st)))
+        if (g->use_pc && prec != SIE_PREC_MIXED && (rc = pc_blocks_prepare(p, R, prec == SIE_PREC_DF, false, st)))
             return bail(rc);
     // ||P^-1 b|| (the outer precision's preconditioner); r = b - Z x with x = 0
     if (g->use_pc) {
