@@ -598,7 +598,8 @@ __global__ void k_pc_solve(const double2 *__restrict__ kappa, const int32_t *__r
 // in the forward sweep, the column-major copy in the backward sweep), and the
 // rows that enter the band take their right-hand sides.  Pending values live in
 // a circular shared-memory window of S >= W + 32 rows.  Three barriers per 32
-// pivots.  Used where k_pc_sweep_pipe's buffers do not fit shared memory.
+// pivots.  Used where k_pc_sweep_pipe's buffers do not fit shared memory, or fit an
+// SM once only and many chains would queue for it (pipe_serves).
 template <typename T, int MAXT>
 __global__ void __launch_bounds__(MAXT) k_pc_sweep_blk(
     const int64_t *__restrict__ blk_off, int32_t nblk, int32_t W, int32_t S, int64_t nunk,
@@ -757,6 +758,34 @@ constexpr int kPipeTri = 32 * 33;
 constexpr size_t kPipeMaxSmem = 227 * 1024;
 template <typename T> size_t pipe_smem(int W, int S) {
     return (size_t(S) + 2 * 32 + 2 * kPipeTri + 2 * size_t(W) * 33) * sizeof(C<T>);
+}
+// Whether the pipeline serves chains (right-hand side x block) of which an SM holds
+// pipe_per_sm: always while they fit one wave.  Beyond, k_pc_sweep_blk keeps more of
+// them on an SM (blk_per_sm), and its waves take longer the fuller they are.  Measured
+// in full waves of the pipeline, with l on an SM:
+//   FP32, one a SM (bands 179 up): 3.2 to 5.0 for 4 to 6; 4.3 is taken.  Two or
+//     more: the pipeline always (band 150, 960 to 1216 chains: 0.92 to 0.98 of the other
+//     kernel's speed, 1.1 to 3.6 times it elsewhere);
+//   FP64, one a SM (bands 76 up), three warps a CTA: 1.9 for up to 2, 2.9 for up to
+//     4; more warps: 2.1 and 2.7 (3); two warps, two a SM (bands 37 to 63): 0.9 +
+//     0.31 l, three a SM (32 to 36): 0.45 + 0.27 l, up to 6.  Otherwise the pipeline.
+// Of several waves of the other kernel the last takes a full one's time.
+// FP64, band 91, 512 chains: 9.1 ms, the pipeline 12.5; 152: 5.1 against 3.2.  FP32,
+// band 203, 912 chains: 23.2 ms, the pipeline 31.4; 1064: 48.0 against 36.6; band 214,
+// 608 chains, is the worst found on this side of the line: 24.0 ms, 18.8 for the other.
+template <typename T> bool pipe_serves(int64_t chains, int64_t sms, int pipe_per_sm, int blk_per_sm, int blk_warps) {
+    const bool f32 = sizeof(T) == 4;
+    if (chains <= sms * pipe_per_sm || blk_per_sm < 1) return true;
+    if (pipe_per_sm > (!f32 && blk_warps <= 2 ? 3 : 1)) return true;
+    auto wave = [&](int64_t l) {
+        if (f32) return 4.3;
+        if (blk_warps <= 2) return pipe_per_sm == 3 ? 0.45 + 0.27 * double(l) : 0.9 + 0.31 * double(l);
+        return blk_warps == 3 ? (l <= 2 ? 1.9 : 2.9) : (l <= 2 ? 2.1 : 2.7);
+    };
+    auto ceil_div = [](int64_t n, int64_t d) { return (n + d - 1) / d; };
+    const int64_t waves = ceil_div(chains, sms * blk_per_sm);
+    const double other = double(waves) * wave(waves > 1 ? blk_per_sm : ceil_div(chains, sms));
+    return double(ceil_div(chains, sms * pipe_per_sm)) <= other;
 }
 template <typename T>
 __global__ void __launch_bounds__(512) k_pc_sweep_pipe(
@@ -1662,25 +1691,29 @@ int pc_apply_t(pfft_plan *p, const double2 *y, double2 *z, int32_t R, cudaStream
             int S = 64;   // window of S >= W + 32 rows in shared memory
             while (S < s->W + 32) S *= 2;
             const unsigned ctas = unsigned(int64_t(R) * nblk);
+            const int wt = (s->W + 1 + 31) / 32 * 32, workers = std::min(15, std::max(7, (s->W + 31) / 32));
+            const auto blk = wt <= 256 ? k_pc_sweep_blk<T, 256> : k_pc_sweep_blk<T, 1024>;
+            const size_t sm = size_t(S + 32 * 33 + 32) * sizeof(C<T>);
             // the pipeline where two panels fit (band below about 400 in FP32, 180 in FP64)
+            // and its chains do not queue (pipe_serves)
             const size_t pipe = pipe_smem<T>(s->W, S);
-            if (pipe <= kPipeMaxSmem) {
-                const int workers = std::min(15, std::max(7, (s->W + 31) / 32));
+            bool piped = pipe <= kPipeMaxSmem;
+            if (piped) {
+                int sms = 0, np = 0, nb = 0;
                 if (int rc = set_smem((const void *)k_pc_sweep_pipe<T>, pipe)) return rc;
+                SIE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
+                if (int64_t(ctas) > sms) {
+                    SIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&np, k_pc_sweep_pipe<T>, 32 * (workers + 1), pipe));
+                    SIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, blk, wt, sm));
+                    piped = pipe_serves<T>(ctas, sms, np, nb, wt / 32);
+                }
+            }
+            if (piped) {
                 k_pc_sweep_pipe<T><<<ctas, 32 * (workers + 1), pipe, st>>>(s->d_blk_off, nblk, s->W, S, s->nunk, band,
                                                                            bandc, s->d_slot, u);
             } else {
-                const int wt = (s->W + 1 + 31) / 32 * 32;
-                const size_t sm = size_t(S + 32 * 33 + 32) * sizeof(C<T>);
-                if (wt <= 256) {
-                    if (int rc = set_smem((const void *)k_pc_sweep_blk<T, 256>, sm)) return rc;
-                    k_pc_sweep_blk<T, 256><<<ctas, wt, sm, st>>>(s->d_blk_off, nblk, s->W, S, s->nunk, band, bandc,
-                                                                 s->d_slot, u);
-                } else {
-                    if (int rc = set_smem((const void *)k_pc_sweep_blk<T, 1024>, sm)) return rc;
-                    k_pc_sweep_blk<T, 1024><<<ctas, wt, sm, st>>>(s->d_blk_off, nblk, s->W, S, s->nunk, band, bandc,
-                                                                  s->d_slot, u);
-                }
+                if (int rc = set_smem((const void *)blk, sm)) return rc;
+                blk<<<ctas, wt, sm, st>>>(s->d_blk_off, nblk, s->W, S, s->nunk, band, bandc, s->d_slot, u);
             }
         } else {
             if constexpr (f32) return fail(SIE_ERR_ARG, "preconditioner: FP32 sweeps need a band width below 1024");

@@ -44,3 +44,27 @@ def test_bands_cover_the_limits():
         pytest.skip("needs every size above")
     w = sorted(bands.values())
     assert w[0] < 64 and any(140 < v < 178 for v in w) and any(180 < v < 390 for v in w) and w[-1] > 400
+
+
+@pytest.mark.parametrize("nx,ny,band,R,prec", [(16, 15, (37, 64), 400, PREC_FP64), (30, 29, (76, 97), 320, PREC_FP64), (38, 37, (97, 113), 400, PREC_FP64),
+                                               (74, 73, (179, 240), 770, PREC_MIXED)])
+def test_many_chains_of_wide_panels(nx, ny, band, R, prec):
+    """Bands whose panels fill an SM, with more chains than the pipeline takes, against a
+    few chains of the same: FP32 takes the same order bit for bit, FP64 fused products
+    in one of them (1e-11, the bar of two orders of one FP64 solve)."""
+    h = 40e-6
+    m = box_mesh(nx * h, ny * h, 35e-6, nx, ny, 1, jitter=0.1, seed=nx)
+    M = api.Mesh.from_synth(m)
+    L = api.Loops(M, m.ports)
+    P = api.Plan(M, L, dict(grid=(16, 16, 8), n_touch=4, near_factor=1.0, near_min_diam=1.0))
+    api.precond_set_method(P, N.PC_BAND)
+    assert band[0] <= api.precond_info(P)["band_width"] < band[1]
+    few = [0, 1, R // 2, R - 1]
+    g = torch.Generator(device="cuda").manual_seed(3)
+    y = torch.randn(R, L.nl, dtype=torch.complex128, device="cuda", generator=g)
+    z = api.pfft_precond_apply(P, y, 2e9, prec=prec)[few]
+    ref = api.pfft_precond_apply(P, y[few].contiguous(), 2e9, prec=prec)
+    if prec == PREC_MIXED:
+        assert torch.equal(z, ref)
+    else:
+        assert (torch.linalg.norm(z - ref, dim=1) / torch.linalg.norm(ref, dim=1)).max().item() < 1e-11
