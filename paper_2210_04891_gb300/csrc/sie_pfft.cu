@@ -1399,35 +1399,48 @@ bool small_rhs(const pfft_plan *p, int32_t R) {
     return R <= kSmallRhs && p->params.kernel == SIE_KERNEL_STATIC && !(p->kt.near == 1 && R % 2 == 0) &&
            p->kt.proj_slab != kChunkRhs;
 }
-// A lane per output component (latency) up to kCompRows rows, a lane per column
-// (fewer load wavefronts) above; rows per warp: as many as fit, fewer while that
-// keeps more warps on the chip.
-bool small_comp(int64_t rows, int32_t R) {
-    constexpr int64_t kCompRows = 152 * 32;
-    return R <= 5 && rows <= kCompRows;
-}
-int small_rows(int64_t rows, int32_t R) {
-    constexpr int64_t kFill = 152 * 16;
-    const int64_t fit = 32 / ((small_comp(rows, R) ? 6 : 2) * R);
-    return int(std::max<int64_t>(1, std::min(fit, rows / kFill)));
+// A lane per output component (COMP) or per column of all three, and rows per warp.
+// Small meshes are bound by latency: the component form has a third of the loads in a
+// lane's chain and three times the warps; larger ones by load wavefronts, of which the
+// column form takes fewer.  us of both at 1, 3 and 5 right-hand sides, component form
+// first: near field, 4.7k triangles 41, 41, 47 and 63, 66, 68; 6.0k 51, 60, 65 and 79,
+// 83, 86; 8.0k 63, 105, 113 and 92, 98, 101: the line is at 40 rows an SM.  Projection,
+// 4.1k nodes 15, 16, 16 and 17, 17, 17; 8.2k 15, 17, 19 and 14, 15, 15: at 32.
+// Several rows per warp, as many as fit (columns or components x rows <= 32), while
+// 16 warps an SM remain; near field of one right-hand side with 8, 16 and 32 of them:
+// 12.0k triangles 119, 111 and 216 us, 5.2k 57, 58 and 89.
+constexpr int kCompTri = 40, kCompNodes = 32, kFillWarps = 16;
+struct SmallShape {
+    bool comp;
+    int rpw;   // rows per warp
+    int64_t blocks;
+};
+int small_shape(const pfft_plan *p, int64_t rows, int32_t R, int comp_rows, SmallShape &o) {
+    int sms = 0;
+    SIE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
+    o.comp = R <= 5 && rows <= int64_t(comp_rows) * sms;
+    const int64_t fit = 32 / ((o.comp ? 6 : 2) * R);
+    o.rpw = int(std::max<int64_t>(1, std::min(fit, rows / (int64_t(kFillWarps) * sms))));
+    o.blocks = (rows + kSmallWarps * o.rpw - 1) / (kSmallWarps * o.rpw);
+    return SIE_OK;
 }
 int project_small(pfft_plan *p, int32_t R, cudaStream_t st) {
-    const int rpw = small_rows(p->Ng, R), nodes = kSmallWarps * rpw;
-    const unsigned blocks = unsigned((p->Ng + nodes - 1) / nodes);
-    const size_t smem = size_t(nodes) * (6 * R + 2) * sizeof(float);
-    const auto fn = small_comp(p->Ng, R) ? k_project_small<true> : k_project_small<false>;
-    fn<<<blocks, 32 * kSmallWarps, smem, st>>>(p->d_pn_ptr, p->d_pn_rec32, (const float4 *)p->scr.cT, p->Ng, R, rpw,
-                                               (float2 *)p->scr.grid);
+    SmallShape g;
+    if (int rc = small_shape(p, p->Ng, R, kCompNodes, g)) return rc;
+    const size_t smem = size_t(kSmallWarps * g.rpw) * (6 * R + 2) * sizeof(float);
+    const auto fn = g.comp ? k_project_small<true> : k_project_small<false>;
+    fn<<<unsigned(g.blocks), 32 * kSmallWarps, smem, st>>>(p->d_pn_ptr, p->d_pn_rec32, (const float4 *)p->scr.cT,
+                                                           p->Ng, R, g.rpw, (float2 *)p->scr.grid);
     SIE_LAUNCH_CHECK(p);
     return SIE_OK;
 }
 int tri_gather_small(pfft_plan *p, int32_t R, cudaStream_t st) {
-    const int rpw = small_rows(p->nt, R);
-    const int64_t rows = int64_t(kSmallWarps) * rpw;
-    const auto fn = small_comp(p->nt, R) ? k_tri_small<true> : k_tri_small<false>;
-    fn<<<unsigned((p->nt + rows - 1) / rows), 32 * kSmallWarps, 0, st>>>(
+    SmallShape g;
+    if (int rc = small_shape(p, p->nt, R, kCompTri, g)) return rc;
+    const auto fn = g.comp ? k_tri_small<true> : k_tri_small<false>;
+    fn<<<unsigned(g.blocks), 32 * kSmallWarps, 0, st>>>(
         p->d_near_ptr, p->d_near_rec32, p->d_pt_ptr, p->d_pt_rec32, (const float4 *)p->scr.cT,
-        (const float4 *)p->scr.phiT, p->d_gram, p->d_cond, coef_dd(p), p->ncond, p->nt, R, rpw,
+        (const float4 *)p->scr.phiT, p->d_gram, p->d_cond, coef_dd(p), p->ncond, p->nt, R, g.rpw,
         (float4 *)p->scr.y_tri);
     SIE_LAUNCH_CHECK(p);
     return SIE_OK;

@@ -13,6 +13,7 @@ import numpy as np
 import pytest
 
 import synth
+from synth.meshes import wire_array_mesh
 from oracle.graph import build_loops
 from oracle.pfft import PfftSystem, PfftParams
 
@@ -81,3 +82,27 @@ def test_empty_grid_rows_are_skipped_without_a_trace():
             api.pfft_convolve(P, g, PREC_MIXED if prec == PREC_MIXED else PREC_FP64)
             api.pfft_matvec(P, torch.full_like(xt[:R], float("nan")), om[:R], SPACE_LOOP, prec)
             check(api.pfft_matvec(P, xt[:R].contiguous(), om[:R], SPACE_LOOP, prec), ref[:R], tol)
+
+
+@pytest.fixture(scope="module", params=[(386, (32, 8, 16)), (930, (64, 16, 16))], ids=["5418", "13034"])
+def long_wire(request):
+    """A seven-sided wire: 5,418 triangles (component form, two rows per warp) and 13,034
+    (column form, up to five), ragged in the last warp and block; 4,096 and 16,384 nodes
+    (one row per warp, up to six)."""
+    seg, grid = request.param
+    m = wire_array_mesh(1, 10e-6, seg * 1e-5, 4e-5, n_sides=7, n_seg=seg, jitter=0.1, seed=seg)
+    assert m.nt == 14 * (seg + 1)
+    M = api.Mesh.from_synth(m)
+    P = api.Plan(M, api.Loops(M, m.ports), dict(grid=grid, n_touch=8))
+    om = 2 * np.pi * np.logspace(7, 10, 17)
+    x = torch.from_numpy(synth.complex_gaussian(P.nl, 17, seed=22)).cuda()
+    alone = torch.cat([api.pfft_matvec(P, x[r:r + 1], om[r:r + 1], SPACE_LOOP, PREC_MIXED) for r in range(17)])
+    return P, om, x, alone, api.pfft_matvec(P, x, om, SPACE_LOOP, PREC_FP64).cpu().numpy()
+
+
+@pytest.mark.parametrize("R", range(1, 18))
+def test_mixed_columns_of_several_rows_per_warp(long_wire, R):
+    P, om, x, alone, ref = long_wire
+    y = api.pfft_matvec(P, x[:R].contiguous(), om[:R], SPACE_LOOP, PREC_MIXED)
+    assert torch.equal(y, alone[:R])
+    check(y, ref[:R], 1e-5)
