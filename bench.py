@@ -60,6 +60,7 @@ def peaks():
 # ------------------------------------------------------------------ algorithmic work per stage launch
 
 FP32_LANES_PER_SM = 128      # FP32 FMA lanes per SM (4 sub-partitions x 32) on Blackwell
+FFT_MAX_ELEMS = 8192         # padded values of the largest (y, z) plane one CTA transforms
 
 
 def sm_count():
@@ -67,24 +68,46 @@ def sm_count():
     import torch
     return int(torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count)
 
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch from an ncu capture of the
-# current kernel, with the number of grids (3 x right-hand sides) of that capture; the
-# figure is scaled to a launch of the bench by grids.  Only kernels captured since their
-# last change are listed.
+# dram__bytes_read.sum + dram__bytes_write.sum of one launch from an ncu capture, with the
+# number of grids (3 x right-hand sides) of that capture; the figure is scaled to a launch
+# of the bench by grids.  MEASURED_TRAFFIC: every row of the planes (pfft_convolve);
+# ROWS_TRAFFIC: the product's launch, which skips the rows without stencil nodes, with the
+# rows it took.  Both on planes of 128 x 64 padded values at 256 x-frequencies.
 MEASURED_TRAFFIC = {"fft_yz": (348.81e6, 48)}   # k_plane_conv<128, 64> (zero-pad pruned), 2 frequencies x 8 ports
-
+ROWS_TRAFFIC = {"fft_yz": (220.33e6, 48, 44)}
+TRAFFIC_PLANE = (128, 128, 64)                  # N_x, M_y, M_z of those captures
 
 def alu_peak_tflops(sm_mhz, nsm):
     """FP32 FMA peak of the CUDA cores: SMs x lanes x 2 flop x SM clock."""
     return nsm * FP32_LANES_PER_SM * 2 * sm_mhz * 1e6 / 1e12
 
 
+def active_rows(nodes, grid):
+    """(y rows, (y, z) columns) that the product's convolution transforms on a grid
+    [N_x, N_y, N_z] with stencil nodes `nodes`: where a plane fits one CTA and has 32 to 128
+    rows, row pairs without a node are skipped if they are an eighth or more of the rows,
+    and the x pencils run over the tiles of columns (16, or 8 from M_x = 512) that hold a
+    row in use.  Otherwise all."""
+    Nx, Ny, Nz = grid
+    one_cta = Ny <= 128 and Nz <= 128 and 48 * Ny * (2 * Nz + 1) <= 200 * 1024 and 4 * Ny * Nz <= FFT_MAX_ELEMS
+    if not one_cta or Ny < 32:
+        return Ny, Ny * Nz
+    used = np.zeros(Ny, bool)
+    used[np.unique(np.asarray(nodes) // Nz % Ny)] = True
+    used = np.repeat(used.reshape(-1, 2).any(1), 2)
+    rows = int(used.sum())
+    if 8 * rows > 7 * Ny:
+        return Ny, Ny * Nz
+    kt = 8 if 2 * Nx > 256 else 16
+    return rows, kt * int(np.repeat(used, Nz).reshape(-1, kt).any(1).sum())
+
+
 def plane_flops(Ny, Nz, My, Mz):
     """Flops of one x-frequency plane of the (y, z) convolution, counted as
     5 n log2 n per complex FFT of length n over the lines that carry data: the
-    forward z transforms of the Ny input rows (rows Ny..My-1 are zero), the
-    forward y transforms of all Mz columns, the real kernel product (2 flops a
-    point), the inverse y transforms of all columns, and the inverse z
+    forward z transforms of the Ny input rows that hold data (the others of My are
+    zero), the forward y transforms of all Mz columns, the real kernel product (2
+    flops a point), the inverse y transforms of all columns, and the inverse z
     transforms of the Ny rows that are kept."""
     return (2 * Ny * 5 * Mz * np.log2(Mz) + 2 * Mz * 5 * My * np.log2(My) + 2 * My * Mz)
 
@@ -98,15 +121,17 @@ def stage_work(stage, c):
     = 36 flop per right-hand side).  c: sizes of the workload and plan."""
     R, cb = c["R"], c["cb"]
     Ng, Nx, My, Mz, nt, nl = c["Ng"], c["Nx"], c["My"], c["Mz"], c["nt"], c["nl"]
+    # grid rows and values per x that the convolution takes (active_rows)
+    rows, cols = c.get("rows", My // 2), c.get("cols", Ng // Nx)
     if stage == "fft_x_fwd":          # grid read, x-padded grid written
-        return "hbm", 3 * R * (Ng + 2 * Ng) * cb, "B"
+        return "hbm", 3 * R * 3 * Nx * cols * cb, "B"
     if stage == "fft_yz":
         # per x-frequency plane (2 Nx of them per grid): plane_flops; the kernel is bound by
         # instruction issue on the FP32 pipe and shared memory (ncu), not by HBM (its bytes:
         # stage_bytes below)
-        return "alu", 3 * R * 2 * Nx * plane_flops(My // 2, Mz // 2, My, Mz), "flop"
+        return "alu", 3 * R * 2 * Nx * plane_flops(rows, Mz // 2, My, Mz), "flop"
     if stage == "fft_x_inv":          # x-padded grid read, grid written
-        return "hbm", 3 * R * (2 * Ng + Ng) * cb, "B"
+        return "hbm", 3 * R * 3 * Nx * cols * cb, "B"
     if stage == "project":
         # c_T read, node-ordered block records read, grid written
         return "hbm", R * nt * 3 * cb + c["n_pair"] * c["rec"] + (Ng + 1) * 8 + 3 * R * Ng * cb, "B"
@@ -133,11 +158,26 @@ def stage_work(stage, c):
 
 def stage_bytes(stage, c):
     """Unique HBM bytes of a stage whose primary bound is not HBM, for the
-    second roofline basis: the (y, z) planes read the x-transformed grids
-    (2 N_g values per grid) and write them back."""
+    second roofline basis: the (y, z) planes read the rows in use of the
+    x-transformed grids (2 N_g values per grid with all rows) and write them back."""
     if stage == "fft_yz":
-        return 3 * c["R"] * 4 * c["Ng"] * c["cb"]
+        return 3 * c["R"] * 4 * c["Nx"] * c.get("rows", c["My"] // 2) * (c["Mz"] // 2) * c["cb"]
     return None
+
+
+def stage_traffic(stage, c):
+    """DRAM bytes of one launch of a stage, scaled from an ncu capture of the kernel
+    on the same planes with the same rows; None without one."""
+    if stage not in MEASURED_TRAFFIC or (c["Nx"], c["My"], c["Mz"]) != TRAFFIC_PLANE:
+        return None
+    rows = c.get("rows", c["My"] // 2)
+    if rows == c["My"] // 2:
+        by, grids = MEASURED_TRAFFIC[stage]
+    else:
+        by, grids, captured = ROWS_TRAFFIC[stage]
+        if rows != captured:
+            return None
+    return by * (3 * c["R"]) / grids
 
 
 class ClockSampler:
@@ -754,6 +794,7 @@ def main():
     pnode = P.export(N.EXPORT_PROJ_NODE)
     ctx = dict(R=R, cb=8, rec=48, Ng=Nx * Ny * Nz, Nx=Nx, My=2 * Ny, Mz=2 * Nz, nt=info["n_tri"], nl=L.nl,
                n_near=info["n_near_pairs"], n_pair=int(pnode.size), n_active=int(np.unique(pnode).size))
+    ctx["rows"], ctx["cols"] = active_rows(pnode, w["grid"])
     timed_stages = [s for s in prof if prof[s][1] > 0]   # none when the step is a graph replay
     dom = max(timed_stages, key=lambda s: prof[s][0]) if timed_stages else None
     ms_dom, n_dom = prof[dom] if dom else (0.0, 0)
@@ -775,10 +816,7 @@ def main():
             achieved, peak, u = amount / sec / 1e12, alu_peak_tflops(mhz, nsm), "TFLOP/s"
             psrc = (f"derived: {nsm} SMs (device query) x {FP32_LANES_PER_SM} FP32 FMA lanes x 2 flop x "
                     f"{mhz:.0f} MHz (sampled max SM clock)")
-        traffic = None
-        if dom in MEASURED_TRAFFIC:
-            tb, grids = MEASURED_TRAFFIC[dom]
-            traffic = tb * (3 * R) / grids
+        traffic = stage_traffic(dom, ctx)
         roofline = {"bound": bound, "achieved": achieved, "peak": peak, "unit": u, "frac": achieved / peak,
                     "traffic": traffic, "kernel": dom, "peak_source": psrc,
                     "algorithmic_per_launch": amount, "algorithmic_unit": unit, "launch_ms": ms_dom / n_dom,

@@ -75,3 +75,42 @@ def test_measured_traffic_scales_to_a_bench_launch():
     tb, grids = bench.MEASURED_TRAFFIC["fft_yz"]
     assert grids == 48
     assert tb * 384 / grids == pytest.approx(2.79048e9, rel=1e-6)
+
+
+def test_active_rows_follow_the_stencil_nodes():
+    # 64 rows of 32 nodes in a plane: rows 10..30 and 51 hold a node, so the pairs 10-11 .. 30-31 and 50-51 do
+    grid = (128, 64, 32)
+    nodes = [(5 * 64 + y) * 32 + 3 for y in list(range(10, 31)) + [51]]
+    # 24 rows, each two x tiles of 16 columns
+    assert bench.active_rows(nodes, grid) == (24, 24 * 32)
+    # one pair in eight empty: skipped; fewer: all rows
+    rows = [y for y in range(64) if y // 8 != 3]
+    assert bench.active_rows([y * 32 for y in rows], grid) == (56, 56 * 32)
+    assert bench.active_rows([y * 32 for y in rows + [24]], grid) == (64, 64 * 32)
+    # N_z = 4: a tile of 16 columns spans four rows (two pairs), 8 columns (M_x = 512) one pair
+    nodes = [y * 4 for y in (0, 6, 33)]
+    assert bench.active_rows(nodes, (64, 64, 4)) == (6, 12 * 4)
+    assert bench.active_rows(nodes, (256, 64, 4)) == (6, 6 * 4)
+    # fewer than 32 rows, or a plane larger than one CTA: all
+    assert bench.active_rows([0], (128, 16, 32)) == (16, 16 * 32)
+    assert bench.active_rows([0], (256, 256, 32)) == (256, 256 * 32)
+
+
+def test_convolution_stages_count_only_the_rows_in_use():
+    c = dict(BOND, rows=40, cols=40 * 32)
+    # x pencils: 384 grids x 128 x-rows x 1,280 of 2,048 columns, read once and written padded; 8 B
+    assert bench.stage_work("fft_x_fwd", c) == ("hbm", 384 * 3 * 128 * 1280 * 8, "B")
+    assert bench.stage_work("fft_x_inv", c) == ("hbm", 384 * 3 * 128 * 1280 * 8, "B")
+    # planes: z transforms of 40 rows both ways (2 * 40 * 5 * 64 * 6 = 153,600), y as with all rows (573,440),
+    # product 16,384
+    assert bench.stage_work("fft_yz", c) == ("alu", 384 * 256 * 743424, "flop")
+    assert bench.stage_bytes("fft_yz", c) == 384 * 256 * 40 * 32 * 2 * 8
+
+
+def test_traffic_is_of_the_same_rows_only():
+    assert bench.stage_traffic("fft_yz", BOND) == pytest.approx(348.81e6 * 8)
+    by, grids, rows = bench.ROWS_TRAFFIC["fft_yz"]
+    assert bench.stage_traffic("fft_yz", dict(BOND, rows=rows)) == pytest.approx(by * 384 / grids)
+    assert bench.stage_traffic("fft_yz", dict(BOND, rows=rows - 2)) is None
+    assert bench.stage_traffic("fft_yz", dict(BOND, Nx=64)) is None
+    assert bench.stage_traffic("near", BOND) is None
