@@ -243,8 +243,12 @@ template <int MY, int MZ> struct Geo {
     static constexpr int kWide = cmax(NYP * cmax(A1, A2) / 2, MZ / 2 * cmax(B1, B2));
     static constexpr int TP = kWide <= 32 ? 32 : kWide <= 64 ? 64 : kWide <= 128 ? 128 : kThreads;
     static constexpr int NG = kThreads / TP;                        // planes side by side in a CTA
-    // CTAs per SM by registers: four where the short transforms are at most 8 long
-    static constexpr int kCtas = TP <= 64 && cmax(A2, B2) <= 8 ? 4 : 2;
+    // CTAs per SM that the registers must allow: four (64 a thread) for planes of a few
+    // long rows, two above, where 64 registers spill.  96 and 384 grids of 64 planes,
+    // us, four and two: 16 x 16 18.2, 55.8 and 19.6, 55.9; 8 x 32 (8 bytes spilled)
+    // 26.1, 83.5 and 29.5, 87.6; 32 x 16 38.4, 136.6 and 38.2, 128.6; 64 x 16 50.7, 189.5
+    // and 48.7, 181.3.
+    static constexpr int kCtas = TP <= 64 && MY <= 16 && cmax(A2, B2) <= 8 ? 4 : 2;
     static constexpr size_t kSmem =
         size_t(NG * (2 * NP + 2 * NQ) + NH) * sizeof(float) + size_t(NTW) * sizeof(float2);
     static_assert(NYP >= 1 && A1 >= 2 && A2 >= 2 && B1 >= 2 && B2 >= 2 && A2 <= 16 && B2 <= 16, "plane size");
