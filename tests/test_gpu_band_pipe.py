@@ -68,3 +68,15 @@ def test_many_chains_of_wide_panels(nx, ny, band, R, prec):
         assert torch.equal(z, ref)
     else:
         assert (torch.linalg.norm(z - ref, dim=1) / torch.linalg.norm(ref, dim=1)).max().item() < 1e-11
+
+
+def test_these_sizes_lie_on_both_sides_of_the_limits():
+    """Alone, from the plans themselves: a band each for the first tiles above a warp, the
+    FP64 pipeline's last, the FP32 pipeline's and the wider kernel's."""
+    h = 40e-6
+    for nx, ny, lo, hi in ((14, 12, 32, 64), (64, 62, 140, 178), (101, 97, 180, 390), (154, 152, 400, 1024)):
+        m = box_mesh(nx * h, ny * h, 35e-6, nx, ny, 1, jitter=0.1, seed=nx)
+        M = api.Mesh.from_synth(m)
+        P = api.Plan(M, api.Loops(M, m.ports), dict(grid=(16, 16, 8), n_touch=4, near_factor=1.0, near_min_diam=1.0))
+        api.precond_set_method(P, N.PC_BAND)
+        assert lo <= api.precond_info(P)["band_width"] < hi, (nx, ny)
