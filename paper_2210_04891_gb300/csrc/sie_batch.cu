@@ -290,8 +290,9 @@ extern "C" int sie_batch_solve(sie_batch *b, const double *const *freqs, const i
     }
     for (auto &t : workers) t.join();
     // out of memory: once more, one plan at a time, without what only speeds the plans up
+    bool spare = false;
     for (size_t i = 0; i < n; ++i)
-        if (rcs[i] == SIE_ERR_OOM && release_spare(b)) {
+        if (rcs[i] == SIE_ERR_OOM && (spare = release_spare(b) || spare)) {
             rcs[i] = sie_solve(b->plans[i], freqs[i], nf[i], ports[i], np[i], opts, Z_out[i],
                                st_out ? &st_out[i] : nullptr);
             msgs[i] = rcs[i] ? sie_last_error() : "";
@@ -400,8 +401,9 @@ extern "C" int sie_batch_solve_graph(sie_batch *b, const double *const *freqs, c
         if (rcs[i]) msgs[i] = sie_last_error();
     });
     // out of memory: once more without what only speeds the plans up
+    bool spare = false;
     for (size_t i = 0; i < n; ++i)
-        if (rcs[i] == SIE_ERR_OOM && release_spare(b)) {
+        if (rcs[i] == SIE_ERR_OOM && (spare = release_spare(b) || spare)) {
             rcs[i] = gmres_create(b->plans[i], freqs[i], nf[i], ports[i], np[i], opts, b->streams[i], &runs[i]);
             msgs[i] = rcs[i] ? sie_last_error() : "";
         }
