@@ -995,7 +995,7 @@ __global__ void __launch_bounds__(256)
 // complex product sit in neighbouring lanes: each lane forms its own half of
 // Eq. Zb from its Gram term and its neighbour's.
 // FP64 on the bond wires (40k triangles, 14.1M records), 48 right-hand sides:
-// 20.3 ms, 96 % of the FP64 pipe, against 38.6 ms with a complex right-hand side
+// 20.3 ms, 96 % of the FP64 pipe (98 % in a capture on 20k triangles), against 38.6 ms with a complex right-hand side
 // per lane (48 of 64 lanes, four operations per term); 20k triangles, 8
 // right-hand sides: 1.71 against 9.06 ms; 1.5k triangles, one: 44 against 843 us.
 // Double-float on the 40k triangles, 16: 2.37 against 3.65 ms.
@@ -1415,18 +1415,16 @@ struct SmallShape {
     int rpw;   // rows per warp
     int64_t blocks;
 };
-int small_shape(const pfft_plan *p, int64_t rows, int32_t R, int comp_rows, SmallShape &o) {
-    int sms = 0;
-    SIE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
-    o.comp = R <= 5 && rows <= int64_t(comp_rows) * sms;
+SmallShape small_shape(const pfft_plan *p, int64_t rows, int32_t R, int comp_rows) {
+    SmallShape o;
+    o.comp = R <= 5 && rows <= int64_t(comp_rows) * p->sms;
     const int64_t fit = 32 / ((o.comp ? 6 : 2) * R);
-    o.rpw = int(std::max<int64_t>(1, std::min(fit, rows / (int64_t(kFillWarps) * sms))));
+    o.rpw = int(std::max<int64_t>(1, std::min(fit, rows / (int64_t(kFillWarps) * p->sms))));
     o.blocks = (rows + kSmallWarps * o.rpw - 1) / (kSmallWarps * o.rpw);
-    return SIE_OK;
+    return o;
 }
 int project_small(pfft_plan *p, int32_t R, cudaStream_t st) {
-    SmallShape g;
-    if (int rc = small_shape(p, p->Ng, R, kCompNodes, g)) return rc;
+    const SmallShape g = small_shape(p, p->Ng, R, kCompNodes);
     const size_t smem = size_t(kSmallWarps * g.rpw) * (6 * R + 2) * sizeof(float);
     const auto fn = g.comp ? k_project_small<true> : k_project_small<false>;
     fn<<<unsigned(g.blocks), 32 * kSmallWarps, smem, st>>>(p->d_pn_ptr, p->d_pn_rec32, (const float4 *)p->scr.cT,
@@ -1435,8 +1433,7 @@ int project_small(pfft_plan *p, int32_t R, cudaStream_t st) {
     return SIE_OK;
 }
 int tri_gather_small(pfft_plan *p, int32_t R, cudaStream_t st) {
-    SmallShape g;
-    if (int rc = small_shape(p, p->nt, R, kCompTri, g)) return rc;
+    const SmallShape g = small_shape(p, p->nt, R, kCompTri);
     const auto fn = g.comp ? k_tri_small<true> : k_tri_small<false>;
     fn<<<unsigned(g.blocks), 32 * kSmallWarps, 0, st>>>(
         p->d_near_ptr, p->d_near_rec32, p->d_pt_ptr, p->d_pt_rec32, (const float4 *)p->scr.cT,

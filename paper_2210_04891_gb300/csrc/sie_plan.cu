@@ -717,6 +717,7 @@ extern "C" int pfft_plan_create(const sie_mesh *m, const sie_loops *L, const pff
     if (!p) return fail(SIE_ERR_OOM, "pfft_plan_create: out of host memory");
     auto bail = [&](int rc) { pfft_plan_destroy(p); return rc; };
     cudaGetDevice(&p->device);
+    cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
     p->stream = static_cast<cudaStream_t>(cuda_stream);
     p->params = *prm;
     p->loops = L;

@@ -65,6 +65,7 @@ struct Scratch {
 
 struct pfft_plan {
     int device = 0;
+    int sms = 0;                        // SMs of the device
     cudaStream_t stream = nullptr;
     int64_t launches = 0;
     // sizes

@@ -22,12 +22,10 @@ int launch_plane(pfft_plan *p, float2 *spec, int32_t ngrids, int lgMx, bool acti
         }
     }
     if (int rc = set_smem((const void *)kern, G::kSmem)) return rc;
-    int nsm = 0;
-    SIE_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device));
     // grids per CTA: one for each of its groups, and up to 8 (the staged spectrum and
     // twiddles serve each of them) while keeping about four waves of two CTAs per SM
     const int64_t planes = int64_t(ngrids) * p->Mx;
-    const int64_t fill = std::max<int64_t>(std::min(G::NG, ngrids), planes / (8 * int64_t(nsm)));
+    const int64_t fill = std::max<int64_t>(std::min(G::NG, ngrids), planes / (8 * int64_t(p->sms)));
     const int gpc = int(std::max<int64_t>(1, std::min<int64_t>(p->kt.plane_gpc > 0 ? p->kt.plane_gpc : 8 * G::NG, fill)));
     const int64_t ctas = int64_t(p->Mx) * ((ngrids + gpc - 1) / gpc);
     kern<<<unsigned(ctas), plane::kThreads, G::kSmem, s>>>(spec, ngrids, gpc, lgMx, p->d_Hp32, p->d_tf32[1],

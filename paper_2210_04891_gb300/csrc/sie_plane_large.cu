@@ -164,12 +164,11 @@ int launch(pfft_plan *p, float2 *spec, int32_t ngrids, cudaStream_t s) {
     using G = LargeGeo<N1, N2, Z1, Z2>;
     auto kern = k_plane_large<N1, N2, Z1, Z2>;
     if (int rc = set_smem((const void *)kern, G::smem)) return rc;
-    int nsm = 0, lgMx = 0;
-    SIE_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device));
+    int lgMx = 0;
     while ((1 << lgMx) < p->Mx) ++lgMx;
     // grids per CTA: up to 8 share the staged spectrum while eight waves remain
     const int64_t planes = int64_t(ngrids) * p->Mx;
-    const int gpc = int(std::max<int64_t>(1, std::min<int64_t>(8, planes / (8 * int64_t(nsm)))));
+    const int gpc = int(std::max<int64_t>(1, std::min<int64_t>(8, planes / (8 * int64_t(p->sms)))));
     const int64_t ctas = int64_t(p->Mx) * ((ngrids + gpc - 1) / gpc);
     if (ctas > INT32_MAX) return fail(SIE_ERR_ARG, "plane convolution: too many grids");
     kern<<<unsigned(ctas), kThreads, G::smem, s>>>(spec, ngrids, gpc, lgMx, p->d_Hp32, p->d_tf32[1], p->d_ti32[1],

@@ -735,7 +735,8 @@ __global__ void __launch_bounds__(MAXT) k_pc_sweep_blk(
 // per 32 pivots.  Every row takes the same contributions in the same order as in
 // k_pc_sweep_blk.  FP32 is bound by the chain, about 31 x 45 cycles a chunk (plates,
 // two blocks of 12.8k unknowns, 4 right-hand sides: 2.4 ms against 10.2 ms,
-// whose panels were read a row per thread), FP64 by the FP64 pipe (9.9, 17.6 ms).
+// whose panels were read a row per thread), FP64 by the chain's FMAs at the latency
+// of the FP64 pipe, which the panels share (half busy on the SMs at work: 9.9, 17.6 ms).
 // Row k of a sweep is row k (forward, row-major band B) or n - 1 - k (backward,
 // column-major copy Bc); its entry at pivot k - d is elem(k)[d].
 template <typename V> __device__ __forceinline__ void cp_async_value(V *dst, const V *src) {
@@ -1699,13 +1700,12 @@ int pc_apply_t(pfft_plan *p, const double2 *y, double2 *z, int32_t R, cudaStream
             const size_t pipe = pipe_smem<T>(s->W, S);
             bool piped = pipe <= kPipeMaxSmem;
             if (piped) {
-                int sms = 0, np = 0, nb = 0;
+                int np = 0, nb = 0;
                 if (int rc = set_smem((const void *)k_pc_sweep_pipe<T>, pipe)) return rc;
-                SIE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
-                if (int64_t(ctas) > sms) {
+                if (int64_t(ctas) > p->sms) {
                     SIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&np, k_pc_sweep_pipe<T>, 32 * (workers + 1), pipe));
                     SIE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, blk, wt, sm));
-                    piped = pipe_serves<T>(ctas, sms, np, nb, wt / 32);
+                    piped = pipe_serves<T>(ctas, p->sms, np, nb, wt / 32);
                 }
             }
             if (piped) {
