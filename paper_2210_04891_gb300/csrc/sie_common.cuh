@@ -85,8 +85,9 @@ template <> __host__ __device__ __forceinline__ cdf cscale<cdf, df>(cdf a, df h)
 // acc += b x for double-float b and x into an unnormalised double-float sum:
 // the high part takes one FP32 add per term (the chain a gather runs along),
 // the two-product error of the high parts, the two-sum error of that add and
-// the cross products of high and low parts go to the low part, one add per
-// term.  A sum of n terms keeps about 48 bits plus log2(n); readers treat
+// the cross products of high and low parts go to the low part, one plain add per
+// term, whose roundings gather: a sum of n terms keeps about 48 - log2(n) bits of the
+// sum of its terms' magnitudes (of a sum that cancels, as many fewer).  Readers treat
 // (hi, lo) as the value hi + lo, whatever its normalisation.
 __device__ __forceinline__ void df_acc(df &acc, df b, df x) {
     const float p = b.hi * x.hi;
