@@ -777,33 +777,54 @@ __global__ void __launch_bounds__(256) k_fft_rows(C<T> *__restrict__ buf, int M,
 
 // ---- (y, z) plane passes with compile-time split (see k_fft_yzc).  The
 // input extent is half of each padded length (Ny = My/2, Nz = Mz/2).  The z
-// passes run over the rows that hold data (Rows); F1 clears the others in Q for F3.
-struct Rows {
-    const uint8_t *list;   // shared memory, ascending
+// passes run over the rows that Rows names:
+//   all of them, by shifts;
+//   the rows that hold data (kListed), by a list, and a division by their number as a
+//     product (exact below 2^11 items of up to 128 rows); F1's caller clears the others
+//     in Q for F3.  FP64 and double-float, whose pipes then have less to do;
+//   all, with those that hold no data taken as zero (kMasked).  FP32, which the list
+//     costs more than the rows it saves: lossy kernel, 96 grids of 32 x 64 x 16 nodes,
+//     34 rows in use, planes 134 us listed, 117 with all rows; none left out, 120 grids
+//     of 64 x 16 x 16, 153 and 125 us.
+enum RowsKind { kAllRows, kListed, kMasked };
+template <RowsKind K> struct Rows {
+    const uint8_t *list;   // shared memory, ascending (kListed)
     int n;
-    __device__ __forceinline__ int row(int i) const { return list[i]; }
+    unsigned inv;          // kListed: ceil(2^20 / n); else log2(n)
+    ulonglong2 mask;       // rows that hold data (kMasked)
+    __device__ __forceinline__ int row(int i) const { return K == kListed ? list[i] : i; }
+    __device__ __forceinline__ bool has(int y) const {
+        return K != kMasked || (((y < 64 ? mask.x : mask.y) >> (y & 63)) & 1);
+    }
+    // item = k n + i
+    __device__ __forceinline__ int split(int item, int &k) const {
+        k = K == kListed ? int((unsigned(item) * inv) >> 20) : item >> inv;
+        return item - k * n;
+    }
 };
-template <typename T, int N1, int N2>   // F1: z pass 1, rows y < Ny, global -> P row slots
-__device__ __forceinline__ void yz_f1(const C<T> *in, C<T> *P, int pitch, const Rows rw, const C<T> *tfz) {
+template <typename T, int N1, int N2, RowsKind K>   // F1: z pass 1, rows y < Ny, global -> P row slots
+__device__ __forceinline__ void yz_f1(const C<T> *in, C<T> *P, int pitch, const Rows<K> rw, const C<T> *tfz) {
     constexpr int Mz = N1 * N2, Nz = Mz / 2, H1 = N1 / 2;
     constexpr int LG2 = N2 == 2 ? 1 : N2 == 4 ? 2 : N2 == 8 ? 3 : 4;
     C<T> v[FFT_NMAX];
     for (int it = threadIdx.x; it < rw.n * N2; it += blockDim.x) {
         const int y = rw.row(it >> LG2), j2 = it & (N2 - 1);
         const C<T> *src = in + y * Nz + j2;
+        const bool has = rw.has(y);
 #pragma unroll
-        for (int j1 = 0; j1 < H1; ++j1) v[j1] = src[N2 * j1];
+        for (int j1 = 0; j1 < H1; ++j1) v[j1] = has ? src[N2 * j1] : mk<T>(T(0.0), T(0.0));
         FourStep<T, N1, N2>::fwd1(v, j2, tfz);
         C<T> *row = P + y * pitch + j2;
 #pragma unroll
         for (int k1 = 0; k1 < N1; ++k1) row[k1 * N2] = v[k1];
     }
 }
-template <typename T, int N1, int N2>   // F2: z pass 2, P row slots -> Q natural rows
-__device__ __forceinline__ void yz_f2(const C<T> *P, C<T> *Q, int pitch, const Rows rw, const C<T> *tfz) {
+template <typename T, int N1, int N2, RowsKind K>   // F2: z pass 2, P row slots -> Q natural rows
+__device__ __forceinline__ void yz_f2(const C<T> *P, C<T> *Q, int pitch, const Rows<K> rw, const C<T> *tfz) {
     C<T> v[FFT_NMAX];
     for (int it = threadIdx.x; it < rw.n * N1; it += blockDim.x) {
-        const int k1 = it / rw.n, y = rw.row(it - k1 * rw.n);
+        int k1;
+        const int y = rw.row(rw.split(it, k1));
         const C<T> *row = P + y * pitch + k1 * N2;
 #pragma unroll
         for (int j2 = 0; j2 < N2; ++j2) v[j2] = row[j2];
@@ -848,11 +869,12 @@ __device__ __forceinline__ void yz_i2(const C<T> *P, C<T> *Q, int pitch, int lgM
 // I3 writes row slot p2 + N2 k1 (not k1 + N1 p2) so that I4's threads, which
 // run over p2 with k1 fixed per load, read consecutive slots: both passes hit
 // distinct shared-memory banks.
-template <typename T, int N1, int N2>   // I3: z inverse pass A, Q rows -> P row slots
-__device__ __forceinline__ void yz_i3(const C<T> *Q, C<T> *P, int pitch, const Rows rw, const C<T> *tiz) {
+template <typename T, int N1, int N2, RowsKind K>   // I3: z inverse pass A, Q rows -> P row slots
+__device__ __forceinline__ void yz_i3(const C<T> *Q, C<T> *P, int pitch, const Rows<K> rw, const C<T> *tiz) {
     C<T> v[FFT_NMAX];
     for (int it = threadIdx.x; it < rw.n * N1; it += blockDim.x) {
-        const int k1 = it / rw.n, y = rw.row(it - k1 * rw.n);
+        int k1;
+        const int y = rw.row(rw.split(it, k1));
         const C<T> *src = Q + y * pitch + k1;
 #pragma unroll
         for (int k2 = 0; k2 < N2; ++k2) v[k2] = src[N1 * k2];
@@ -862,8 +884,8 @@ __device__ __forceinline__ void yz_i3(const C<T> *Q, C<T> *P, int pitch, const R
         for (int p2 = 0; p2 < N2; ++p2) o[p2] = v[p2];
     }
 }
-template <typename T, int N1, int N2>   // I4: z inverse pass B, P row slots -> global, z < Nz
-__device__ __forceinline__ void yz_i4(const C<T> *P, C<T> *out, int pitch, const Rows rw, const C<T> *tiz) {
+template <typename T, int N1, int N2, RowsKind K>   // I4: z inverse pass B, P row slots -> global, z < Nz
+__device__ __forceinline__ void yz_i4(const C<T> *P, C<T> *out, int pitch, const Rows<K> rw, const C<T> *tiz) {
     constexpr int Mz = N1 * N2, Nz = Mz / 2, H1 = N1 / 2;
     constexpr int LG2 = N2 == 2 ? 1 : N2 == 4 ? 2 : N2 == 8 ? 3 : 4;
     C<T> v[FFT_NMAX];
@@ -936,24 +958,34 @@ __device__ __forceinline__ void yz_mid(C<T> *P, int pitch, int lgMz, const HT *_
 // Hp: kernel spectrum [fold(kx)][fold(ky)][fold(kz)], scaled by 1/(Mx My Mz):
 // real (HT = T, the static kernel) or complex (HT = C<T>, the lossy kernel).
 // Htab / gslot: as in k_fft_zconv (grid g = blockIdx.x / Mx uses Htab[gslot[g]]).
-// rows: bit mask of the rows y < Ny that hold data and are wanted (the others are
-// not written).
-template <typename T, int NT, typename HT>
+// SP: only the rows y < Ny of the bit mask rows hold data and are wanted (see Rows;
+// listed, the others are not written).
+template <typename T, int NT, typename HT, bool SP>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_fft_yzc(C<T> *__restrict__ buf, int lgMx, int My, int Mz,
                                                  const HT *__restrict__ Hp, const C<T> *__restrict__ tfy,
                                                  const C<T> *__restrict__ tiy, const C<T> *__restrict__ tfz,
                                                  const C<T> *__restrict__ tiz, const HT *const *__restrict__ Htab,
                                                  const int32_t *__restrict__ gslot, ulonglong2 rows) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint8_t s_rows[128];
+    __shared__ uint8_t s_rows[SP && sizeof(T) != 4 ? 128 : 1];
     const int pitch = Mz + 1, Ny = My / 2, Nz = Mz / 2;
     const int lgMz = ilog2(Mz);
-    const Rows rw{s_rows, __popcll(rows.x) + __popcll(rows.y)};
-    for (int y = threadIdx.x; y < Ny; y += NT) {
-        const uint64_t below = y < 64 ? rows.x : rows.y, bit = 1ull << (y & 63);
-        if (below & bit) s_rows[(y < 64 ? 0 : __popcll(rows.x)) + __popcll(below & (bit - 1))] = uint8_t(y);
+    constexpr RowsKind K = !SP ? kAllRows : sizeof(T) == 4 ? kMasked : kListed;
+    Rows<K> rw;
+    rw.mask = rows;
+    rw.list = s_rows;
+    if constexpr (K == kListed) {
+        rw.n = __popcll(rows.x) + __popcll(rows.y);
+        rw.inv = ((1u << 20) + rw.n - 1) / rw.n;
+        for (int y = threadIdx.x; y < Ny; y += NT) {
+            const uint64_t below = y < 64 ? rows.x : rows.y, bit = 1ull << (y & 63);
+            if (below & bit) s_rows[(y < 64 ? 0 : __popcll(rows.x)) + __popcll(below & (bit - 1))] = uint8_t(y);
+        }
+        __syncthreads();
+    } else {
+        rw.n = Ny;
+        rw.inv = ilog2(Ny);
     }
-    __syncthreads();
     const int Mx = 1 << lgMx;
     const int kx = blockIdx.x & (Mx - 1);
     C<T> *P = reinterpret_cast<C<T> *>(smem_raw);
@@ -961,23 +993,23 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_fft_yzc(C<T> *__
     C<T> *plane = buf + int64_t(blockIdx.x) * Ny * Nz;
     const HT *Hg = Htab ? Htab[gslot[blockIdx.x >> lgMx]] : Hp;
     const HT *Hk = Hg + int64_t(fold_index(kx, Mx)) * (My / 2 + 1) * (Mz / 2 + 1);
-    SIE_SPLIT_DISPATCH(Mz, (yz_f1<T, N1, N2>(plane, P, pitch, rw, tfz)));
-    if (rw.n < Ny)
+    SIE_SPLIT_DISPATCH(Mz, (yz_f1<T, N1, N2, K>(plane, P, pitch, rw, tfz)));
+    if constexpr (K == kListed)
         for (int i = threadIdx.x; i < Ny * Mz; i += NT) {
             const int y = i >> lgMz;
             if (!(((y < 64 ? rows.x : rows.y) >> (y & 63)) & 1)) Qb[y * pitch + (i & (Mz - 1))] = mk<T>(T(0.0), T(0.0));
         }
     __syncthreads();
-    SIE_SPLIT_DISPATCH(Mz, (yz_f2<T, N1, N2>(P, Qb, pitch, rw, tfz)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_f2<T, N1, N2, K>(P, Qb, pitch, rw, tfz)));
     __syncthreads();
     SIE_SPLIT_DISPATCH(My, (yz_f3<T, N1, N2>(Qb, P, pitch, lgMz, tfy)));
     __syncthreads();
     SIE_SPLIT_DISPATCH(My, (yz_mid<T, N1, N2, HT>(P, pitch, lgMz, Hk, tfy, tiy)));
     SIE_SPLIT_DISPATCH(My, (yz_i2<T, N1, N2>(P, Qb, pitch, lgMz, tiy)));
     __syncthreads();
-    SIE_SPLIT_DISPATCH(Mz, (yz_i3<T, N1, N2>(Qb, P, pitch, rw, tiz)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_i3<T, N1, N2, K>(Qb, P, pitch, rw, tiz)));
     __syncthreads();
-    SIE_SPLIT_DISPATCH(Mz, (yz_i4<T, N1, N2>(P, plane, pitch, rw, tiz)));
+    SIE_SPLIT_DISPATCH(Mz, (yz_i4<T, N1, N2, K>(P, plane, pitch, rw, tiz)));
 }
 
 }  // namespace sie

@@ -588,15 +588,15 @@ int launch_yzc(pfft_plan *p, C<T> *spec, int32_t ngrids, const HT *Hp, bool acti
     while ((1 << lgMx) < p->Mx) ++lgMx;
     split4(p->My, n1y, n2y);
     split4(p->Mz, n1z, n2z);
-    ulonglong2 rows = make_ulonglong2(~0ull, ~0ull);   // every row of N_y <= 128
-    if (p->Ny < 64) rows.x = (1ull << p->Ny) - 1;
-    if (p->Ny < 128) rows.y = p->Ny > 64 ? (1ull << (p->Ny - 64)) - 1 : 0;
-    if (active) rows = make_ulonglong2(p->act_rows[0], p->act_rows[1]);
     auto launch = [&](auto nt) -> int {
         constexpr int NT = decltype(nt)::value;
-        if (int rc = set_smem((const void *)k_fft_yzc<T, NT, HT>, plane_bytes)) return rc;
-        k_fft_yzc<T, NT, HT><<<unsigned(ngrids * p->Mx), NT, plane_bytes, s>>>(
-            spec, lgMx, p->My, p->Mz, Hp, Tb::tf(p, 1), Tb::ti(p, 1), Tb::tf(p, 2), Tb::ti(p, 2), Htab, gslot, rows);
+        auto kern = k_fft_yzc<T, NT, HT, false>;
+        if constexpr (NT > 64)   // rows are left out of planes of 32 rows and more only
+            if (active) kern = k_fft_yzc<T, NT, HT, true>;
+        if (int rc = set_smem((const void *)kern, plane_bytes)) return rc;
+        kern<<<unsigned(ngrids * p->Mx), NT, plane_bytes, s>>>(spec, lgMx, p->My, p->Mz, Hp, Tb::tf(p, 1), Tb::ti(p, 1),
+                                                               Tb::tf(p, 2), Tb::ti(p, 2), Htab, gslot,
+                                                               make_ulonglong2(p->act_rows[0], p->act_rows[1]));
         SIE_LAUNCH_CHECK(p);
         return SIE_OK;
     };

@@ -182,3 +182,17 @@ def test_batch_rejects_lossy_plans(wires):
     m, O, S, P = wires
     with pytest.raises(N.SieError):
         api.Batch([P])
+
+
+@pytest.mark.parametrize("prec,tol", [(PREC_FP64, 1e-10), (PREC_MIXED, 1e-5)])
+def test_lossy_product_on_a_grid_with_empty_rows(prec, tol):
+    """Wires far apart: most y rows of the grid have no stencil node and take no part in
+    the product, whatever another product, here of NaN currents, left in the buffers."""
+    m = synth.wire_array_mesh(2, 10e-6, 60e-6, 900e-6, n_sides=6, n_seg=4, jitter=0.1, seed=9)
+    O, S, P = build(m, dict(PARAMS, grid=(8, 64, 4), order=2, near_factor=1.0, n_touch=8))
+    x = synth.complex_gaussian(O.nl, len(OMEGAS), seed=24)
+    ref = np.stack([S.matvec(x[r], OMEGAS[r]) for r in range(len(OMEGAS))])
+    xt = torch.from_numpy(x).cuda()
+    api.pfft_matvec(P, torch.full_like(xt, float("nan")), OMEGAS, SPACE_LOOP, prec)
+    got = api.pfft_matvec(P, xt, OMEGAS, SPACE_LOOP, prec).cpu().numpy()
+    assert rel(got, ref).max() < tol
